@@ -87,6 +87,10 @@ struct alm_handle {
     bool fused_dual = false;
     int sms = 0;
     double *up_sel_a = nullptr, *d_sel_a = nullptr, *gd_a = nullptr, *gu_a = nullptr, *g_a = nullptr;
+    int n_gchunk = 0;
+    int *gc_con = nullptr, *g_cptr = nullptr;
+    double *g_part = nullptr;
+    unsigned int *g_cnt = nullptr;
     double *g_a1 = nullptr, *g_a2 = nullptr, *lr_u = nullptr, *lr_s = nullptr, *b = nullptr;
     // state and work
     DevState *st = nullptr;
@@ -280,6 +284,11 @@ static SparseView<T> view(const alm_handle *h) {
     v.g_a = h->g_a;
     v.g_a1 = h->g_a1;
     v.g_a2 = h->g_a2;
+    v.n_gchunk = h->n_gchunk;
+    v.gc_con = h->gc_con;
+    v.g_cptr = h->g_cptr;
+    v.g_part = h->g_part;
+    v.g_cnt = h->g_cnt;
     v.lr_k = h->lr_k;
     v.lr_u = h->lr_u;
     v.lr_s = h->lr_s;
@@ -529,6 +538,19 @@ static alm_status create_impl(alm_handle *h, const alm_problem *p, const alm_opt
     if (hp.m_gen > 0) {
         TRY(dalloc(h, reinterpret_cast<void **>(&h->g_a1), sizeof(double) * size_t(hp.m_gen)));
         TRY(dalloc(h, reinterpret_cast<void **>(&h->g_a2), sizeof(double) * size_t(hp.m_gen)));
+        std::vector<int32_t> con, cptr(1, 0);
+        for (int64_t g = 0; g < hp.m_gen; ++g) {
+            const int32_t cnt = hp.g_ptr[size_t(g) + 1] - hp.g_ptr[size_t(g)];
+            con.insert(con.end(), size_t(std::max(1, (cnt + kGenChunk - 1) / kGenChunk)), int32_t(g));
+            cptr.push_back(int32_t(con.size()));
+        }
+        h->n_gchunk = int(con.size());
+        TRY(upload(h, &h->gc_con, con));
+        TRY(upload(h, &h->g_cptr, cptr));
+        CK(cudaStreamSynchronize(h->stream));  // con and cptr end here
+        TRY(dalloc(h, reinterpret_cast<void **>(&h->g_part), sizeof(double) * 2 * con.size()));
+        TRY(dalloc(h, reinterpret_cast<void **>(&h->g_cnt), sizeof(unsigned int) * size_t(hp.m_gen)));
+        CK(cudaMemsetAsync(h->g_cnt, 0, sizeof(unsigned int) * size_t(hp.m_gen), h->stream));
     }
     TRY(upload(h, &h->lr_u, hp.lr_u));
     TRY(upload(h, &h->lr_s, hp.lr_s));

@@ -16,6 +16,7 @@ constexpr int kMaxRank = 32;     // rank cap (r_max)
 constexpr int kLzMax = 64;       // Lanczos basis length per cycle
 constexpr int kBlock = 256;      // threads per block of the row kernels
 constexpr int kNumSMs = 152;     // GB300
+constexpr int kGenChunk = 256;   // entries of a general constraint per CTA
 constexpr int kPartStride = 160; // doubles of partial sums per block (>= kLzMax + 4, >= 1 + kMaxLR*kMaxRank)
 
 // ------------------------------------------------------------------------------------
@@ -159,6 +160,10 @@ struct SparseView {
     const int *g_con, *g_ptr, *g_i, *g_j;
     const double *g_a;
     double *g_a1, *g_a2;             // per general constraint: A1, A2 of the line search
+    int n_gchunk;                    // chunks of at most kGenChunk entries of the general constraints:
+    const int *gc_con, *g_cptr;      // each chunk's constraint, each constraint's first chunk
+    double *g_part;                  // two partial sums per chunk
+    unsigned int *g_cnt;             // chunks of each constraint that have finished (0 between launches)
     int lr_k;
     const double *lr_u, *lr_s;
     const double *b;

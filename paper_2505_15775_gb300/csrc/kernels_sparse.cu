@@ -5,7 +5,7 @@
 //                for problems whose constraints are all diagonal selectors (MaxCut)
 //                also the dual update w = y - sigma(A(X) - b), diag(S) and the L / KKT
 //                reductions                                            [hot path (a)]
-//   k_gen_eval   A(RR^T)_k of the general (multi-entry) constraints
+//   k_gen        A(RR^T)_k of the general (multi-entry) constraints, or their a1, a2
 //   k_dual_slack w, the L / KKT reductions and S = C - A^*(w) (general problems)
 //   k_spmm       G = 2 S R (+ the low-rank part of C), ||G||^2 and the CG inner
 //                products                                              [hot path (b)]
@@ -13,7 +13,6 @@
 //   k_ls         the quartic phi(alpha) = L(R + alpha D): a1 = A(RD^T + DR^T),
 //                a2 = A(DD^T), <S, RD^T + DR^T>, <S, DD^T> in one pass over R and D,
 //                FP64 coefficients and the exact minimiser            [hot path (c)]
-//   k_gen_ls     a1, a2 of the general constraints
 //   k_axpy       R += alpha D
 //
 // Work decomposition.  A group of LANES lanes owns one row of R (lane l holds the
@@ -29,6 +28,7 @@
 // per thread, summed per block in FP64 and over blocks in FP64 by the last block to
 // finish (a fixed order: results are deterministic).  The dual w and the constraint
 // residuals are FP64 throughout.
+#include <algorithm>
 #include <cfloat>
 #include <cmath>
 #include <mutex>
@@ -291,23 +291,76 @@ __global__ void __launch_bounds__(kBlock) k_eval(SparseView<T> v, const T *__res
     }
 }
 
-// general constraints: A(X)_k = sum over its entries of kappa a (r_i . r_j); one block each
-template <typename T>
-__global__ void __launch_bounds__(kBlock) k_gen_eval(SparseView<T> v, const T *__restrict__ R, int r, int ldr,
-                                                     double *__restrict__ AX, const int *done) {
+// ---------------------------------------------------------------------------------------
+// General (multi-entry) constraints: A(X)_k = sum over its entries of kappa a (r_i . r_j)
+// (LS: a1_k = A(RD^T + DR^T)_k and a2_k = A(DD^T)_k into g_a1, g_a2).  The entries are cut
+// into chunks of kGenChunk, one CTA each, so that a constraint on every row (the trace of a
+// theta SDP) fills the chip instead of one CTA; a row group of LANES lanes reads each row as
+// one coalesced vector per lane and keeps its columns' share of the sum in FP64 (no reduction
+// per entry).  The last chunk of a constraint to finish adds up the chunks in order.
+// With one CTA per constraint and a thread per entry walking its columns the trace over 20,000
+// rows at r = 29 took 575 us, its line-search form 1189 us; alm_linesearch on that theta SDP
+// went from 2.03 to 0.30 ms with the chunks.
+// ---------------------------------------------------------------------------------------
+template <typename T, int LANES, bool LS>
+__global__ void __launch_bounds__(kBlock) k_gen(SparseView<T> v, const T *__restrict__ R, const T *__restrict__ D,
+                                                int r, int ldr, double *__restrict__ AX, const int *done) {
     if (*done) return;
+    using V = typename VecT<T>::type;
+    constexpr int W = VecT<T>::W;
     __shared__ double shm[32];
-    for (int g = blockIdx.x; g < v.m_gen; g += gridDim.x) {
-        double acc = 0.0;
-        for (int t = v.g_ptr[g] + threadIdx.x; t < v.g_ptr[g + 1]; t += blockDim.x) {
+    __shared__ bool last;
+    const int gl = threadIdx.x & (LANES - 1);
+    const bool active = gl * W < r;
+    for (int c = blockIdx.x; c < v.n_gchunk; c += gridDim.x) {
+        const int g = v.gc_con[c], c0 = v.g_cptr[g], nc = v.g_cptr[g + 1] - c0;
+        const int e0 = v.g_ptr[g] + (c - c0) * kGenChunk;
+        const int e1 = min(e0 + kGenChunk, v.g_ptr[g + 1]);
+        double a1 = 0.0, a2 = 0.0;
+        for (int t = e0 + threadIdx.x / LANES; t < e1; t += kBlock / LANES) {
             const int i = v.g_i[t], j = v.g_j[t];
-            T x = T(0);
-            for (int c = 0; c < r; ++c) x += R[int64_t(i) * ldr + c] * R[int64_t(j) * ldr + c];
-            acc += (i == j ? 1.0 : 2.0) * v.g_a[t] * double(x);
+            const double ka = (i == j ? 1.0 : 2.0) * v.g_a[t];
+            const V ri = mask_tail(load_row(R, i, ldr, gl, active), gl * W, r);
+            const V rj = load_row(R, j, ldr, gl, active);
+            if (LS) {
+                const V di = mask_tail(load_row(D, i, ldr, gl, active), gl * W, r);
+                const V dj = load_row(D, j, ldr, gl, active);
+                a1 = fma(ka, double(dot(ri, dj) + dot(di, rj)), a1);
+                a2 = fma(ka, double(dot(di, dj)), a2);
+            } else {
+                a1 = fma(ka, double(dot(ri, rj)), a1);
+            }
         }
-        const double s = block_sum(acc, shm);
-        if (threadIdx.x == 0) AX[v.g_con[g]] = s;
-        __syncthreads();
+        a1 = block_sum(a1, shm);
+        if (LS) a2 = block_sum(a2, shm);
+        if (nc > 1) {
+            if (threadIdx.x == 0) {
+                v.g_part[2 * c] = a1;
+                v.g_part[2 * c + 1] = a2;
+                __threadfence();
+                last = atomicAdd(v.g_cnt + g, 1u) == unsigned(nc - 1);
+                if (last) v.g_cnt[g] = 0u;
+            }
+            __syncthreads();
+            if (!last) continue;  // block-uniform
+            __threadfence();
+            double s1 = 0.0, s2 = 0.0;
+            for (int q = threadIdx.x; q < nc; q += kBlock) {
+                s1 += __ldcg(v.g_part + 2 * (c0 + q));
+                if (LS) s2 += __ldcg(v.g_part + 2 * (c0 + q) + 1);
+            }
+            a1 = block_sum(s1, shm);
+            if (LS) a2 = block_sum(s2, shm);
+        }
+        if (threadIdx.x == 0) {
+            if (LS) {
+                v.g_a1[g] = a1;
+                v.g_a2[g] = a2;
+            } else {
+                AX[v.g_con[g]] = a1;
+            }
+        }
+        __syncthreads();  // `last` is reused
     }
 }
 
@@ -786,6 +839,18 @@ __global__ void __launch_bounds__(kBlock, 3) k_ls(SparseView<T> v, const T *__re
                 const double t = sum_partials(partials, 8 + l * kMaxRank + col, shm);
                 if (threadIdx.x == 0) st->zd[l][col] = t;
             }
+    if (v.m_gen > 0) {
+        double g11 = 0.0, g12 = 0.0, g22 = 0.0;
+        for (int g = threadIdx.x; g < v.m_gen; g += blockDim.x) {
+            const double A1 = v.g_a1[g], A2 = v.g_a2[g];
+            g11 += A1 * A1;
+            g12 += A1 * A2;
+            g22 += A2 * A2;
+        }
+        tot[2] += block_sum(g11, shm);
+        tot[3] += block_sum(g12, shm);
+        tot[4] += block_sum(g22, shm);
+    }
     if (threadIdx.x == 0) ls_finish<T, MODE, LR>(v, st, r, tot);
 }
 
@@ -865,37 +930,6 @@ __global__ void __launch_bounds__(kBlock, 4) k_ls_ell(SparseView<T> v, const T *
 }
 
 
-// general constraints of the line search: A1_g, A2_g; one block each
-template <typename T>
-__global__ void __launch_bounds__(kBlock) k_gen_ls(SparseView<T> v, const T *__restrict__ R,
-                                                   const T *__restrict__ D, int r, int ldr, const int *done) {
-    if (*done) return;
-    __shared__ double shm[32];
-    for (int g = blockIdx.x; g < v.m_gen; g += gridDim.x) {
-        double a1 = 0.0, a2 = 0.0;
-        for (int t = v.g_ptr[g] + threadIdx.x; t < v.g_ptr[g + 1]; t += blockDim.x) {
-            const int i = v.g_i[t], j = v.g_j[t];
-            T x1 = T(0), x2 = T(0);
-            for (int c = 0; c < r; ++c) {
-                const T ric = R[int64_t(i) * ldr + c], rjc = R[int64_t(j) * ldr + c];
-                const T dic = D[int64_t(i) * ldr + c], djc = D[int64_t(j) * ldr + c];
-                x1 += ric * djc + dic * rjc;
-                x2 += dic * djc;
-            }
-            const double ka = (i == j ? 1.0 : 2.0) * v.g_a[t];
-            a1 += ka * double(x1);
-            a2 += ka * double(x2);
-        }
-        const double s1 = block_sum(a1, shm);
-        const double s2 = block_sum(a2, shm);
-        if (threadIdx.x == 0) {
-            v.g_a1[g] = s1;
-            v.g_a2[g] = s2;
-        }
-        __syncthreads();
-    }
-}
-
 // R += alpha D  (skipped when done == 1; done == 2, the step that reached the iteration cap,
 // still takes this update and then becomes done == 1, so that the remaining launches of the
 // chunk apply nothing)
@@ -962,7 +996,9 @@ void launch_eval(const LaunchCtx &c, const SparseView<T> &v, const T *R, int r, 
     constexpr int W = VecT<T>::W;
     const int L = lanes_for(r, W);
     if (v.m_gen > 0) {
-        k_gen_eval<T><<<v.m_gen < c.grid ? v.m_gen : c.grid, kBlock, 0, c.stream>>>(v, R, r, ldr, AX, done);
+        ALM_DISPATCH_LANES(L, {
+            k_gen<T, LN, false><<<std::min(v.n_gchunk, c.grid), kBlock, 0, c.stream>>>(v, R, R, r, ldr, AX, done);
+        });
         ++*c.launches;
     }
     const bool fused = v.fused_dual && y && w;
@@ -1111,7 +1147,9 @@ void launch_ls(const LaunchCtx &c, const SparseView<T> &v, const T *R, const T *
         return;
     }
     if (v.m_gen > 0) {
-        k_gen_ls<T><<<v.m_gen < c.grid ? v.m_gen : c.grid, kBlock, 0, c.stream>>>(v, R, D, r, ldr, done);
+        ALM_DISPATCH_LANES(L, {
+            k_gen<T, LN, true><<<std::min(v.n_gchunk, c.grid), kBlock, 0, c.stream>>>(v, R, D, r, ldr, nullptr, done);
+        });
         ++*c.launches;
     }
     const bool off = v.has_off_sel, lr = v.lr_k > 0;

@@ -141,7 +141,8 @@ __device__ __forceinline__ void spmm_finish(DevState *st, double gg, double go, 
 // exact step and (MODE 1) the inner-loop bookkeeping
 template <typename T, int MODE, bool LR>
 __device__ __forceinline__ void ls_finish(const SparseView<T> &v, DevState *st, int r, const double (&tot)[5]) {
-        double s1 = tot[0], s2 = tot[1], a11 = tot[2], a12 = tot[3], a22 = tot[4];
+        double s1 = tot[0], s2 = tot[1];
+        const double a11 = tot[2], a12 = tot[3], a22 = tot[4];
         if (LR)  // <s u u^T, RD^T + DR^T> = 2 s (R^T u).(D^T u),  <s u u^T, DD^T> = s |D^T u|^2
             for (int l = 0; l < v.lr_k; ++l) {
                 double zr = 0.0, dd = 0.0;
@@ -152,12 +153,6 @@ __device__ __forceinline__ void ls_finish(const SparseView<T> &v, DevState *st, 
                 s1 += v.lr_s[l] * 2.0 * zr;
                 s2 += v.lr_s[l] * dd;
             }
-        for (int g = 0; g < v.m_gen; ++g) {
-            const double A1 = v.g_a1[g], A2 = v.g_a2[g];
-            a11 += A1 * A1;
-            a12 += A1 * A2;
-            a22 += A2 * A2;
-        }
         const double sigma = st->sigma;
         double q[5];
         q[0] = st->L;
