@@ -87,6 +87,10 @@ struct alm_handle {
     bool fused_dual = false;
     int sms = 0;
     double *up_sel_a = nullptr, *d_sel_a = nullptr, *gd_a = nullptr, *gu_a = nullptr, *g_a = nullptr;
+    int n_heavy = 0;             // rows above kHeavyRow entries, and segments of long upper rows
+    int64_t n_useg = 0;
+    int *hv_row = nullptr, *us_row = nullptr, *us_e0 = nullptr;
+    void *hv_sum = nullptr;
     int n_gchunk = 0;
     int *gc_con = nullptr, *g_cptr = nullptr;
     double *g_part = nullptr;
@@ -284,6 +288,12 @@ static SparseView<T> view(const alm_handle *h) {
     v.g_a = h->g_a;
     v.g_a1 = h->g_a1;
     v.g_a2 = h->g_a2;
+    v.n_heavy = h->n_heavy;
+    v.hv_row = h->hv_row;
+    v.hv_sum = static_cast<T *>(h->hv_sum);
+    v.n_useg = h->n_useg;
+    v.us_row = h->us_row;
+    v.us_e0 = h->us_e0;
     v.n_gchunk = h->n_gchunk;
     v.gc_con = h->gc_con;
     v.g_cptr = h->g_cptr;
@@ -522,6 +532,27 @@ static alm_status create_impl(alm_handle *h, const alm_problem *p, const alm_opt
         int32_t *slot = nullptr;
         TRY(upload(h, &slot, hp.up_slot));
         h->up_slot = reinterpret_cast<int2 *>(slot);
+    }
+    if (hp.ell_kf == 0) {  // the CSR kernels' long rows
+        std::vector<int32_t> hv;
+        for (int64_t i = 0; i < h->n; ++i)
+            if (hp.f_ptr[size_t(i) + 1] - hp.f_ptr[size_t(i)] > kHeavyRow) hv.push_back(int32_t(i));
+        h->n_heavy = int(hv.size());
+        TRY(upload(h, &h->hv_row, hv));
+        TRY(dalloc(h, &h->hv_sum, sizeof(double) * 2 * kMaxRank * hv.size()));
+        CK(cudaStreamSynchronize(h->stream));
+    }
+    {
+        std::vector<int32_t> row, e0;
+        for (int64_t i = 0; i < h->n; ++i)
+            for (int64_t e = int64_t(hp.up_ptr[size_t(i)]) + kUpSeg; e < hp.up_ptr[size_t(i) + 1]; e += kUpSeg) {
+                row.push_back(int32_t(i));
+                e0.push_back(int32_t(e));
+            }
+        h->n_useg = int64_t(row.size());
+        TRY(upload(h, &h->us_row, row));
+        TRY(upload(h, &h->us_e0, e0));
+        CK(cudaStreamSynchronize(h->stream));
     }
     TRY(dalloc(h, &h->d_s, h->esz * size_t(h->n)));
     TRY(upload(h, &h->gd_ptr, hp.gd_ptr));

@@ -17,6 +17,8 @@ constexpr int kLzMax = 64;       // Lanczos basis length per cycle
 constexpr int kBlock = 256;      // threads per block of the row kernels
 constexpr int kNumSMs = 152;     // GB300
 constexpr int kGenChunk = 256;   // entries of a general constraint per CTA
+constexpr int kHeavyRow = 256;   // longer rows of the full pattern are summed by a CTA each
+constexpr int kUpSeg = 128;      // longer rows of the strict upper pattern are cut into segments
 constexpr int kPartStride = 160; // doubles of partial sums per block (>= kLzMax + 4, >= 1 + kMaxLR*kMaxRank)
 
 // ------------------------------------------------------------------------------------
@@ -147,6 +149,11 @@ struct SparseView {
     const double *d_sel_a;
     const int *f_ptr, *f_col;
     T *f_val;                        // S_ij on the full pattern
+    int n_heavy;                     // rows of more than kHeavyRow entries in the full pattern:
+    const int *hv_row;               // ascending
+    T *hv_sum;                       // their off-diagonal sums (k_spmm_heavy)
+    int64_t n_useg;                  // segments of kUpSeg entries of the strict upper rows beyond
+    const int *us_row, *us_e0;       // their first kUpSeg: row and first entry
     T *d_s;                          // S_ii (FP32 form: the leading float of a float pair)
     T *d_s_lo;                       // FP32 form: S_ii - d_s as a float (null in the FP64 form)
     const T *base_hi, *base_lo;      // C_ii - a_i y_k(i) for diagonal selectors, per outer iteration

@@ -25,6 +25,18 @@ struct AccD {
     __device__ __forceinline__ void add(double s, double2 x) { v = fma4(s, x, v); }
     __device__ __forceinline__ void add_lo(double s, double2 x) { v = fma4(s, x, v); }
     __device__ __forceinline__ double2 value() const { return v; }
+    // add up the accumulators of lanes FROM, 2 FROM, .. < TO apart
+    template <int FROM, int TO>
+    __device__ __forceinline__ void merge(unsigned mask) {
+#pragma unroll
+        for (int o = FROM; o < TO; o <<= 1) {
+            v.x += __shfl_xor_sync(mask, v.x, o);
+            v.y += __shfl_xor_sync(mask, v.y, o);
+        }
+    }
+    static constexpr int kWords = 1;  // W-vectors of its state
+    __device__ __forceinline__ void store(double *p) const { stv(p, v); }
+    __device__ __forceinline__ void add_stored(const double *p) { v = fma4(1.0, ld(p), v); }
 };
 struct AccF {
     float hi[4], lo[4];
@@ -47,6 +59,33 @@ struct AccF {
         lo[2] = fmaf(s, x.z, lo[2]);
         lo[3] = fmaf(s, x.w, lo[3]);
     }
+    template <int FROM, int TO>
+    __device__ __forceinline__ void merge(unsigned mask) {
+#pragma unroll
+        for (int o = FROM; o < TO; o <<= 1)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float h2 = __shfl_xor_sync(mask, hi[k], o), l2 = __shfl_xor_sync(mask, lo[k], o);
+                two_sum_acc(hi[k], lo[k], h2);
+                lo[k] += l2;
+            }
+    }
+    static constexpr int kWords = 2;
+    __device__ __forceinline__ void store(float *p) const {
+        stv(p, make_float4(hi[0], hi[1], hi[2], hi[3]));
+        stv(p + 4, make_float4(lo[0], lo[1], lo[2], lo[3]));
+    }
+    __device__ __forceinline__ void add_stored(const float *p) {
+        const float4 h = ld(p), l = ld(p + 4);
+        two_sum_acc(hi[0], lo[0], h.x);
+        two_sum_acc(hi[1], lo[1], h.y);
+        two_sum_acc(hi[2], lo[2], h.z);
+        two_sum_acc(hi[3], lo[3], h.w);
+        lo[0] += l.x;
+        lo[1] += l.y;
+        lo[2] += l.z;
+        lo[3] += l.w;
+    }
     __device__ __forceinline__ float4 value() const {
         return make_float4(hi[0] + lo[0], hi[1] + lo[1], hi[2] + lo[2], hi[3] + lo[3]);
     }
@@ -61,6 +100,39 @@ template <>
 struct AccOf<double> {
     using type = AccD;
 };
+
+// The lane's a . b as a float pair (products split exactly, sums with two-sum): the constraint
+// values, whose residual is far smaller than they are and is multiplied by sigma.  The FP64
+// form returns its plain sum in hi.
+__device__ __forceinline__ void dot_pair(float4 a, float4 b, float &hi, float &lo) {
+    const float x[4] = {a.x, a.y, a.z, a.w}, y[4] = {b.x, b.y, b.z, b.w};
+    hi = x[0] * y[0];
+    lo = fmaf(x[0], y[0], -hi);
+#pragma unroll
+    for (int k = 1; k < 4; ++k) {
+        const float p = x[k] * y[k];
+        lo += fmaf(x[k], y[k], -p);
+        two_sum_acc(hi, lo, p);
+    }
+}
+__device__ __forceinline__ void dot_pair(double2 a, double2 b, double &hi, double &lo) {
+    hi = dot(a, b);
+    lo = 0.0;
+}
+// sum of the pairs over the LANES lanes of a row
+template <int LANES>
+__device__ __forceinline__ void pair_group_sum(float &hi, float &lo, unsigned mask) {
+#pragma unroll
+    for (int o = LANES / 2; o > 0; o >>= 1) {
+        const float h2 = __shfl_xor_sync(mask, hi, o), l2 = __shfl_xor_sync(mask, lo, o);
+        two_sum_acc(hi, lo, h2);
+        lo += l2;
+    }
+}
+template <int LANES>
+__device__ __forceinline__ void pair_group_sum(double &hi, double &, unsigned mask) {
+    hi = group_sum<LANES>(hi, mask);
+}
 
 // float-pair sum of squares of a lane's vector over the row group (FP32 form); the
 // FP64 form returns its plain sum in hi

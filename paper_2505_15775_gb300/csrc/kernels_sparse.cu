@@ -15,13 +15,19 @@
 //                FP64 coefficients and the exact minimiser            [hot path (c)]
 //   k_axpy       R += alpha D
 //
-// Work decomposition.  A group of LANES lanes owns one row of R (lane l holds the
-// 16-byte vector of columns [l W, l W + W), W = 4 floats or 2 doubles), so a gathered
-// row is one coalesced 16*LANES-byte read and a dot product is a shuffle reduction
-// inside the group.  The SDDMMs run a streaming pass over the diagonal (rows) and an
-// entry-parallel pass over the strict upper pattern (COO), two entries per group and
-// iteration, so that every lane keeps four independent row gathers in flight.  The
-// SpMM walks two rows per group and iteration with predicated, independent gathers.
+// Work decomposition.  LANES lanes hold one row of R (lane l the 16-byte vector of columns
+// [l W, l W + W), W = 4 floats or 2 doubles), so a gathered row is one coalesced
+// 16*LANES-byte read.  SP such subgroups share a row of the pattern (k_eval, k_spmm, k_ls):
+// subgroup s takes its entries s, s + SP, .., and a row group is LANES x SP lanes.  SP is
+// a whole warp's worth when the rows are long enough to give each subgroup two entries, else
+// one (wide_rows): with one subgroup a row of 80 entries is a serial walk and 10,000 rows at
+// rank 3 fill 40 of 152 multiprocessors.  Rows above kHeavyRow entries
+// (heavy-tailed graphs) would still be one warp's serial walk: the SpMM's are summed
+// beforehand by a CTA each (k_spmm_heavy); the SDDMMs' sums are scalars, so their rows are
+// cut into segments of kUpSeg entries that any row group takes.
+// In FP32, against one subgroup a row and two rows a group: alm_grad on a Kronecker graph of
+// 2^16 rows at r = 32 1.62 -> 0.36 ms; 32 inner steps of matrix completion (n = 1e4, 829,000
+// entries, rank 3) 10.4 -> 4.5 ms.
 //
 // Precision.  FP64 arithmetic is scarce on GB300, so in the FP32 form every per-entry
 // product and every per-thread partial sum is FP32; partials are promoted to FP64 once
@@ -42,33 +48,61 @@ namespace alm {
 // helpers
 // ---------------------------------------------------------------------------------------
 
-// Block-reduce the per-lane column vectors acc[l][k] (column gl*W + k of term l) over the
-// row groups of the block into part[l*kMaxRank + col] (columns no lane covers are 0).
+// The block's share of X^T u_l of the low-rank terms (u_l in FP64) into part[l*kMaxRank + col],
+// from a pass of its own over the rows with LANES lanes a row: FP64 instructions cost the same
+// for one active lane as for 32, so the split row groups of the kernels would pay SP times.
 template <typename T, int LANES>
-__device__ __forceinline__ void block_reduce_cols(double (*acc)[VecT<T>::W], int nl, double *part, double *shm) {
+__device__ __forceinline__ void block_lr_cols(const SparseView<T> &v, const T *__restrict__ X, int r, int ldr,
+                                              double *part, double *shm) {
+    using V = typename VecT<T>::type;
     constexpr int W = VecT<T>::W;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int t = threadIdx.x; t < nl * kMaxRank; t += blockDim.x) part[t] = 0.0;
-    for (int l = 0; l < nl; ++l) {
-        for (int k = 0; k < W; ++k) {
-            double x = acc[l][k];
+    const int gl = lane & (LANES - 1);
+    const bool active = gl * W < r;
+    for (int l = 0; l < v.lr_k; ++l) {
+        double acc[W];
 #pragma unroll
-            for (int o = 16; o >= LANES; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-            __syncthreads();
-            if (lane < LANES) shm[warp * 32 + lane] = x;
-            __syncthreads();
-            if (threadIdx.x < LANES) {
-                double t = 0.0;
-                for (int w = 0; w < nw; ++w) t += shm[w * 32 + threadIdx.x];
-                const int col = threadIdx.x * W + k;
-                if (col < kMaxRank) part[l * kMaxRank + col] = t;
-            }
+        for (int k = 0; k < W; ++k) acc[k] = 0.0;
+        for (int64_t i = int64_t(blockIdx.x) * (kBlock / LANES) + threadIdx.x / LANES; i < v.n;
+             i += int64_t(gridDim.x) * (kBlock / LANES)) {
+            const V x = mask_tail(load_row(X, i, ldr, gl, active), gl * W, r);
+            const double u = v.lr_u[int64_t(l) * v.n + i];
+#pragma unroll
+            for (int k = 0; k < W; ++k) acc[k] = fma(u, double(comp(x, k)), acc[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < W; ++k)
+#pragma unroll
+            for (int o = 16; o >= LANES; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+        __syncthreads();
+        if (lane < LANES)
+#pragma unroll
+            for (int k = 0; k < W; ++k)
+                if (lane * W + k < kMaxRank) shm[warp * 32 + lane * W + k] = acc[k];
+        __syncthreads();
+        if (threadIdx.x < kMaxRank) {
+            double t = 0.0;
+            if (threadIdx.x < LANES * W)
+                for (int q = 0; q < nw; ++q) t += shm[q * 32 + threadIdx.x];
+            part[l * kMaxRank + threadIdx.x] = t;
         }
     }
 }
 
-
-
+// In the last block: z[l][col] = sum over the blocks of part (one warp per column, lanes over
+// the blocks in a fixed order), zero from column r on; visible to the block on return
+__device__ __forceinline__ void sum_lr_cols(const double *part, int nl, int r, double (*z)[kMaxRank]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int t = warp; t < nl * kMaxRank; t += nw) {
+        const int col = t % kMaxRank;
+        double a = 0.0;
+        if (col < r)
+            for (int b = lane; b < int(gridDim.x); b += 32) a += __ldcg(part + size_t(b) * kPartStride + t);
+        a = warp_sum(a);
+        if (lane == 0) z[t / kMaxRank][col] = a;
+    }
+    __syncthreads();
+}
 
 template <typename T, int LANES>
 __device__ __forceinline__ void slack_row(const SparseView<T> &v, int64_t i, T xh, T xl, T sigma) {
@@ -166,7 +200,7 @@ __global__ void __launch_bounds__(kBlock) k_prep_base(SparseView<T> v, const dou
 // ---------------------------------------------------------------------------------------
 // (a) constraint map + <C, RR^T> (+ fused dual update for diagonal-selector problems)
 // ---------------------------------------------------------------------------------------
-template <typename T, int LANES, bool OFFSEL, bool LR, bool FUSED>
+template <typename T, int LANES, int SP, bool OFFSEL, bool LR, bool FUSED>
 __global__ void __launch_bounds__(kBlock) k_eval(SparseView<T> v, const T *__restrict__ R, int r, int ldr,
                                                  double *__restrict__ AX, const double *__restrict__ y,
                                                  double *__restrict__ w, DevState *st, double *partials,
@@ -174,28 +208,58 @@ __global__ void __launch_bounds__(kBlock) k_eval(SparseView<T> v, const T *__res
     if (*done) return;
     using V = typename VecT<T>::type;
     constexpr int W = VecT<T>::W;
+    constexpr int GW = LANES * SP;
+    constexpr int U = 2;  // entries per subgroup and round
     __shared__ double shm[32 * 32];
     const int lane = threadIdx.x & 31;
-    const int gl = lane & (LANES - 1);
-    const unsigned gmask = group_mask<LANES>(lane);
-    const int gpb = kBlock / LANES;
-    const int64_t g0 = int64_t(blockIdx.x) * gpb + threadIdx.x / LANES;
-    const int64_t ng = int64_t(gridDim.x) * gpb;
+    const int gl = lane & (LANES - 1), sub = (lane & (GW - 1)) / LANES;
+    const unsigned gmask = group_mask<GW>(lane);
+    const int64_t g0 = int64_t(blockIdx.x) * (kBlock / GW) + threadIdx.x / GW;
+    const int64_t ng = int64_t(gridDim.x) * (kBlock / GW);
     const bool active = gl * W < r;
     const double sigma = FUSED ? st->sigma : 0.0;
     T pc = T(0);
     double pyres = 0.0, pres2 = 0.0, pbw = 0.0;
-    double lacc[LR ? kMaxLR : 1][W];
-    if (LR)
-        for (int l = 0; l < kMaxLR; ++l)
-            for (int k = 0; k < W; ++k) lacc[l][k] = 0.0;
 
-    // diagonal entries: one streaming pass over the rows of R
+    // strict upper entries e0 .. e1-1 of a row (ri its masked vector)
+    auto upper = [&](V ri, int64_t i, int e0, int e1) {
+        T acc = T(0);
+        for (int e = e0 + sub; e < e1 + sub; e += U * SP) {  // group-uniform trip count
+            int j[U];
+            T c[U];
+            V x[U];
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+                const bool in = e + k * SP < e1;
+                j[k] = in ? v.up_col[e + k * SP] : int(i);
+                c[k] = in ? v.up_c[e + k * SP] : T(0);
+            }
+#pragma unroll
+            for (int k = 0; k < U; ++k) x[k] = load_row(R, j[k], ldr, gl, active);
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+                if (OFFSEL) {
+                    T hi, lo;
+                    dot_pair(ri, x[k], hi, lo);
+                    acc += c[k] * hi;
+                    pair_group_sum<LANES>(hi, lo, gmask);
+                    if (gl == 0 && e + k * SP < e1) {
+                        const int q = v.up_sel_k[e + k * SP];
+                        if (q >= 0) AX[q] = 2.0 * v.up_sel_a[e + k * SP] * (double(hi) + double(lo));
+                    }
+                } else {
+                    acc += c[k] * dot(ri, x[k]);
+                }
+            }
+        }
+        pc += T(2) * acc;
+    };
     for (int64_t i = g0; i < v.n; i += ng) {
         const V ri = mask_tail(load_row(R, i, ldr, gl, active), gl * W, r);
+        const int e0 = v.up_ptr[i], e1 = min(v.up_ptr[i + 1], e0 + kUpSeg);
         const double viid = ff_norm2<LANES>(ri, gmask);  // compensated in FP32
-        const T vii = T(viid);
-        if (gl == 0) {
+        if (gl == 0 && sub == 0) {
+            const T vii = T(viid);
             const T cii = v.d_c[i];
             pc += cii * vii;
             const int k = v.d_sel_k[i];
@@ -216,36 +280,11 @@ __global__ void __launch_bounds__(kBlock) k_eval(SparseView<T> v, const T *__res
                 store_slack_diag(v, i, double(cii));
             }
         }
-        if (LR)
-            for (int l = 0; l < v.lr_k; ++l) {
-                const double u = v.lr_u[int64_t(l) * v.n + i];
-                for (int k = 0; k < W; ++k) lacc[l][k] += u * double(comp(ri, k));
-            }
+        upper(ri, i, e0, e1);
     }
-    // strict upper entries: two per group and iteration
-    for (int64_t e = g0; e < v.nnz_u; e += 2 * ng) {
-        const int64_t e2 = e + ng;
-        const bool has2 = e2 < v.nnz_u;
-        const int i0 = v.up_row[e], j0 = v.up_col[e];
-        const int i1 = has2 ? v.up_row[e2] : i0, j1 = has2 ? v.up_col[e2] : j0;
-        const V a0 = load_row(R, i0, ldr, gl, active);
-        const V b0 = load_row(R, j0, ldr, gl, active);
-        const V a1 = load_row(R, i1, ldr, gl, active);
-        const V b1 = load_row(R, j1, ldr, gl, active);
-        const T x0 = group_sum<LANES>(dot(mask_tail(a0, gl * W, r), b0), gmask);
-        const T x1 = group_sum<LANES>(dot(mask_tail(a1, gl * W, r), b1), gmask);
-        if (gl == 0) {
-            pc += T(2) * v.up_c[e] * x0;
-            if (has2) pc += T(2) * v.up_c[e2] * x1;
-            if (OFFSEL) {
-                const int k0 = v.up_sel_k[e];
-                if (k0 >= 0) AX[k0] = 2.0 * v.up_sel_a[e] * double(x0);
-                if (has2) {
-                    const int k1 = v.up_sel_k[e2];
-                    if (k1 >= 0) AX[k1] = 2.0 * v.up_sel_a[e2] * double(x1);
-                }
-            }
-        }
+    for (int64_t q = g0; q < v.n_useg; q += ng) {  // the rest of the long rows
+        const int i = v.us_row[q], e0 = v.us_e0[q], e1 = min(v.up_ptr[i + 1], e0 + kUpSeg);
+        upper(mask_tail(load_row(R, i, ldr, gl, active), gl * W, r), i, e0, e1);
     }
     double *part = partials + size_t(blockIdx.x) * kPartStride;
     if (FUSED) {
@@ -255,23 +294,19 @@ __global__ void __launch_bounds__(kBlock) k_eval(SparseView<T> v, const T *__res
         const double vals[1] = {double(pc)};
         block_partials<1>(vals, part, shm);
     }
-    if (LR) block_reduce_cols<T, LANES>(lacc, v.lr_k, part + 4, shm);
+    if (LR) block_lr_cols<T, LANES>(v, R, r, ldr, part + 4, shm);
     if (!last_block(&st->counter[CNT_EVAL])) return;
-    const double c0 = sum_partials(partials, 0, shm);
-    double yres = 0.0, res2 = 0.0, bw = 0.0;
+    double tot[4] = {0.0, 0.0, 0.0, 0.0};
     if (FUSED) {
-        yres = sum_partials(partials, 1, shm);
-        res2 = sum_partials(partials, 2, shm);
-        bw = sum_partials(partials, 3, shm);
+        sum_partials_n<4>(partials, tot, shm);
+    } else {
+        double t1[1];
+        sum_partials_n<1>(partials, t1, shm);
+        tot[0] = t1[0];
     }
-    if (LR)
-        for (int l = 0; l < v.lr_k; ++l)
-            for (int col = 0; col < kMaxRank; ++col) {
-                const double t = sum_partials(partials, 4 + l * kMaxRank + col, shm);
-                if (threadIdx.x == 0) st->z[l][col] = t;
-            }
+    if (LR) sum_lr_cols(partials + 4, v.lr_k, r, st->z);
     if (threadIdx.x == 0) {
-        double c = c0;
+        double c = tot[0];
         for (int l = 0; LR && l < v.lr_k; ++l) {
             double zz = 0.0;
             for (int col = 0; col < r; ++col) zz += st->z[l][col] * st->z[l][col];
@@ -279,10 +314,10 @@ __global__ void __launch_bounds__(kBlock) k_eval(SparseView<T> v, const T *__res
         }
         st->c0 = c;
         if (FUSED) {
-            st->yres = yres;
-            st->res2 = res2;
-            st->bw = bw;
-            st->L = c - yres + 0.5 * sigma * res2;
+            st->yres = tot[1];
+            st->res2 = tot[2];
+            st->bw = tot[3];
+            st->L = c - tot[1] + 0.5 * sigma * tot[2];
             if (!isfinite(st->L)) {
                 st->status = ALM_ERR_NUMERIC;
                 st->done = 1;
@@ -328,7 +363,10 @@ __global__ void __launch_bounds__(kBlock) k_gen(SparseView<T> v, const T *__rest
                 a1 = fma(ka, double(dot(ri, dj) + dot(di, rj)), a1);
                 a2 = fma(ka, double(dot(di, dj)), a2);
             } else {
-                a1 = fma(ka, double(dot(ri, rj)), a1);
+                T hi, lo;
+                dot_pair(ri, rj, hi, lo);
+                a1 = fma(ka, double(hi), a1);
+                if (sizeof(T) == 4) a1 = fma(ka, double(lo), a1);
             }
         }
         a1 = block_sum(a1, shm);
@@ -437,22 +475,71 @@ __global__ void __launch_bounds__(kBlock) k_dual_slack(SparseView<T> v, const do
 //   MODE 1: inner CG step: also <G, G_old> (G is updated in place) and <G, D_old>, the
 //           stop test ||G|| <= tau and the Polak-Ribiere+ coefficient
 // ---------------------------------------------------------------------------------------
-template <typename T, int LANES, bool LR, int MODE>
-__global__ void __launch_bounds__(kBlock, 3) k_spmm(SparseView<T> v, const T *__restrict__ R, int r, int ldr,
-                                                 T *G, const T *D, DevState *st, double *partials,
-                                                 const int *done) {
+// Off-diagonal sums of the rows above kHeavyRow entries, one CTA each, into hv_sum (the
+// accumulator's state per column vector; k_spmm adds it to the row's diagonal part).
+template <typename T, int LANES>
+__global__ void __launch_bounds__(kBlock) k_spmm_heavy(SparseView<T> v, const T *__restrict__ R, int r, int ldr,
+                                                       const int *done) {
     if (*done) return;
     using V = typename VecT<T>::type;
+    using Acc = typename AccOf<T>::type;
     constexpr int W = VecT<T>::W;
-    constexpr int U = 4;  // neighbours per row and round
+    constexpr int U = 4;
+    constexpr int NSUB = kBlock / LANES;
+    __shared__ __align__(16) T sh[kBlock / 32][LANES][Acc::kWords * W];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int gl = lane & (LANES - 1);
+    const bool active = gl * W < r;
+    for (int q = blockIdx.x; q < v.n_heavy; q += gridDim.x) {
+        const int i = v.hv_row[q];
+        const int e1 = v.f_ptr[i + 1];
+        Acc acc;
+        acc.init();
+        for (int e = v.f_ptr[i] + threadIdx.x / LANES; e < e1; e += U * NSUB) {
+            int j[U];
+            T c[U];
+            V x[U];
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+                const bool in = e + k * NSUB < e1;
+                j[k] = in ? v.f_col[e + k * NSUB] : i;
+                c[k] = in ? v.f_val[e + k * NSUB] : T(0);
+            }
+#pragma unroll
+            for (int k = 0; k < U; ++k) x[k] = load_row(R, j[k], ldr, gl, active);
+#pragma unroll
+            for (int k = 0; k < U; ++k) acc.add(c[k], x[k]);
+        }
+        __syncwarp();
+        acc.template merge<LANES, 32>(0xffffffffu);
+        if (lane < LANES) acc.store(sh[warp][lane]);
+        __syncthreads();
+        if (threadIdx.x < LANES) {
+            for (int ww = 1; ww < kBlock / 32; ++ww) acc.add_stored(sh[ww][lane]);
+            acc.store(v.hv_sum + (int64_t(q) * LANES + lane) * (Acc::kWords * W));
+        }
+        __syncthreads();
+    }
+}
+
+template <typename T, int LANES, int SP, bool LR, int MODE>
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 3 : 4) k_spmm(SparseView<T> v, const T *__restrict__ R,
+                                                                      int r, int ldr, T *G, const T *D, DevState *st,
+                                                                      double *partials, const int *done) {
+    if (*done) return;
+    using V = typename VecT<T>::type;
+    using Acc = typename AccOf<T>::type;
+    constexpr int W = VecT<T>::W;
+    constexpr int GW = LANES * SP;
+    constexpr int U = 4;  // entries per subgroup and round
     __shared__ double shm[32];
     const int lane = threadIdx.x & 31;
-    const int gl = lane & (LANES - 1);
-    const int gpb = kBlock / LANES;
-    const int64_t g0 = int64_t(blockIdx.x) * gpb + threadIdx.x / LANES;
-    const int64_t ng = int64_t(gridDim.x) * gpb;
+    const int gl = lane & (LANES - 1), sub = (lane & (GW - 1)) / LANES;
+    const unsigned gmask = group_mask<GW>(lane);
+    const int64_t g0 = int64_t(blockIdx.x) * (kBlock / GW) + threadIdx.x / GW;
+    const int64_t ng = int64_t(gridDim.x) * (kBlock / GW);
     const bool active = gl * W < r;
-    const bool writer = gl * W < ldr;
+    const bool writer = sub == 0 && gl * W < ldr;
     V zl[LR ? kMaxLR : 1];
     if (LR)
         for (int l = 0; l < v.lr_k; ++l) {
@@ -465,146 +552,89 @@ __global__ void __launch_bounds__(kBlock, 3) k_spmm(SparseView<T> v, const T *__
             else zl[l] = make_double2(zz[0], zz[1]);
         }
     T pgg = T(0), pgo = T(0), pgd = T(0), pzg = T(0);
-    const unsigned gmask = group_mask<LANES>(lane);
     const bool pc = MODE == 1 && st->precond;
     const T sig = T(st->sigma);
     const T pc_floor = T(st->pc_floor);
-    for (int64_t i = g0; i < v.n; i += 2 * ng) {
-        const int64_t i2 = i + ng;
-        const bool has2 = i2 < v.n;
-        const int64_t ib = has2 ? i2 : i;  // a valid row for predicated accesses
+    for (int64_t i = g0; i < v.n; i += ng) {
         const V ri = mask_tail(load_row(R, i, ldr, gl, active), gl * W, r);
-        const V rb = mask_tail(load_row(R, ib, ldr, gl, active), gl * W, r);
-        using Acc = typename AccOf<T>::type;
-        Acc acc, acb;
+        const int e0 = v.f_ptr[i], e1 = v.f_ptr[i + 1];
+        const T ds = v.d_s[i], dlo = v.d_s_lo ? v.d_s_lo[i] : T(0);
+        V gold = vzero(T()), dold = vzero(T());
+        if (MODE == 1 && active && sub == 0) {
+            gold = ld(G + i * ldr + gl * W);
+            dold = ld(D + i * ldr + gl * W);
+        }
+        Acc acc;
         acc.init();
-        acb.init();
-        acc.add(v.d_s[i], ri);
-        acb.add(has2 ? v.d_s[ib] : T(0), rb);
-        if (v.d_s_lo) {
-            acc.add_lo(v.d_s_lo[i], ri);
-            acb.add_lo(has2 ? v.d_s_lo[ib] : T(0), rb);
+        if (sub == 0) {
+            acc.add(ds, ri);
+            acc.add_lo(dlo, ri);
+            if (LR)
+                for (int l = 0; l < v.lr_k; ++l) acc.add(T(v.lr_u[int64_t(l) * v.n + i]), zl[l]);
         }
-        int e = v.f_ptr[i];
-        const int e1 = v.f_ptr[i + 1];
-        int f = has2 ? v.f_ptr[ib] : 0;
-        const int f1 = has2 ? v.f_ptr[ib + 1] : 0;
-        while (e < e1 || f < f1) {
-            int ja[U], jb[U];
-            T sa[U], sb[U];
-#pragma unroll
-            for (int k = 0; k < U; ++k) {
-                const bool oa = e + k < e1, ob = f + k < f1;
-                ja[k] = oa ? v.f_col[e + k] : int(i);
-                sa[k] = oa ? v.f_val[e + k] : T(0);
-                jb[k] = ob ? v.f_col[f + k] : int(ib);
-                sb[k] = ob ? v.f_val[f + k] : T(0);
+        if (v.n_heavy > 0 && e1 - e0 > kHeavyRow) {  // its entries are summed already
+            int a = 0, b = v.n_heavy - 1;
+            while (a < b) {
+                const int mid = (a + b) / 2;
+                if (v.hv_row[mid] < int(i)) a = mid + 1;
+                else b = mid;
             }
-            V ga[U], gb[U];
+            if (sub == 0) acc.add_stored(v.hv_sum + (int64_t(a) * LANES + gl) * (Acc::kWords * W));
+        } else {
+            for (int e = e0 + sub; e < e1; e += U * SP) {
+                int j[U];
+                T c[U];
+                V x[U];
 #pragma unroll
-            for (int k = 0; k < U; ++k) {
-                ga[k] = load_row(R, ja[k], ldr, gl, active);
-                gb[k] = load_row(R, jb[k], ldr, gl, active);
-            }
+                for (int k = 0; k < U; ++k) {
+                    const bool in = e + k * SP < e1;
+                    j[k] = in ? v.f_col[e + k * SP] : int(i);
+                    c[k] = in ? v.f_val[e + k * SP] : T(0);
+                }
 #pragma unroll
-            for (int k = 0; k < U; ++k) {
-                acc.add(sa[k], ga[k]);
-                acb.add(sb[k], gb[k]);
+                for (int k = 0; k < U; ++k) x[k] = load_row(R, j[k], ldr, gl, active);
+#pragma unroll
+                for (int k = 0; k < U; ++k) acc.add(c[k], x[k]);
             }
-            e += U;
-            f += U;
+            __syncwarp(gmask);
+            acc.template merge<LANES, GW>(gmask);
         }
-        if (LR)
-            for (int l = 0; l < v.lr_k; ++l) {
-                acc.add(T(v.lr_u[int64_t(l) * v.n + i]), zl[l]);
-                acb.add(T(v.lr_u[int64_t(l) * v.n + ib]), zl[l]);
-            }
-        const V ga = mask_tail(scale4(T(2), acc.value()), gl * W, r);
-        const V gb = mask_tail(scale4(T(2), acb.value()), gl * W, r);
-        pgg += dot(ga, ga);
-        if (has2) pgg += dot(gb, gb);
+        const V g = mask_tail(scale4(T(2), acc.value()), gl * W, r);
+        if (sub == 0) pgg += dot(g, g);
         if (MODE == 1) {
             // Row-block Jacobi preconditioner Z = P^{-1} G with P_i = 2 s_i I + 4 sigma a_i^2 r_i r_i^T
             // (the block of the Hessian of L in row i: the S_ii part and the penalty of the
             // diagonal selector a_i e_i e_i^T), inverted by Sherman-Morrison; s_i = S_ii floored.
-            V za = ga, zb = gb;
+            V z = g;
             if (pc) {
-                const T rga = group_sum<LANES>(dot(ri, ga), gmask), rra = group_sum<LANES>(dot(ri, ri), gmask);
-                const T rgb = group_sum<LANES>(dot(rb, gb), gmask), rrb = group_sum<LANES>(dot(rb, rb), gmask);
-                auto precond_row = [&](int64_t row, T rg, T rr, V g, V rv) -> V {
-                    T sdi = v.d_s[row] + (v.d_s_lo ? v.d_s_lo[row] : T(0));
-                    sdi = sdi > pc_floor ? sdi : pc_floor;
-                    const int k = v.d_sel_k[row];
-                    const T a = k >= 0 ? T(v.d_sel_a[row]) : T(0);
-                    const T ka = T(4) * sig * a * a;
-                    const T coef = ka * rg / (T(2) * sdi + ka * rr);
-                    const T inv = T(1) / (T(2) * sdi);
-                    V z = fma4(-coef, rv, g);
-                    return scale4(inv, z);
-                };
-                za = precond_row(i, rga, rra, ga, ri);
-                zb = precond_row(ib, rgb, rrb, gb, rb);
+                const T rg = group_sum<LANES>(dot(ri, g), gmask), rr = group_sum<LANES>(dot(ri, ri), gmask);
+                T sdi = ds + dlo;
+                sdi = sdi > pc_floor ? sdi : pc_floor;
+                const int k = v.d_sel_k[i];
+                const T a = k >= 0 ? T(v.d_sel_a[i]) : T(0);
+                const T ka = T(4) * sig * a * a;
+                const T coef = ka * rg / (T(2) * sdi + ka * rr);
+                z = scale4(T(1) / (T(2) * sdi), fma4(-coef, ri, g));
             }
-            if (active) {
-                pzg += dot(za, ga);
-                pgo += dot(ga, ld(G + i * ldr + gl * W));
-                pgd += dot(ga, ld(D + i * ldr + gl * W));
-                if (has2) {
-                    pzg += dot(zb, gb);
-                    pgo += dot(gb, ld(G + ib * ldr + gl * W));
-                    pgd += dot(gb, ld(D + ib * ldr + gl * W));
-                }
+            if (sub == 0) {
+                pzg += dot(z, g);
+                pgo += dot(g, gold);
+                pgd += dot(g, dold);
             }
-            if (writer) {
-                stv(G + i * ldr + gl * W, za);
-                if (has2) stv(G + ib * ldr + gl * W, zb);
-            }
+            if (writer) stv(G + i * ldr + gl * W, z);
         } else if (writer) {
-            stv(G + i * ldr + gl * W, ga);
-            if (has2) stv(G + ib * ldr + gl * W, gb);
+            stv(G + i * ldr + gl * W, g);
         }
     }
     double *part = partials + size_t(blockIdx.x) * kPartStride;
-    if (MODE == 1) {
-        const double vals[4] = {double(pgg), double(pgo), double(pgd), double(pzg)};
-        block_partials<4>(vals, part, shm);
-    } else {
-        const double vals[1] = {double(pgg)};
-        block_partials<1>(vals, part, shm);
-    }
+    const double vals[4] = {double(pgg), double(pgo), double(pgd), double(pzg)};
+    block_partials<4>(vals, part, shm);
     if (!last_block(&st->counter[CNT_SPMM])) return;
-    const double gg = sum_partials(partials, 0, shm);
-    double go = 0.0, gd = 0.0, zg = 0.0;
-    if (MODE == 1) {
-        go = sum_partials(partials, 1, shm);
-        gd = sum_partials(partials, 2, shm);
-        zg = sum_partials(partials, 3, shm);
-    }
+    double tot[4];
+    sum_partials_n<4>(partials, tot, shm);
     if (threadIdx.x == 0) {
-        st->gg = gg;
-        if (MODE == 1) {
-            if (!isfinite(gg)) {
-                st->status = ALM_ERR_NUMERIC;
-                st->done = 1;
-            } else if (sqrt(gg) <= st->tau_abs) {
-                st->done = 1;
-            }
-            // Polak-Ribiere+ on the preconditioned gradient Z (Z = G without preconditioning):
-            // beta = max(0, <Z, G - G_old> / <Z_old, G_old>), with <Z, G_old> taken as
-            // <G, Z_old> (P symmetric and slowly varying), so that only Z is stored
-            double beta = 0.0;
-            if (!st->restart && st->method == ALM_INNER_CG && st->zg_prev > 0.0) {
-                beta = fmax(0.0, (zg - go) / st->zg_prev);
-                if (-zg + beta * gd >= 0.0) beta = 0.0;  // not a descent direction: restart
-            }
-            st->beta = beta;
-            st->g_gprev = go;
-            st->g_dprev = gd;
-            st->gg_prev = gg;
-            st->zg = zg;
-            st->zg_prev = zg;
-            st->restart = 0;
-        }
+        if (MODE == 1) spmm_finish(st, tot[0], tot[1], tot[2], tot[3]);
+        else st->gg = tot[0];
     }
 }
 
@@ -722,29 +752,22 @@ __global__ void __launch_bounds__(kBlock) k_dir(const T *__restrict__ G, T *__re
 //   MODE 1: inner loop: q1 from the SpMM's inner products (<G, D> = -|G|^2 + beta <G, D_old>,
 //           free of cancellation), plus the done / iteration bookkeeping.
 // ---------------------------------------------------------------------------------------
-template <typename T, int LANES, bool OFFSEL, bool LR, int MODE>
+template <typename T, int LANES, int SP, bool OFFSEL, bool LR, int MODE>
 __global__ void __launch_bounds__(kBlock, 3) k_ls(SparseView<T> v, const T *__restrict__ R, const T *__restrict__ D,
                                                int r, int ldr, DevState *st, double *partials, const int *done) {
     if (*done) return;
     using V = typename VecT<T>::type;
     constexpr int W = VecT<T>::W;
+    constexpr int GW = LANES * SP;
+    constexpr int U = 2;  // entries per subgroup and round (each gathers a row of R and one of D)
     __shared__ double shm[32 * 32];
     const int lane = threadIdx.x & 31;
-    const int gl = lane & (LANES - 1);
-    const unsigned gmask = group_mask<LANES>(lane);
-    const int gpb = kBlock / LANES;
-    const int64_t g0 = int64_t(blockIdx.x) * gpb + threadIdx.x / LANES;
-    const int64_t ng = int64_t(gridDim.x) * gpb;
+    const int gl = lane & (LANES - 1), sub = (lane & (GW - 1)) / LANES;
+    const unsigned gmask = group_mask<GW>(lane);
+    const int64_t g0 = int64_t(blockIdx.x) * (kBlock / GW) + threadIdx.x / GW;
+    const int64_t ng = int64_t(gridDim.x) * (kBlock / GW);
     const bool active = gl * W < r;
     T p1 = T(0), p2 = T(0), p11 = T(0), p12 = T(0), p22 = T(0);
-    double lacc[LR ? kMaxLR : 1][W];
-    if (LR)
-        for (int l = 0; l < kMaxLR; ++l)
-            for (int k = 0; k < W; ++k) lacc[l][k] = 0.0;
-
-    // one row-based pass: rows i and i + ng per group and iteration, each with its strict
-    // upper neighbours (two per round, predicated), so that R and D stream from HBM once
-    constexpr int U = 2;
     auto sel_terms = [&](int k, double a_k, T x1, T x2) {
         if (k >= 0) {
             const T a = T(a_k);
@@ -754,91 +777,69 @@ __global__ void __launch_bounds__(kBlock, 3) k_ls(SparseView<T> v, const T *__re
             p22 += A2 * A2;
         }
     };
-    for (int64_t i = g0; i < v.n; i += 2 * ng) {
-        const int64_t i2 = i + ng;
-        const bool has2 = i2 < v.n;
-        const int64_t ib = has2 ? i2 : i;
-        const V ri = mask_tail(load_row(R, i, ldr, gl, active), gl * W, r);
-        const V di = mask_tail(load_row(D, i, ldr, gl, active), gl * W, r);
-        const V rb = mask_tail(load_row(R, ib, ldr, gl, active), gl * W, r);
-        const V db = mask_tail(load_row(D, ib, ldr, gl, active), gl * W, r);
-        const T a1i = T(2) * group_sum<LANES>(dot(ri, di), gmask);
-        const T a2i = group_sum<LANES>(dot(di, di), gmask);
-        const T a1b = T(2) * group_sum<LANES>(dot(rb, db), gmask);
-        const T a2b = group_sum<LANES>(dot(db, db), gmask);
-        if (gl == 0) {
-            const T si = v.d_s[i];
-            p1 += si * a1i;
-            p2 += si * a2i;
-            sel_terms(v.d_sel_k[i], v.d_sel_a[i], a1i, a2i);
-            if (has2) {
-                const T sb = v.d_s[ib];
-                p1 += sb * a1b;
-                p2 += sb * a2b;
-                sel_terms(v.d_sel_k[ib], v.d_sel_a[ib], a1b, a2b);
-            }
-        }
-        if (LR)
-            for (int l = 0; l < v.lr_k; ++l) {
-                const double u = v.lr_u[int64_t(l) * v.n + i];
-                const double ub = has2 ? v.lr_u[int64_t(l) * v.n + ib] : 0.0;
-                for (int k = 0; k < W; ++k) lacc[l][k] += u * double(comp(di, k)) + ub * double(comp(db, k));
-            }
-        int e = v.up_ptr[i];
-        const int e1 = v.up_ptr[i + 1];
-        int f = has2 ? v.up_ptr[ib] : 0;
-        const int f1 = has2 ? v.up_ptr[ib + 1] : 0;
-        while (e < e1 || f < f1) {
-            int ja[U], jb[U];
-            T sa[U], sbv[U];
+    // strict upper entries e0 .. e1-1 of a row: <S, RD^T + DR^T> and <S, DD^T> are lane-local
+    // sums over the lane's columns; only an entry's selector needs its whole dot products
+    auto upper = [&](V ri, V di, int64_t i, int e0, int e1) {
+        for (int e = e0 + sub; e < e1 + sub; e += U * SP) {  // group-uniform trip count
+            int j[U];
+            T s2[U];
+            V rj[U], dj[U];
 #pragma unroll
             for (int k = 0; k < U; ++k) {
-                const bool oa = e + k < e1, ob = f + k < f1;
-                ja[k] = oa ? v.up_col[e + k] : int(i);
-                sa[k] = oa ? T(2) * v.up_s[e + k] : T(0);
-                jb[k] = ob ? v.up_col[f + k] : int(ib);
-                sbv[k] = ob ? T(2) * v.up_s[f + k] : T(0);
-            }
-            V rja[U], dja[U], rjb[U], djb[U];
-#pragma unroll
-            for (int k = 0; k < U; ++k) {
-                rja[k] = load_row(R, ja[k], ldr, gl, active);
-                dja[k] = load_row(D, ja[k], ldr, gl, active);
-                rjb[k] = load_row(R, jb[k], ldr, gl, active);
-                djb[k] = load_row(D, jb[k], ldr, gl, active);
+                const bool in = e + k * SP < e1;
+                j[k] = in ? v.up_col[e + k * SP] : int(i);
+                s2[k] = in ? T(2) * v.up_s[e + k * SP] : T(0);
             }
 #pragma unroll
             for (int k = 0; k < U; ++k) {
-                const T x1a = group_sum<LANES>(dot(ri, dja[k]) + dot(di, rja[k]), gmask);
-                const T x2a = group_sum<LANES>(dot(di, dja[k]), gmask);
-                const T x1b = group_sum<LANES>(dot(rb, djb[k]) + dot(db, rjb[k]), gmask);
-                const T x2b = group_sum<LANES>(dot(db, djb[k]), gmask);
-                if (gl == 0) {
-                    p1 += sa[k] * x1a + sbv[k] * x1b;
-                    p2 += sa[k] * x2a + sbv[k] * x2b;
-                    if (OFFSEL) {
-                        if (e + k < e1) sel_terms(v.up_sel_k[e + k], 2.0 * v.up_sel_a[e + k], x1a, x2a);
-                        if (f + k < f1) sel_terms(v.up_sel_k[f + k], 2.0 * v.up_sel_a[f + k], x1b, x2b);
-                    }
+                rj[k] = load_row(R, j[k], ldr, gl, active);
+                dj[k] = load_row(D, j[k], ldr, gl, active);
+            }
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+                T x1 = dot(ri, dj[k]) + dot(di, rj[k]);
+                T x2 = dot(di, dj[k]);
+                p1 += s2[k] * x1;
+                p2 += s2[k] * x2;
+                if (OFFSEL) {
+                    x1 = group_sum<LANES>(x1, gmask);
+                    x2 = group_sum<LANES>(x2, gmask);
+                    if (gl == 0 && e + k * SP < e1) sel_terms(v.up_sel_k[e + k * SP], 2.0 * v.up_sel_a[e + k * SP], x1, x2);
                 }
             }
-            e += U;
-            f += U;
         }
+    };
+    for (int64_t i = g0; i < v.n; i += ng) {
+        const V ri = mask_tail(load_row(R, i, ldr, gl, active), gl * W, r);
+        const V di = mask_tail(load_row(D, i, ldr, gl, active), gl * W, r);
+        const int e0 = v.up_ptr[i], e1 = min(v.up_ptr[i + 1], e0 + kUpSeg);
+        const T rdi = T(2) * dot(ri, di), ddi = dot(di, di);
+        if (sub == 0) {
+            const T si = v.d_s[i];
+            p1 += si * rdi;
+            p2 += si * ddi;
+        }
+        const int ksel = v.d_sel_k[i];
+        if (ksel >= 0) {  // group-uniform
+            const T a1 = group_sum<LANES>(rdi, gmask);
+            const T a2 = group_sum<LANES>(ddi, gmask);
+            if (gl == 0 && sub == 0) sel_terms(ksel, v.d_sel_a[i], a1, a2);
+        }
+        upper(ri, di, i, e0, e1);
+    }
+    for (int64_t q = g0; q < v.n_useg; q += ng) {  // the rest of the long rows
+        const int i = v.us_row[q], e0 = v.us_e0[q], e1 = min(v.up_ptr[i + 1], e0 + kUpSeg);
+        upper(mask_tail(load_row(R, i, ldr, gl, active), gl * W, r),
+              mask_tail(load_row(D, i, ldr, gl, active), gl * W, r), i, e0, e1);
     }
     double *part = partials + size_t(blockIdx.x) * kPartStride;
     const double vals[5] = {double(p1), double(p2), double(p11), double(p12), double(p22)};
     block_partials<5>(vals, part, shm);
-    if (LR) block_reduce_cols<T, LANES>(lacc, v.lr_k, part + 8, shm);
+    if (LR) block_lr_cols<T, LANES>(v, D, r, ldr, part + 8, shm);
     if (!last_block(&st->counter[CNT_LS])) return;
     double tot[5];
-    for (int k = 0; k < 5; ++k) tot[k] = sum_partials(partials, k, shm);
-    if (LR)
-        for (int l = 0; l < v.lr_k; ++l)
-            for (int col = 0; col < kMaxRank; ++col) {
-                const double t = sum_partials(partials, 8 + l * kMaxRank + col, shm);
-                if (threadIdx.x == 0) st->zd[l][col] = t;
-            }
+    sum_partials_n<5>(partials, tot, shm);
+    if (LR) sum_lr_cols(partials + 8, v.lr_k, r, st->zd);
     if (v.m_gen > 0) {
         double g11 = 0.0, g12 = 0.0, g22 = 0.0;
         for (int g = threadIdx.x; g < v.m_gen; g += blockDim.x) {
@@ -982,12 +983,22 @@ static __global__ void __launch_bounds__(kBlock) k_sumsq(const double *__restric
 // host launchers
 // ---------------------------------------------------------------------------------------
 
+// Subgroups per row: a warp's worth when the pattern's rows give each of them two entries on
+// average, else one: with fewer, the split's reductions and idle lanes cost more than the
+// shorter walk saves.
+static inline bool wide_rows(int64_t entries, int64_t n, int LN) { return entries >= 2 * (32 / LN) * n; }
+#define ALM_ROW_SPLIT(wide, LN, ...)                                             \
+    if (wide) { constexpr int SPW = 32 / LN; __VA_ARGS__; }                      \
+    else { constexpr int SPW = 1; __VA_ARGS__; }
+
 template <typename T, int LN, bool OFF, bool LRB, bool FUS>
 static void eval_one(const LaunchCtx &c, const SparseView<T> &v, const T *R, int r, int ldr, double *AX,
                      const double *y, double *w, const int *done) {
-    auto *fn = k_eval<T, LN, OFF, LRB, FUS>;
-    const int grid = grid_for(c, fn, v.n + v.nnz_u, kBlock / LN);
-    fn<<<grid, kBlock, 0, c.stream>>>(v, R, r, ldr, AX, y, w, c.st, c.partials, done);
+    ALM_ROW_SPLIT(wide_rows(v.nnz_u, v.n, LN), LN, {
+        auto *fn = k_eval<T, LN, SPW, OFF, LRB, FUS>;
+        const int grid = grid_for(c, fn, v.n + v.n_useg, kBlock / (LN * SPW));
+        fn<<<grid, kBlock, 0, c.stream>>>(v, R, r, ldr, AX, y, w, c.st, c.partials, done);
+    });
 }
 
 template <typename T>
@@ -1056,9 +1067,15 @@ void launch_dual_slack(const LaunchCtx &c, const SparseView<T> &v, const double 
 template <typename T, int LN, bool LRB, int MODE>
 static void spmm_one(const LaunchCtx &c, const SparseView<T> &v, const T *R, int r, int ldr, T *G, const T *D,
                      const int *done) {
-    auto *fn = k_spmm<T, LN, LRB, MODE>;
-    const int grid = grid_for(c, fn, v.n, 2 * (kBlock / LN));
-    fn<<<grid, kBlock, 0, c.stream>>>(v, R, r, ldr, G, D, c.st, c.partials, done);
+    if (v.n_heavy > 0) {
+        k_spmm_heavy<T, LN><<<std::min(v.n_heavy, c.grid), kBlock, 0, c.stream>>>(v, R, r, ldr, done);
+        ++*c.launches;
+    }
+    ALM_ROW_SPLIT(wide_rows(2 * v.nnz_u, v.n, LN), LN, {
+        auto *fn = k_spmm<T, LN, SPW, LRB, MODE>;
+        const int grid = grid_for(c, fn, v.n, kBlock / (LN * SPW));
+        fn<<<grid, kBlock, 0, c.stream>>>(v, R, r, ldr, G, D, c.st, c.partials, done);
+    });
 }
 
 template <typename T, int LN, int KF>
@@ -1113,9 +1130,11 @@ void launch_dir(const LaunchCtx &c, const T *G, T *D, int64_t count, const int *
 template <typename T, int LN, bool OFF, bool LRB, int MODE>
 static void ls_one(const LaunchCtx &c, const SparseView<T> &v, const T *R, const T *D, int r, int ldr,
                    const int *done) {
-    auto *fn = k_ls<T, LN, OFF, LRB, MODE>;
-    const int grid = grid_for(c, fn, v.n, 2 * (kBlock / LN));
-    fn<<<grid, kBlock, 0, c.stream>>>(v, R, D, r, ldr, c.st, c.partials, done);
+    ALM_ROW_SPLIT(wide_rows(v.nnz_u, v.n, LN), LN, {
+        auto *fn = k_ls<T, LN, SPW, OFF, LRB, MODE>;
+        const int grid = grid_for(c, fn, v.n + v.n_useg, kBlock / (LN * SPW));
+        fn<<<grid, kBlock, 0, c.stream>>>(v, R, D, r, ldr, c.st, c.partials, done);
+    });
 }
 
 template <typename T, int LN, int KU>
