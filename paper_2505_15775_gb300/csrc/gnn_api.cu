@@ -72,6 +72,11 @@ GnnGraph graph_of(const alm_batch *hb) {
     return gr;
 }
 
+// CTAs (and vectors of gradient partials) of the backward kernels: two per multiprocessor
+int grad_blocks(const alm_gnn *g, int64_t rows) {
+    return int(std::max<int64_t>(1, std::min<int64_t>(2 * int64_t(g->sms), (rows + 63) / 64)));
+}
+
 template <typename T>
 void carve(alm_gnn *g, GnnActs<T> &a, int64_t rows, bool training) {
     T *p = static_cast<T *>(g->act);
@@ -87,18 +92,17 @@ void carve(alm_gnn *g, GnnActs<T> &a, int64_t rows, bool training) {
         a.AGG[l] = p;
         p += rows * kGnnHid;
     }
+    const int64_t rows4 = (rows + 3) / 4 * 4;  // what follows is read by 16-byte vectors
     float *f = g->fbuf;
     g->rhat = f;
     f += rows * kGnnRank;
     g->yhat = f;
-    f += rows;
+    f += rows4;
     if (training) {
         a.dR = f;
         f += rows * kGnnRank;
         a.dY = f;
-        f += rows;
-        a.dH = f;
-        f += rows * kGnnHid;
+        f += rows4;
         a.dZ = f;
         f += rows * kGnnHid;
         a.dHp = f;
@@ -108,8 +112,8 @@ void carve(alm_gnn *g, GnnActs<T> &a, int64_t rows, bool training) {
         a.part = f;
         a.lpart = g->lpart;
     }
-    a.nblk = std::max(1, std::min(2 * g->sms, int((rows + 31) / 32)));
-    a.ldp = kGnnLdp;
+    a.nblk = grad_blocks(g, rows);
+    a.ldp = gnn_ldp();
 }
 
 alm_status ensure_buffers(alm_gnn *g, int64_t rows, bool training) {
@@ -124,11 +128,9 @@ alm_status ensure_buffers(alm_gnn *g, int64_t rows, bool training) {
         g->trainbufs = false;
         const size_t esz = g->storage == ALM_GNN_BF16 ? 2 : 4;
         const size_t acts = size_t(cap) * (2 * kGnnFeat + (2 * kGnnLayers - 1) * kGnnHid);
-        size_t fl = size_t(cap) * (kGnnRank + 1);
-        if (tr) {
-            const int nblk = std::max(1, std::min(2 * g->sms, int((cap + 31) / 32)));
-            fl += size_t(cap) * (kGnnRank + 1 + 4 * kGnnHid) + size_t(nblk) * size_t(kGnnLdp);
-        }
+        size_t fl = size_t(cap) * (kGnnRank + 1) + 4;
+        if (tr)
+            fl += size_t(cap) * (kGnnRank + 1 + 3 * kGnnHid) + 4 + size_t(grad_blocks(g, cap)) * size_t(gnn_ldp());
         GCK(cudaMalloc(&g->act, esz * acts));
         GCK(cudaMalloc(&g->fbuf, sizeof(float) * fl));
         g->cap_rows = cap;
@@ -142,32 +144,31 @@ alm_status ensure_buffers(alm_gnn *g, int64_t rows, bool training) {
     return ALM_OK;
 }
 
-alm_status forward(alm_gnn *g, const alm_batch *hb) {
+alm_status forward(alm_gnn *g, const alm_batch *hb, bool store) {
     const GnnGraph gr = graph_of(hb);
     const GnnParams p = gnn_views(g->theta);
     cudaError_t e;
-    if (g->storage == ALM_GNN_BF16) e = gnn_forward(gr, p, g->feat_seed, g->a16, g->rhat, g->yhat, g->sms, g->stream);
-    else e = gnn_forward(gr, p, g->feat_seed, g->a32, g->rhat, g->yhat, g->sms, g->stream);
-    g->launches += 2 + kGnnLayers;
+    if (g->storage == ALM_GNN_BF16) e = gnn_forward(gr, p, g->feat_seed, g->a16, g->rhat, g->yhat, store, g->sms, g->stream);
+    else e = gnn_forward(gr, p, g->feat_seed, g->a32, g->rhat, g->yhat, store, g->sms, g->stream);
+    g->launches += 1 + kGnnLayers;
     GCK(e);
     return ALM_OK;
 }
 
 // loss and gradient into g->grad (device); the loss in g->loss (device)
 alm_status loss_grad(alm_gnn *g, const alm_batch *hb, const float *Rs, const double *ys, double lam) {
-    GTRY(forward(g, hb));
+    GTRY(forward(g, hb, true));
     const GnnGraph gr = graph_of(hb);
     const GnnParams p = gnn_views(g->theta);
-    const GnnParams gp = gnn_views(g->grad);
     const double npat = double(hb->rows) + 0.5 * double(hb->nnz);  // diagonal + strict upper entries
     cudaError_t e;
     if (g->storage == ALM_GNN_BF16)
-        e = gnn_loss_grad(gr, p, gp, g->a16, g->rhat, g->yhat, Rs, ys, hb->cbar, lam, npat, double(hb->rows), g->loss,
+        e = gnn_loss_grad(gr, p, g->grad, g->a16, g->rhat, g->yhat, Rs, ys, hb->cbar, lam, npat, double(hb->rows), g->loss,
                           g->sms, g->stream);
     else
-        e = gnn_loss_grad(gr, p, gp, g->a32, g->rhat, g->yhat, Rs, ys, hb->cbar, lam, npat, double(hb->rows), g->loss,
+        e = gnn_loss_grad(gr, p, g->grad, g->a32, g->rhat, g->yhat, Rs, ys, hb->cbar, lam, npat, double(hb->rows), g->loss,
                           g->sms, g->stream);
-    g->launches += 30;
+    g->launches += 4 + 2 * (kGnnLayers - 1);
     GCK(e);
     return ALM_OK;
 }
@@ -288,7 +289,7 @@ extern "C" alm_status alm_gnn_forward(alm_gnn *g, const alm_batch *hb, float *rh
     if (!g) return ALM_ERR_INVALID_ARG;
     GTRY(check_batch_arrays(g, hb));
     GTRY(ensure_buffers(g, hb->rows, false));
-    GTRY(forward(g, hb));
+    GTRY(forward(g, hb, false));
     if (rhat)
         GCK(cudaMemcpyAsync(rhat, g->rhat, sizeof(float) * size_t(hb->rows) * kGnnRank, cudaMemcpyDeviceToDevice,
                             g->stream));
@@ -304,7 +305,7 @@ extern "C" alm_status alm_gnn_warm_start(alm_gnn *g, const alm_batch *hb, double
     GTRY(check_batch_arrays(g, hb));
     if (reinterpret_cast<uintptr_t>(R0) % 16 != 0) GFAIL(ALM_ERR_INVALID_ARG, "R0 must be 16-byte aligned");
     GTRY(ensure_buffers(g, hb->rows, false));
-    GTRY(forward(g, hb));
+    GTRY(forward(g, hb, false));
     if (!(mix >= 0.0) || !std::isfinite(mix)) GFAIL(ALM_ERR_INVALID_ARG, "mix must be finite and >= 0");
     GCK(gnn_warm(graph_of(hb), g->rhat, g->yhat, hb->cbar, float(mix), g->feat_seed ^ 0x3a1dULL, R0, y0, g->sms,
                  g->stream));

@@ -63,23 +63,33 @@ template <typename T>
 struct GnnActs {
     T *H[kGnnLayers + 1] = {nullptr, nullptr, nullptr, nullptr};  // H[0]: rows x 8, H[1..3]: rows x 64
     T *AGG[kGnnLayers] = {nullptr, nullptr, nullptr};               // rows x din of each layer
-    float *dR = nullptr, *dY = nullptr, *dH = nullptr, *dZ = nullptr, *dHp = nullptr, *U = nullptr;
-    float *part = nullptr;   // nblk x ldp weight-gradient partials
+    float *dR = nullptr, *dY = nullptr, *dZ = nullptr, *dHp = nullptr, *U = nullptr;
+    float *part = nullptr;   // nblk x ldp gradient partials, a whole parameter vector per block
     double *lpart = nullptr; // loss partials (one per CTA of the loss kernel)
     int nblk = 0;
     int64_t ldp = 0;
 };
-constexpr int64_t kGnnLdp = int64_t(kGnnHid) * kGnnHid + kGnnHid;  // widest partial: 64 x 64 + 64
+inline int64_t gnn_ldp() { return (gnn_num_params() + 31) / 32 * 32; }
 
+// One layer of the forward pass: parameters, input and output activations, heads (last layer).
+template <typename T>
+struct GnnLayerArgs {
+    const float *Ws, *Wn, *bias, *WR, *wy, *by;
+    const T *H;
+    T *AGG, *Hout;
+    float *rhat, *yhat;
+};
+
+// store: keep the activations that the backward pass reads (all AGG and the last H)
 template <typename T>
 cudaError_t gnn_forward(const GnnGraph &g, const GnnParams &p, uint64_t feat_seed, GnnActs<T> &a, float *rhat,
-                        float *yhat, int sms, cudaStream_t s);
+                        float *yhat, bool store, int sms, cudaStream_t s);
 cudaError_t gnn_warm(const GnnGraph &g, const float *rhat, const float *yhat, const double *cbar, float mix,
                      uint64_t mix_seed, float *R0, double *y0, int sms, cudaStream_t s);
 template <typename T>
-cudaError_t gnn_loss_grad(const GnnGraph &g, const GnnParams &p, const GnnParams &grad, GnnActs<T> &a,
-                          const float *rhat, const float *yhat, const float *Rs, const double *ys, const double *cbar,
-                          double lam, double n_pattern, double n_rows, double *loss_dev, int sms, cudaStream_t s);
+cudaError_t gnn_loss_grad(const GnnGraph &g, const GnnParams &p, float *grad, GnnActs<T> &a, const float *rhat,
+                          const float *yhat, const float *Rs, const double *ys, const double *cbar, double lam,
+                          double n_pattern, double n_rows, double *loss_dev, int sms, cudaStream_t s);
 cudaError_t gnn_adam(float *theta, const float *grad, float *m, float *v, int cnt, double lr, int step,
                      cudaStream_t s);
 

@@ -6,9 +6,11 @@
 //     agg_i = (sum_j a_ij h_j) / max(deg_i, 1),   h'_i = relu(Ws h_i + Wn agg_i + b),
 // a_ij = C_ij / mean|C_ij|, then the heads rhat_i = W_R h_i (32 columns) and
 // yhat_i = w_y . h_i + b_y.  Activations are stored in BF16 (or FP32) and every product
-// accumulates in FP32; gradients are FP32.  The 64-wide layers move ~0.5 KB per row and
-// do ~16 KFLOP per row: they stay on the CUDA cores (below the tensor-core ridge once
-// the neighbour gathers are counted), one warp per row with the weights in shared memory.
+// accumulates in FP32; gradients are FP32.  The products stay FP32 FMAs in a fixed order per
+// output: a BF16 activation is rounded from the FP32 sum, and a sum in another order (or from
+// split operands on the tensor cores) rounds some of them the other way, 2^-8 off.  A 64-wide
+// layer is then 8192 FMAs a row, bound by the FP32 pipe, provided that its operands come from
+// registers: tiles of rows (k_gnn_layer), each thread 8 rows x 4 outputs.
 //
 // Rows are the global rows of a batch (alm_batch); row g belongs to instance
 // row_inst[g], whose first row is row_off[row_inst[g]] and whose pattern uses local
@@ -40,12 +42,14 @@ __device__ __forceinline__ float warp_sumf(float x) {
 
 // SplitMix64 counter generator mapped to [-1, 1) (the same definition as the Lanczos
 // start vector)
+// (m 2^-52 - 1 for the 53-bit integer m, which FP64 holds exactly, rounded to float once:
+// the integer m - 2^52 converted and scaled gives the same float without the FP64 pipe)
 __device__ __forceinline__ float smx_pm1(uint64_t seed, uint64_t i) {
     uint64_t z = seed + (i + 1) * 0x9e3779b97f4a7c15ULL;
     z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ULL;
     z = (z ^ (z >> 27)) * 0x94d049bb133111ebULL;
     z ^= z >> 31;
-    return float(2.0 * (double(z >> 11) * (1.0 / 9007199254740992.0)) - 1.0);
+    return __ll2float_rn(static_cast<long long>(z >> 11) - (1LL << 52)) * 0x1p-52f;
 }
 
 // x_i = [1, deg_i/dbar, s_i/sbar, log(n)/8, u_1..u_4]
@@ -67,97 +71,277 @@ __global__ void k_gnn_features(GnnGraph g, uint64_t feat_seed, T *__restrict__ H
     }
 }
 
-// One layer, one warp per row: agg (stored for the backward), h' = relu(Ws h + Wn agg + b).
-// Lane l owns inputs l and l + 32 (DIN = 64) or input l (DIN = 8, l < 8), outputs l, l + 32.
-template <typename T, int DIN>
-__global__ void __launch_bounds__(256) k_gnn_layer_fwd(GnnGraph g, const float *__restrict__ Ws,
-                                                       const float *__restrict__ Wn, const float *__restrict__ bias,
-                                                       const T *__restrict__ H, T *__restrict__ AGG,
-                                                       T *__restrict__ Hout) {
-    __shared__ float ws[kGnnHid * (DIN + 1)], wn[kGnnHid * (DIN + 1)], bs[kGnnHid];
-    __shared__ float hv[8][DIN], av[8][DIN];
-    for (int t = threadIdx.x; t < kGnnHid * DIN; t += blockDim.x) {
-        const int o = t / DIN, k = t % DIN;
-        ws[o * (DIN + 1) + k] = Ws[t];
-        wn[o * (DIN + 1) + k] = Wn[t];
-    }
-    for (int t = threadIdx.x; t < kGnnHid; t += blockDim.x) bs[t] = bias[t];
-    __syncthreads();
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int64_t nwarps = int64_t(gridDim.x) * (blockDim.x >> 5);
-    for (int64_t r = int64_t(blockIdx.x) * (blockDim.x >> 5) + wid; r < g.rows; r += nwarps) {
-        const int b = g.row_inst[r];
-        const int64_t base = g.row_off[b];
-        const float icb = g.scal[b].y;
-        const int e0 = g.rowptr[r], e1 = g.rowptr[r + 1];
-        float a0 = 0.f, a1 = 0.f;
-        for (int e = e0; e < e1; ++e) {
-            const float a = g.val[e] * icb;
-            const T *hj = H + (base + g.col[e]) * DIN;
-            if (DIN == 64) {
-                a0 = fmaf(a, tof(hj[lane]), a0);
-                a1 = fmaf(a, tof(hj[lane + 32]), a1);
-            } else if (lane < DIN) {
-                a0 = fmaf(a, tof(hj[lane]), a0);
-            }
+// two neighbouring channels of a row
+__device__ __forceinline__ float2 ld2(const float *p) { return *reinterpret_cast<const float2 *>(p); }
+__device__ __forceinline__ float2 ld2(const __nv_bfloat16 *p) {
+    return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p));
+}
+__device__ __forceinline__ void st2(float *p, float x, float y) { *reinterpret_cast<float2 *>(p) = make_float2(x, y); }
+__device__ __forceinline__ void st2(__nv_bfloat16 *p, __nv_bfloat16 x, __nv_bfloat16 y) {
+    *reinterpret_cast<__nv_bfloat162 *>(p) = __halves2bfloat162(x, y);
+}
+// four neighbouring channels
+__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ float4 ld4(const __nv_bfloat16 *p) {
+    const uint2 u = *reinterpret_cast<const uint2 *>(p);
+    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u.x));
+    const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u.y));
+    return make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ void st4(float *p, const float (&q)[4]) {
+    *reinterpret_cast<float4 *>(p) = make_float4(q[0], q[1], q[2], q[3]);
+}
+__device__ __forceinline__ void st4(__nv_bfloat16 *p, const float (&q)[4]) {
+    st2(p, __float2bfloat16_rn(q[0]), __float2bfloat16_rn(q[1]));
+    st2(p + 2, __float2bfloat16_rn(q[2]), __float2bfloat16_rn(q[3]));
+}
+// N consecutive floats of shared memory (N = 2 or a multiple of 4) into registers
+template <int N>
+__device__ __forceinline__ void lds_vec(const float *p, float (&x)[N]) {
+    if constexpr (N == 2) {
+        const float2 v = *reinterpret_cast<const float2 *>(p);
+        x[0] = v.x;
+        x[1] = v.y;
+    } else {
+#pragma unroll
+        for (int q = 0; q < N / 4; ++q) {
+            const float4 v = *reinterpret_cast<const float4 *>(p + 4 * q);
+            x[4 * q] = v.x;
+            x[4 * q + 1] = v.y;
+            x[4 * q + 2] = v.z;
+            x[4 * q + 3] = v.w;
         }
-        const float inv = 1.f / float(max(e1 - e0, 1));
-        const T *hi = H + r * DIN;
-        __syncwarp();
-        if (DIN == 64) {
-            const T q0 = fromf<T>(a0 * inv), q1 = fromf<T>(a1 * inv);
-            AGG[r * DIN + lane] = q0;
-            AGG[r * DIN + lane + 32] = q1;
-            hv[wid][lane] = tof(hi[lane]);
-            hv[wid][lane + 32] = tof(hi[lane + 32]);
-            av[wid][lane] = tof(q0);  // the backward sees the stored (rounded) value
-            av[wid][lane + 32] = tof(q1);
-        } else if (lane < DIN) {
-            const T q0 = fromf<T>(a0 * inv);
-            AGG[r * DIN + lane] = q0;
-            hv[wid][lane] = tof(hi[lane]);
-            av[wid][lane] = tof(q0);
-        }
-        __syncwarp();
-        float z0 = bs[lane], z1 = bs[lane + 32];
-#pragma unroll 8
-        for (int k = 0; k < DIN; ++k) {
-            const float h = hv[wid][k], a = av[wid][k];
-            z0 = fmaf(ws[lane * (DIN + 1) + k], h, fmaf(wn[lane * (DIN + 1) + k], a, z0));
-            z1 = fmaf(ws[(lane + 32) * (DIN + 1) + k], h, fmaf(wn[(lane + 32) * (DIN + 1) + k], a, z1));
-        }
-        Hout[r * kGnnHid + lane] = fromf<T>(fmaxf(z0, 0.f));
-        Hout[r * kGnnHid + lane + 32] = fromf<T>(fmaxf(z1, 0.f));
-        __syncwarp();
     }
 }
 
-// heads: rhat = W_R h (lane c -> column c), yhat = w_y . h + b_y
-template <typename T>
-__global__ void __launch_bounds__(256) k_gnn_heads(GnnGraph g, const float *__restrict__ WR,
-                                                   const float *__restrict__ wy, const float *__restrict__ by,
-                                                   const T *__restrict__ H, float *__restrict__ rhat,
-                                                   float *__restrict__ yhat) {
-    __shared__ float wr[kGnnRank * (kGnnHid + 1)], wys[kGnnHid];
-    __shared__ float hv[8][kGnnHid];
-    for (int t = threadIdx.x; t < kGnnRank * kGnnHid; t += blockDim.x) wr[(t / kGnnHid) * (kGnnHid + 1) + t % kGnnHid] = WR[t];
-    for (int t = threadIdx.x; t < kGnnHid; t += blockDim.x) wys[t] = wy[t];
+// One layer over tiles of TR rows: agg_i, h'_i = relu(Ws h_i + Wn agg_i + b), and with HEADS
+// (the last layer) rhat_i = W_R h'_i, yhat_i = w_y . h'_i + b_y from the tile in shared memory.
+// STORE: keep agg and, in the last layer, h' for the backward pass (inference needs neither).
+//   gather   64 channels: a warp takes four rows at once, a lane two channels of each; the rows'
+//            columns and weights are loaded by the lanes beforehand, so that the gathers of up
+//            to eight neighbour rows (two per row) are in flight.  8 channels: two threads a row.
+//   product  thread (rg, og) holds TR / 16 rows x 4 outputs; inputs lie transposed in shared
+//            memory ([channel][row]), so an input costs TR / 16 x 4 FMAs per 16-byte load.
+//            Per output the FMAs run over k in order, Wn's before Ws's, from the bias on.
+// 128 rows a tile hold the FP32 pipe busy (6 shared loads per 64 FMAs); fewer rows than one
+// such tile per multiprocessor take tiles of 32, to use more of them.
+// Bound: the FP32 pipe (8192 FMAs a row: 0.21 ms per million rows) and the gathers.  One warp
+// per row with both operands of every FMA from shared memory took 1.25 ms a layer on 1e6 torus
+// rows and 0.37 ms for the heads: alm_gnn_warm_start 3.60 -> 1.56 ms.
+template <int DIN, int TR, bool HEADS>
+constexpr int gnn_layer_smem() {
+    return 4 * (DIN * (2 * kGnnHid + 4) + kGnnHid + 2 * DIN * (TR + 4) +
+                (HEADS ? kGnnHid * (kGnnRank + 4) + kGnnHid : 0));
+}
+template <typename T, int DIN, int TR, bool HEADS, bool STORE>
+__global__ void __launch_bounds__(256, 2) k_gnn_layer(GnnGraph g, GnnLayerArgs<T> p) {
+    extern __shared__ __align__(16) float gsm[];
+    constexpr int WP = 2 * kGnnHid + 4;  // pitch of [k][Ws row | Wn row]
+    constexpr int TP = TR + 4;           // pitch of [k][row]
+    constexpr int RPT = TR / 16;         // rows per thread of the product
+    float *w = gsm, *bs = w + DIN * WP, *hx = bs + kGnnHid, *ax = hx + DIN * TP, *wr = ax + DIN * TP;
+    float *wy = wr + kGnnHid * (kGnnRank + 4);
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    for (int t = tid; t < kGnnHid * DIN; t += 256) {
+        const int o = t / DIN, k = t % DIN;
+        w[k * WP + o] = p.Ws[t];
+        w[k * WP + kGnnHid + o] = p.Wn[t];
+    }
+    for (int t = tid; t < kGnnHid; t += 256) bs[t] = p.bias[t];
+    float by = 0.f;
+    if (HEADS) {
+        for (int t = tid; t < kGnnRank * kGnnHid; t += 256) wr[(t % kGnnHid) * (kGnnRank + 4) + t / kGnnHid] = p.WR[t];
+        for (int t = tid; t < kGnnHid; t += 256) wy[t] = p.wy[t];
+        by = p.by[0];
+    }
     __syncthreads();
-    const float b0 = by[0];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int64_t nwarps = int64_t(gridDim.x) * (blockDim.x >> 5);
-    for (int64_t r = int64_t(blockIdx.x) * (blockDim.x >> 5) + wid; r < g.rows; r += nwarps) {
-        const float h0 = tof(H[r * kGnnHid + lane]), h1 = tof(H[r * kGnnHid + lane + 32]);
-        hv[wid][lane] = h0;
-        hv[wid][lane + 32] = h1;
-        __syncwarp();
-        float acc = 0.f;
+    const int og = tid & 15, rg = tid >> 4;
+    for (int64_t r0 = int64_t(blockIdx.x) * TR; r0 < g.rows; r0 += int64_t(gridDim.x) * TR) {
+        if constexpr (DIN == kGnnHid) {
+            for (int q4 = 0; q4 < TR / 8; q4 += 4) {  // four rows at once
+                const int lr = wid * (TR / 8) + q4;
+                int64_t base = 0;
+                int e0 = 0, e1 = 0;
+                float icb = 0.f;
+                if (lane < 4 && r0 + lr + lane < g.rows) {
+                    const int64_t r = r0 + lr + lane;
+                    const int b = g.row_inst[r];
+                    base = g.row_off[b];
+                    icb = g.scal[b].y;
+                    e0 = g.rowptr[r];
+                    e1 = g.rowptr[r + 1];
+                }
+                float a0[4] = {0.f, 0.f, 0.f, 0.f}, a1[4] = {0.f, 0.f, 0.f, 0.f};
+                int deg[4];
+                int most = 0;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    deg[q] = __shfl_sync(0xffffffffu, e1 - e0, q);
+                    most = max(most, deg[q]);
+                }
+                float2 own[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int64_t r = r0 + lr + q;
+                    own[q] = r < g.rows ? ld2(p.H + r * DIN + 2 * lane) : make_float2(0.f, 0.f);
+                }
+                for (int c0 = 0; c0 < most; c0 += 32) {  // 32 entries of each row at a time
+                    int64_t jr[4];
+                    float aw[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const int64_t bq = __shfl_sync(0xffffffffu, base, q);
+                        const int eq = __shfl_sync(0xffffffffu, e0, q) + c0 + lane;
+                        const float iq = __shfl_sync(0xffffffffu, icb, q);
+                        const bool in = c0 + lane < deg[q];
+                        jr[q] = in ? bq + g.col[eq] : 0;
+                        aw[q] = in ? g.val[eq] * iq : 0.f;
+                    }
+                    const int lim = min(32, most - c0);
+                    for (int t = 0; t < lim; t += 2) {
+                        float2 x[2][4];
+                        float a[2][4];
+#pragma unroll
+                        for (int u = 0; u < 2; ++u)
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                const int64_t j = __shfl_sync(0xffffffffu, jr[q], (t + u) & 31);
+                                a[u][q] = __shfl_sync(0xffffffffu, aw[q], (t + u) & 31);
+                                x[u][q] = make_float2(0.f, 0.f);
+                                if (t + u < 32 && c0 + t + u < deg[q]) x[u][q] = ld2(p.H + j * DIN + 2 * lane);
+                            }
+#pragma unroll
+                        for (int u = 0; u < 2; ++u)
+#pragma unroll
+                            for (int q = 0; q < 4; ++q)
+                                if (t + u < 32 && c0 + t + u < deg[q]) {  // warp-uniform
+                                    a0[q] = fmaf(a[u][q], x[u][q].x, a0[q]);
+                                    a1[q] = fmaf(a[u][q], x[u][q].y, a1[q]);
+                                }
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float inv = 1.f / float(max(deg[q], 1));
+                    const T q0 = fromf<T>(a0[q] * inv), q1 = fromf<T>(a1[q] * inv);
+                    if (STORE && r0 + lr + q < g.rows) st2(p.AGG + (r0 + lr + q) * DIN + 2 * lane, q0, q1);
+                    a0[q] = tof(q0);  // the backward sees the stored (rounded) value
+                    a1[q] = tof(q1);
+                }
+                *reinterpret_cast<float4 *>(hx + (2 * lane) * TP + lr) = make_float4(own[0].x, own[1].x, own[2].x, own[3].x);
+                *reinterpret_cast<float4 *>(hx + (2 * lane + 1) * TP + lr) = make_float4(own[0].y, own[1].y, own[2].y, own[3].y);
+                *reinterpret_cast<float4 *>(ax + (2 * lane) * TP + lr) = make_float4(a0[0], a0[1], a0[2], a0[3]);
+                *reinterpret_cast<float4 *>(ax + (2 * lane + 1) * TP + lr) = make_float4(a1[0], a1[1], a1[2], a1[3]);
+            }
+        } else {
+            for (int t = tid; t < 2 * TR; t += 256) {  // two threads a row, four channels each
+                const int lr = t >> 1, c = 4 * (t & 1);
+                const int64_t r = r0 + lr;
+                float q[4] = {0.f, 0.f, 0.f, 0.f}, h[4] = {0.f, 0.f, 0.f, 0.f};
+                if (r < g.rows) {
+                    const int b = g.row_inst[r];
+                    const int64_t base = g.row_off[b];
+                    const float icb = g.scal[b].y;
+                    const int e0 = g.rowptr[r], e1 = g.rowptr[r + 1];
+                    const float4 o = ld4(p.H + r * DIN + c);
+                    h[0] = o.x, h[1] = o.y, h[2] = o.z, h[3] = o.w;
+                    for (int e = e0; e < e1; e += 4) {
+                        float4 x[4];
+                        float a[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const int ee = min(e + u, e1 - 1);
+                            a[u] = g.val[ee] * icb;
+                            x[u] = ld4(p.H + (base + g.col[ee]) * DIN + c);
+                        }
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (e + u < e1) {
+                                q[0] = fmaf(a[u], x[u].x, q[0]);
+                                q[1] = fmaf(a[u], x[u].y, q[1]);
+                                q[2] = fmaf(a[u], x[u].z, q[2]);
+                                q[3] = fmaf(a[u], x[u].w, q[3]);
+                            }
+                    }
+                    const float inv = 1.f / float(max(e1 - e0, 1));
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) q[k] = tof(fromf<T>(q[k] * inv));
+                    if (STORE) st4(p.AGG + r * DIN + c, q);
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    hx[(c + k) * TP + lr] = h[k];
+                    ax[(c + k) * TP + lr] = q[k];
+                }
+            }
+        }
+        __syncthreads();
+        float z[RPT][4];
+#pragma unroll
+        for (int i = 0; i < RPT; ++i)
+#pragma unroll
+            for (int o = 0; o < 4; ++o) z[i][o] = bs[4 * og + o];
+#pragma unroll 4
+        for (int k = 0; k < DIN; ++k) {
+            float h[RPT], a[RPT], ws[4], wn[4];
+            lds_vec<RPT>(hx + k * TP + RPT * rg, h);
+            lds_vec<RPT>(ax + k * TP + RPT * rg, a);
+            lds_vec<4>(w + k * WP + 4 * og, ws);
+            lds_vec<4>(w + k * WP + kGnnHid + 4 * og, wn);
+#pragma unroll
+            for (int i = 0; i < RPT; ++i)
+#pragma unroll
+                for (int o = 0; o < 4; ++o) z[i][o] = fmaf(ws[o], h[i], fmaf(wn[o], a[i], z[i][o]));
+        }
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) {
+            const int64_t r = r0 + RPT * rg + i;
+#pragma unroll
+            for (int o = 0; o < 4; ++o) z[i][o] = tof(fromf<T>(fmaxf(z[i][o], 0.f)));
+            if ((!HEADS || STORE) && r < g.rows) st4(p.Hout + r * kGnnHid + 4 * og, z[i]);
+        }
+        __syncthreads();  // hx and ax may be overwritten
+        if constexpr (HEADS) {
+#pragma unroll
+            for (int o = 0; o < 4; ++o)
+#pragma unroll
+                for (int i = 0; i < RPT; ++i) hx[(4 * og + o) * TP + RPT * rg + i] = z[i][o];
+            __syncthreads();
+            constexpr int RPH = TR / 32;  // rows per thread of the factor head (8 threads a row)
+            const int cg = tid & 7, rh = (tid >> 3) * RPH;
+            float acc[RPH][4];
+#pragma unroll
+            for (int i = 0; i < RPH; ++i)
+#pragma unroll
+                for (int o = 0; o < 4; ++o) acc[i][o] = 0.f;
+#pragma unroll 4
+            for (int k = 0; k < kGnnHid; ++k) {
+                float v[4];
+                lds_vec<4>(wr + k * (kGnnRank + 4) + 4 * cg, v);
+#pragma unroll
+                for (int i = 0; i < RPH; ++i) {
+                    const float h = hx[k * TP + rh + i];
+#pragma unroll
+                    for (int o = 0; o < 4; ++o) acc[i][o] = fmaf(v[o], h, acc[i][o]);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < RPH; ++i)
+                if (r0 + rh + i < g.rows)
+                    *reinterpret_cast<float4 *>(p.rhat + (r0 + rh + i) * kGnnRank + 4 * cg) =
+                        make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+            for (int lr = tid; lr < TR; lr += 256)
+                if (r0 + lr < g.rows) {
+                    float s0 = 0.f, s1 = 0.f;
 #pragma unroll 8
-        for (int k = 0; k < kGnnHid; ++k) acc = fmaf(wr[lane * (kGnnHid + 1) + k], hv[wid][k], acc);
-        rhat[r * kGnnRank + lane] = acc;
-        const float yv = warp_sumf(fmaf(wys[lane], h0, wys[lane + 32] * h1));
-        if (lane == 0) yhat[r] = yv + b0;
-        __syncwarp();
+                    for (int k = 0; k < kGnnHid; k += 2) {
+                        s0 = fmaf(wy[k], hx[k * TP + lr], s0);
+                        s1 = fmaf(wy[k + 1], hx[(k + 1) * TP + lr], s1);
+                    }
+                    p.yhat[r0 + lr] = (s0 + s1) + by;
+                }
+            __syncthreads();
+        }
     }
 }
 
@@ -199,204 +383,393 @@ __global__ void k_gnn_warm(GnnGraph g, const float *__restrict__ rhat, const flo
     }
 }
 
-// Loss and its gradient w.r.t. the heads' outputs, one warp per row i (lane c = column c):
+// Loss and its gradient w.r.t. the heads' outputs, 8 lanes per row i (a float4 of columns each):
 //   e_ii = |rhat_i|^2 - |r*_i|^2,  e_ij = rhat_i.rhat_j - r*_i.r*_j (j a pattern neighbour)
 //   dL/drhat_i = (4/np) e_ii rhat_i + (2/np) sum_j e_ij rhat_j   (both (i,j) and (j,i) in the
 //   full pattern, so each unordered pair reaches both rows);  loss terms e_ii^2 and, for j > i,
 //   e_ij^2;  ey = yhat_i - y*_i/cbar,  dL/dyhat_i = 2 lam ey / nrow.
-// Also dH3_i = W_R^T dr_i + w_y dy_i.  Per-block loss partials in part[block].
+// One reduction (3 shuffles) of the difference per neighbour; bound by the gathers of two
+// 128-byte rows per neighbour.  Per-block loss partials in part[block].
+__device__ __forceinline__ float dot4(float4 a, float4 b) {
+    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, a.x * b.x)));
+}
+__device__ __forceinline__ float oct_sum(float x, unsigned m) {
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(m, x, o);
+    return x;
+}
 __global__ void __launch_bounds__(256) k_gnn_loss(GnnGraph g, const float *__restrict__ rhat,
                                                   const float *__restrict__ yhat, const float *__restrict__ Rs,
                                                   const double *__restrict__ ys, const double *__restrict__ cbar,
-                                                  const float *__restrict__ WR, const float *__restrict__ wy,
-                                                  float inv_np, float lam_nrow, float *__restrict__ dR,
-                                                  float *__restrict__ dY, float *__restrict__ dH,
-                                                  double *__restrict__ part) {
-    __shared__ float wr[kGnnRank * (kGnnHid + 1)], wys[kGnnHid];
-    __shared__ float dv[8][kGnnRank];
+                                                  float inv_np, float lam_nrow, int rs_vec, float *__restrict__ dR,
+                                                  float *__restrict__ dY, double *__restrict__ part) {
     __shared__ double red[8];
-    for (int t = threadIdx.x; t < kGnnRank * kGnnHid; t += blockDim.x) wr[(t / kGnnHid) * (kGnnHid + 1) + t % kGnnHid] = WR[t];
-    for (int t = threadIdx.x; t < kGnnHid; t += blockDim.x) wys[t] = wy[t];
-    __syncthreads();
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int64_t nwarps = int64_t(gridDim.x) * (blockDim.x >> 5);
+    // the caller's rows may lie at any float address
+    auto ldrs = [&](int64_t row, int c) {
+        const float *q = Rs + row * kGnnRank + c;
+        return rs_vec ? ld4(q) : make_float4(q[0], q[1], q[2], q[3]);
+    };
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, gl = lane & 7;
+    const unsigned gm = 0xffu << (lane & ~7);
     float lsum = 0.f, lcomp = 0.f;
-    for (int64_t r = int64_t(blockIdx.x) * (blockDim.x >> 5) + wid; r < g.rows; r += nwarps) {
+    for (int64_t r = int64_t(blockIdx.x) * 32 + (threadIdx.x >> 3); r < g.rows; r += int64_t(gridDim.x) * 32) {
         const int b = g.row_inst[r];
         const int64_t base = g.row_off[b];
         const int64_t li = r - base;
-        const float ri = rhat[r * kGnnRank + lane], si = Rs[r * kGnnRank + lane];
-        const float eii = warp_sumf(ri * ri) - warp_sumf(si * si);
-        float d = 4.f * inv_np * eii * ri;
+        const float4 ri = ld4(rhat + r * kGnnRank + 4 * gl), si = ldrs(r, 4 * gl);
+        const float eii = oct_sum(dot4(ri, ri) - dot4(si, si), gm);
+        const float c0 = 4.f * inv_np * eii;
+        float4 d = make_float4(c0 * ri.x, c0 * ri.y, c0 * ri.z, c0 * ri.w);
         float le = eii * eii;
         const int e1 = g.rowptr[r + 1];
-        for (int e = g.rowptr[r]; e < e1; ++e) {
-            const int j = g.col[e];
-            const float rj = rhat[(base + j) * kGnnRank + lane], sj = Rs[(base + j) * kGnnRank + lane];
-            const float eij = warp_sumf(ri * rj) - warp_sumf(si * sj);
-            d = fmaf(2.f * inv_np * eij, rj, d);
-            if (j > li) le += eij * eij;
+        for (int e = g.rowptr[r]; e < e1; e += 2) {
+            const bool two = e + 1 < e1;
+            const int j0 = g.col[e], j1 = two ? g.col[e + 1] : j0;
+            const float4 ra = ld4(rhat + (base + j0) * kGnnRank + 4 * gl), sa = ldrs(base + j0, 4 * gl);
+            const float4 rb = ld4(rhat + (base + j1) * kGnnRank + 4 * gl), sb = ldrs(base + j1, 4 * gl);
+            const float ea = oct_sum(dot4(ri, ra) - dot4(si, sa), gm);
+            const float eb = two ? oct_sum(dot4(ri, rb) - dot4(si, sb), gm) : 0.f;  // uniform in the group
+            const float ca = 2.f * inv_np * ea, cb = 2.f * inv_np * eb;
+            d = make_float4(fmaf(cb, rb.x, fmaf(ca, ra.x, d.x)), fmaf(cb, rb.y, fmaf(ca, ra.y, d.y)),
+                            fmaf(cb, rb.z, fmaf(ca, ra.z, d.z)), fmaf(cb, rb.w, fmaf(ca, ra.w, d.w)));
+            if (j0 > li) le += ea * ea;
+            if (j1 > li) le += eb * eb;
         }
-        dR[r * kGnnRank + lane] = d;
-        const float ey = float(double(yhat[r]) - ys[r] / cbar[b]);
-        const float dy = 2.f * lam_nrow * ey;
-        if (lane == 0) {
-            dY[r] = dy;
+        *reinterpret_cast<float4 *>(dR + r * kGnnRank + 4 * gl) = d;
+        if (gl == 0) {
+            const float ey = float(double(yhat[r]) - ys[r] / cbar[b]);
+            dY[r] = 2.f * lam_nrow * ey;
             const float t = le * inv_np + lam_nrow * ey * ey;
             const float s2 = lsum + t;  // two-sum
             const float bb = s2 - lsum;
             lcomp += (lsum - (s2 - bb)) + (t - bb);
             lsum = s2;
         }
-        dv[wid][lane] = d;
-        __syncwarp();
-        float h0 = wys[lane] * dy, h1 = wys[lane + 32] * dy;
-#pragma unroll 8
-        for (int c = 0; c < kGnnRank; ++c) {
-            const float dc = dv[wid][c];
-            h0 = fmaf(wr[c * (kGnnHid + 1) + lane], dc, h0);
-            h1 = fmaf(wr[c * (kGnnHid + 1) + lane + 32], dc, h1);
-        }
-        dH[r * kGnnHid + lane] = h0;
-        dH[r * kGnnHid + lane + 32] = h1;
-        __syncwarp();
     }
-    if (lane == 0) red[wid] = double(lsum) + double(lcomp);
+    double l = double(lsum) + double(lcomp);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    if (lane == 0) red[wid] = l;
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
-        for (int w = 0; w < int(blockDim.x >> 5); ++w) t += red[w];
+        for (int w = 0; w < 8; ++w) t += red[w];
         part[blockIdx.x] = t;
     }
 }
 
-// Layer backward, one warp per row: dz = dH (.) [h' > 0] (stored), dHprev_i = Ws^T dz,
-// U_i = (Wn^T dz) / max(deg_i, 1) (the aggregation's adjoint is applied by k_gnn_agg_t).
-template <typename T, int DIN>
-__global__ void __launch_bounds__(256) k_gnn_layer_bwd(GnnGraph g, const float *__restrict__ Ws,
-                                                       const float *__restrict__ Wn, const T *__restrict__ Hout,
-                                                       const float *__restrict__ dH, float *__restrict__ dZ,
-                                                       float *__restrict__ dHprev, float *__restrict__ U,
-                                                       int want_prev) {
-    __shared__ float ws[kGnnHid * DIN], wn[kGnnHid * DIN];
-    __shared__ float zv[8][kGnnHid];
-    for (int t = threadIdx.x; t < kGnnHid * DIN; t += blockDim.x) {
-        ws[t] = Ws[t];
-        wn[t] = Wn[t];
-    }
-    __syncthreads();
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int64_t nwarps = int64_t(gridDim.x) * (blockDim.x >> 5);
-    for (int64_t r = int64_t(blockIdx.x) * (blockDim.x >> 5) + wid; r < g.rows; r += nwarps) {
-        const float z0 = tof(Hout[r * kGnnHid + lane]) > 0.f ? dH[r * kGnnHid + lane] : 0.f;
-        const float z1 = tof(Hout[r * kGnnHid + lane + 32]) > 0.f ? dH[r * kGnnHid + lane + 32] : 0.f;
-        dZ[r * kGnnHid + lane] = z0;
-        dZ[r * kGnnHid + lane + 32] = z1;
-        if (!want_prev) continue;
-        zv[wid][lane] = z0;
-        zv[wid][lane + 32] = z1;
-        __syncwarp();
-        const float inv = 1.f / float(max(g.rowptr[r + 1] - g.rowptr[r], 1));
-        for (int k = lane; k < DIN; k += 32) {
-            float s = 0.f, u = 0.f;
-#pragma unroll 8
-            for (int o = 0; o < kGnnHid; ++o) {
-                const float zo = zv[wid][o];
-                s = fmaf(ws[o * DIN + k], zo, s);
-                u = fmaf(wn[o * DIN + k], zo, u);
-            }
-            dHprev[r * DIN + k] = s;
-            U[r * DIN + k] = u * inv;
-        }
-        __syncwarp();
-    }
-}
+// The backward kernels work on tiles of kBwdRows rows in shared memory, 256 threads, two CTAs
+// per multiprocessor, each CTA walking tiles with its weight-gradient outputs in registers
+// (written once, as this block's vector of partials: part[block * ldp + parameter offset]).
+// A product's operands come as 16-byte shared loads for tiles of 4 x 4 or 4 x 8 outputs a
+// thread.  One warp per row with operands from shared memory, a kernel for each weight matrix
+// and a serial sum of 304 partials for each took 2.7 ms for a gradient on 137,000 rows
+// (1.1 M edges); the tiles take 1.2 ms, forward pass included.
+constexpr int kBwdRows = 64;
+constexpr int kBwdPitch = kGnnHid + 4;
 
-// dHprev_j += sum_{i in N(j)} a_ij U_i (the pattern is symmetric), one warp per row
-template <int DIN>
-__global__ void __launch_bounds__(256) k_gnn_agg_t(GnnGraph g, const float *__restrict__ U,
-                                                   float *__restrict__ dHprev) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int64_t nwarps = int64_t(gridDim.x) * (blockDim.x >> 5);
-    for (int64_t r = int64_t(blockIdx.x) * (blockDim.x >> 5) + wid; r < g.rows; r += nwarps) {
-        const int b = g.row_inst[r];
-        const int64_t base = g.row_off[b];
-        const float icb = g.scal[b].y;
-        float s0 = 0.f, s1 = 0.f;
-        const int e1 = g.rowptr[r + 1];
-        for (int e = g.rowptr[r]; e < e1; ++e) {
-            const float a = g.val[e] * icb;
-            const float *uj = U + (base + g.col[e]) * DIN;
-            if (lane < DIN) s0 = fmaf(a, uj[lane], s0);
-            if (DIN == 64) s1 = fmaf(a, uj[lane + 32], s1);
-        }
-        if (lane < DIN) dHprev[r * DIN + lane] += s0;
-        if (DIN == 64) dHprev[r * DIN + lane + 32] += s1;
-    }
-}
-
-// Per-block partial of sum_rows A_r^T B_r (M x K, A FP32 rows x M, B rows x K in T) and,
-// when `colsum`, of sum_rows A_r (M): tiles of 32 rows staged in shared memory; thread t
-// owns outputs t, t + blockDim, ...  part[block * ldp + ...].
-template <typename T, int M, int K>
-__global__ void __launch_bounds__(256) k_gnn_outer(const float *__restrict__ A, const T *__restrict__ B, int64_t rows,
-                                                   int colsum, float *__restrict__ part, int64_t ldp) {
-    constexpr int TR = 32;
-    constexpr int NOUT = M * K;
-    constexpr int PER = (NOUT + 255) / 256;
-    __shared__ float at[TR][M], bt[TR][K];
-    float acc[PER];
+// Heads: dW_R = dR^T H3, dw_y = dY^T H3, db_y = sum dY, and the last layer's
+// dZ = (W_R^T dR + w_y dY) (.) [H3 > 0]
+template <typename T>
+__global__ void __launch_bounds__(256, 2) k_gnn_heads_bwd(int64_t rows, const float *__restrict__ dR,
+                                                          const float *__restrict__ dY, const T *__restrict__ H,
+                                                          const float *__restrict__ WR, const float *__restrict__ wy,
+                                                          float *__restrict__ dZ, float *__restrict__ part, int64_t ldp,
+                                                          int off_WR, int off_wy, int off_by) {
+    __shared__ __align__(16) float dt[kGnnRank][kBwdRows + 4], hs[kBwdRows][kBwdPitch], wr[kGnnRank][kBwdPitch];
+    __shared__ __align__(16) float drow[kBwdRows][kGnnRank + 4], wys[kGnnHid], dys[kBwdRows];
+    const int tid = threadIdx.x;
+    for (int t = tid; t < kGnnRank * kGnnHid; t += 256) wr[t / kGnnHid][t % kGnnHid] = WR[t];
+    if (tid < kGnnHid) wys[tid] = wy[tid];
+    const int kg = tid & 15, mg = tid >> 4;  // 4 channels x (2 columns | 4 rows)
+    float acc[2][4], accy = 0.f, accb = 0.f;
 #pragma unroll
-    for (int q = 0; q < PER; ++q) acc[q] = 0.f;
-    float cs = 0.f;
-    for (int64_t r0 = int64_t(blockIdx.x) * TR; r0 < rows; r0 += int64_t(gridDim.x) * TR) {
-        for (int t = threadIdx.x; t < TR * M; t += blockDim.x) {
-            const int64_t r = r0 + t / M;
-            at[t / M][t % M] = r < rows ? A[r * M + t % M] : 0.f;
-        }
-        for (int t = threadIdx.x; t < TR * K; t += blockDim.x) {
-            const int64_t r = r0 + t / K;
-            bt[t / K][t % K] = r < rows ? tof(B[r * K + t % K]) : 0.f;
-        }
-        __syncthreads();
+    for (int m = 0; m < 2; ++m)
 #pragma unroll
-        for (int q = 0; q < PER; ++q) {
-            const int o = threadIdx.x + q * 256;
-            if (o < NOUT) {
-                const int m = o / K, k = o % K;
-                float s = acc[q];
-#pragma unroll 8
-                for (int rr = 0; rr < TR; ++rr) s = fmaf(at[rr][m], bt[rr][k], s);
-                acc[q] = s;
-            }
-        }
-        if (colsum && threadIdx.x < M)
-            for (int rr = 0; rr < TR; ++rr) cs += at[rr][threadIdx.x];
+        for (int k = 0; k < 4; ++k) acc[m][k] = 0.f;
+    for (int64_t r0 = int64_t(blockIdx.x) * kBwdRows; r0 < rows; r0 += int64_t(gridDim.x) * kBwdRows) {
         __syncthreads();
+        for (int t = tid; t < kBwdRows * (kGnnRank / 4); t += 256) {
+            const int lr = t / (kGnnRank / 4), c = 4 * (t % (kGnnRank / 4));
+            const float4 x = r0 + lr < rows ? ld4(dR + (r0 + lr) * kGnnRank + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+            *reinterpret_cast<float4 *>(&drow[lr][c]) = x;
+            dt[c][lr] = x.x, dt[c + 1][lr] = x.y, dt[c + 2][lr] = x.z, dt[c + 3][lr] = x.w;
+        }
+        for (int t = tid; t < kBwdRows * (kGnnHid / 4); t += 256) {
+            const int lr = t / (kGnnHid / 4), c = 4 * (t % (kGnnHid / 4));
+            *reinterpret_cast<float4 *>(&hs[lr][c]) =
+                r0 + lr < rows ? ld4(H + (r0 + lr) * kGnnHid + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        if (tid < kBwdRows) dys[tid] = r0 + tid < rows ? dY[r0 + tid] : 0.f;
+        __syncthreads();
+#pragma unroll 4
+        for (int lr = 0; lr < kBwdRows; ++lr) {
+            float h[4], d[2];
+            lds_vec<4>(&hs[lr][4 * kg], h);
+            lds_vec<2>(&drow[lr][2 * mg], d);
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) acc[m][k] = fmaf(d[m], h[k], acc[m][k]);
+        }
+        if (tid < kGnnHid) {
+            for (int lr = 0; lr < kBwdRows; ++lr) accy = fmaf(dys[lr], hs[lr][tid], accy);
+        } else if (tid == kGnnHid) {
+            for (int lr = 0; lr < kBwdRows; ++lr) accb += dys[lr];
+        }
+        float z[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) z[i][k] = wys[4 * kg + k] * dys[4 * mg + i];
+#pragma unroll 4
+        for (int c = 0; c < kGnnRank; ++c) {
+            float d[4], w[4];
+            lds_vec<4>(&dt[c][4 * mg], d);
+            lds_vec<4>(&wr[c][4 * kg], w);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) z[i][k] = fmaf(w[k], d[i], z[i][k]);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int lr = 4 * mg + i;
+            if (r0 + lr >= rows) continue;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (!(hs[lr][4 * kg + k] > 0.f)) z[i][k] = 0.f;
+            st4(dZ + (r0 + lr) * kGnnHid + 4 * kg, z[i]);
+        }
     }
     float *p = part + int64_t(blockIdx.x) * ldp;
 #pragma unroll
-    for (int q = 0; q < PER; ++q) {
-        const int o = threadIdx.x + q * 256;
-        if (o < NOUT) p[o] = acc[q];
-    }
-    if (colsum && threadIdx.x < M) p[NOUT + threadIdx.x] = cs;
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) p[off_WR + (2 * mg + m) * kGnnHid + 4 * kg + k] = acc[m][k];
+    if (tid < kGnnHid) p[off_wy + tid] = accy;
+    else if (tid == kGnnHid) p[off_by] = accb;
 }
 
-// grad[dst + k] = sum over blocks of part[b * ldp + k], k < cnt (fixed order)
-__global__ void k_gnn_reduce(const float *__restrict__ part, int nblk, int64_t ldp, int cnt, float *__restrict__ grad) {
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < cnt; k += gridDim.x * blockDim.x) {
-        double s = 0.0;
-        for (int b = 0; b < nblk; ++b) s += double(part[int64_t(b) * ldp + k]);
-        grad[k] = float(s);
+// One 64-wide layer: dWs = dZ^T H, dWn = dZ^T AGG, db = sum dZ, and of its input
+// dHp = Ws^T dZ (the direct part) and U = (Wn^T dZ) / max(deg, 1) (its aggregation's adjoint is
+// applied by k_gnn_agg_t)
+template <typename T>
+constexpr int gnn_bwd_smem() { return 4 * (4 * kBwdRows * kBwdPitch + 2 * kGnnHid * kGnnHid); }
+template <typename T>
+__global__ void __launch_bounds__(256, 2) k_gnn_layer_bwd(GnnGraph g, const float *__restrict__ Ws,
+                                                          const float *__restrict__ Wn, const T *__restrict__ H,
+                                                          const T *__restrict__ AGG, const float *__restrict__ dZ,
+                                                          float *__restrict__ dHp, float *__restrict__ U,
+                                                          float *__restrict__ part, int64_t ldp, int off_Ws, int off_Wn,
+                                                          int off_b) {
+    extern __shared__ __align__(16) float gsm[];
+    constexpr int P = kBwdPitch;
+    float *ws = gsm, *wn = ws + kGnnHid * kGnnHid, *dz = wn + kGnnHid * kGnnHid;  // dz: [row][o]
+    float *dzt = dz + kBwdRows * P, *hs = dzt + kBwdRows * P, *as = hs + kBwdRows * P;  // dzt: [o][row]
+    const int tid = threadIdx.x;
+    for (int t = tid; t < kGnnHid * kGnnHid; t += 256) {
+        ws[t] = Ws[t];
+        wn[t] = Wn[t];
+    }
+    const int kg = tid & 15, mg = tid >> 4;
+    float accs[4][4], accn[4][4], accb = 0.f;
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) accs[m][k] = accn[m][k] = 0.f;
+    for (int64_t r0 = int64_t(blockIdx.x) * kBwdRows; r0 < g.rows; r0 += int64_t(gridDim.x) * kBwdRows) {
+        __syncthreads();
+        for (int t = tid; t < kBwdRows * (kGnnHid / 4); t += 256) {
+            const int lr = t / (kGnnHid / 4), c = 4 * (t % (kGnnHid / 4));
+            const int64_t r = r0 + lr;
+            const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 d = r < g.rows ? ld4(dZ + r * kGnnHid + c) : zero;
+            *reinterpret_cast<float4 *>(dz + lr * P + c) = d;
+            dzt[c * P + lr] = d.x, dzt[(c + 1) * P + lr] = d.y, dzt[(c + 2) * P + lr] = d.z, dzt[(c + 3) * P + lr] = d.w;
+            *reinterpret_cast<float4 *>(hs + lr * P + c) = r < g.rows ? ld4(H + r * kGnnHid + c) : zero;
+            *reinterpret_cast<float4 *>(as + lr * P + c) = r < g.rows ? ld4(AGG + r * kGnnHid + c) : zero;
+        }
+        __syncthreads();
+#pragma unroll 2
+        for (int lr = 0; lr < kBwdRows; ++lr) {
+            float d[4], h[4], a[4];
+            lds_vec<4>(dz + lr * P + 4 * mg, d);
+            lds_vec<4>(hs + lr * P + 4 * kg, h);
+            lds_vec<4>(as + lr * P + 4 * kg, a);
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    accs[m][k] = fmaf(d[m], h[k], accs[m][k]);
+                    accn[m][k] = fmaf(d[m], a[k], accn[m][k]);
+                }
+        }
+        if (tid < kGnnHid)
+            for (int lr = 0; lr < kBwdRows; ++lr) accb += dz[lr * P + tid];
+        float s[4][4], u[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) s[i][k] = u[i][k] = 0.f;
+#pragma unroll 2
+        for (int o = 0; o < kGnnHid; ++o) {
+            float d[4], w[4], v[4];
+            lds_vec<4>(dzt + o * P + 4 * mg, d);
+            lds_vec<4>(ws + o * kGnnHid + 4 * kg, w);
+            lds_vec<4>(wn + o * kGnnHid + 4 * kg, v);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    s[i][k] = fmaf(w[k], d[i], s[i][k]);
+                    u[i][k] = fmaf(v[k], d[i], u[i][k]);
+                }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int64_t r = r0 + 4 * mg + i;
+            if (r >= g.rows) continue;
+            const float inv = 1.f / float(max(g.rowptr[r + 1] - g.rowptr[r], 1));
+#pragma unroll
+            for (int k = 0; k < 4; ++k) u[i][k] *= inv;
+            st4(dHp + r * kGnnHid + 4 * kg, s[i]);
+            st4(U + r * kGnnHid + 4 * kg, u[i]);
+        }
+    }
+    float *p = part + int64_t(blockIdx.x) * ldp;
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            p[off_Ws + (4 * mg + m) * kGnnHid + 4 * kg + k] = accs[m][k];
+            p[off_Wn + (4 * mg + m) * kGnnHid + 4 * kg + k] = accn[m][k];
+        }
+    if (tid < kGnnHid) p[off_b + tid] = accb;
+}
+
+// The first layer's weight gradients (its input has none): dWs = dZ^T H0, dWn = dZ^T AGG0, db
+template <typename T>
+__global__ void __launch_bounds__(256) k_gnn_first_bwd(int64_t rows, const T *__restrict__ H,
+                                                       const T *__restrict__ AGG, const float *__restrict__ dZ,
+                                                       float *__restrict__ part, int64_t ldp, int off_Ws, int off_Wn,
+                                                       int off_b) {
+    __shared__ __align__(16) float dz[kBwdRows][kBwdPitch], xs[kBwdRows][2 * kGnnFeat + 4];
+    const int tid = threadIdx.x, kk = tid & 15, mg = tid >> 4;  // input kk (H0 | AGG0), outputs 4 mg ..
+    float acc[4] = {0.f, 0.f, 0.f, 0.f}, accb = 0.f;
+    for (int64_t r0 = int64_t(blockIdx.x) * kBwdRows; r0 < rows; r0 += int64_t(gridDim.x) * kBwdRows) {
+        __syncthreads();
+        for (int t = tid; t < kBwdRows * (kGnnHid / 4); t += 256) {
+            const int lr = t / (kGnnHid / 4), c = 4 * (t % (kGnnHid / 4));
+            *reinterpret_cast<float4 *>(&dz[lr][c]) =
+                r0 + lr < rows ? ld4(dZ + (r0 + lr) * kGnnHid + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        {
+            const int lr = tid >> 2, c = 4 * (tid & 1);
+            const T *src = (tid & 2) ? AGG : H;
+            *reinterpret_cast<float4 *>(&xs[lr][((tid & 2) ? kGnnFeat : 0) + c]) =
+                r0 + lr < rows ? ld4(src + (r0 + lr) * kGnnFeat + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int lr = 0; lr < kBwdRows; ++lr) {
+            float d[4];
+            lds_vec<4>(&dz[lr][4 * mg], d);
+            const float x = xs[lr][kk];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) acc[m] = fmaf(d[m], x, acc[m]);
+        }
+        if (tid < kGnnHid)
+            for (int lr = 0; lr < kBwdRows; ++lr) accb += dz[lr][tid];
+    }
+    float *p = part + int64_t(blockIdx.x) * ldp + (kk < kGnnFeat ? off_Ws : off_Wn) + kk % kGnnFeat;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) p[(4 * mg + m) * kGnnFeat] = acc[m];
+    if (tid < kGnnHid) part[int64_t(blockIdx.x) * ldp + off_b + tid] = accb;
+}
+
+// The previous layer's dZ_i = (dHp_i + sum_{j in N(i)} a_ij U_j) (.) [H_i > 0] (the pattern is
+// symmetric), one warp per row, a lane two channels; the row's columns and weights are loaded
+// by the lanes beforehand, so that four 256-byte gathers are in flight
+template <typename T>
+__global__ void __launch_bounds__(256) k_gnn_agg_t(GnnGraph g, const float *__restrict__ U,
+                                                   const float *__restrict__ dHp, const T *__restrict__ H,
+                                                   float *__restrict__ dZ) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t nwarps = int64_t(gridDim.x) * 8;
+    for (int64_t r = int64_t(blockIdx.x) * 8 + wid; r < g.rows; r += nwarps) {
+        const int b = g.row_inst[r];
+        const int64_t base = g.row_off[b];
+        const float icb = g.scal[b].y;
+        const int e0 = g.rowptr[r], deg = g.rowptr[r + 1] - e0;
+        const float2 d = ld2(dHp + r * kGnnHid + 2 * lane), h = ld2(H + r * kGnnHid + 2 * lane);
+        float s0 = 0.f, s1 = 0.f;
+        for (int c0 = 0; c0 < deg; c0 += 32) {
+            const bool in = c0 + lane < deg;
+            const int jl = in ? g.col[e0 + c0 + lane] : 0;
+            const float al = in ? g.val[e0 + c0 + lane] * icb : 0.f;
+            const int lim = min(32, deg - c0);
+            for (int t = 0; t < lim; t += 4) {
+                float2 x[4];
+                float a[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {  // lanes past the row hold column 0 and weight 0
+                    const int j = __shfl_sync(0xffffffffu, jl, t + u);
+                    a[u] = __shfl_sync(0xffffffffu, al, t + u);
+                    x[u] = t + u < lim ? ld2(U + (base + j) * kGnnHid + 2 * lane) : make_float2(0.f, 0.f);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    s0 = fmaf(a[u], x[u].x, s0);
+                    s1 = fmaf(a[u], x[u].y, s1);
+                }
+            }
+        }
+        st2(dZ + r * kGnnHid + 2 * lane, h.x > 0.f ? d.x + s0 : 0.f, h.y > 0.f ? d.y + s1 : 0.f);
     }
 }
 
-__global__ void k_gnn_sum_loss(const double *__restrict__ part, int nblk, double *__restrict__ out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double s = 0.0;
-        for (int b = 0; b < nblk; ++b) s += part[b];
-        *out = s;
+// grad[k] = sum over blocks of part[b * ldp + k], k < cnt, and the loss, in a fixed order: 32
+// parameters x 8 slices of the blocks per CTA, float pairs (an FP64 add holds a warp 64 cycles)
+__global__ void __launch_bounds__(256) k_gnn_reduce(const float *__restrict__ part, int nblk, int64_t ldp, int cnt,
+                                                    float *__restrict__ grad, const double *__restrict__ lpart,
+                                                    int nl, double *__restrict__ loss) {
+    __shared__ float hs[8][32], ls[8][32];
+    __shared__ double red[8];
+    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+    if (int(blockIdx.x) == int(gridDim.x) - 1) {  // the last CTA: the loss
+        double t = 0.0;
+        for (int b = threadIdx.x; b < nl; b += 256) t += lpart[b];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (x == 0) red[y] = t;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double s = 0.0;
+            for (int w = 0; w < 8; ++w) s += red[w];
+            *loss = s;
+        }
+        return;
+    }
+    const int k = blockIdx.x * 32 + x;
+    float h = 0.f, l = 0.f;
+    auto add = [&](float v) {
+        const float s = h + v;
+        const float bb = s - h;
+        l += (h - (s - bb)) + (v - bb);
+        h = s;
+    };
+    if (k < cnt)
+        for (int b = y; b < nblk; b += 8) add(part[int64_t(b) * ldp + k]);
+    hs[y][x] = h;
+    ls[y][x] = l;
+    __syncthreads();
+    if (y == 0 && k < cnt) {
+        for (int w = 1; w < 8; ++w) {
+            add(hs[w][x]);
+            l += ls[w][x];
+        }
+        grad[k] = h + l;
     }
 }
 
@@ -425,17 +798,43 @@ static int warp_grid(int64_t rows, int sms) {
     return int(std::max<int64_t>(1, std::min(need, cap)));
 }
 
+template <typename T, int DIN, int TR, bool HEADS, bool STORE>
+static cudaError_t layer_launch(const GnnGraph &g, const GnnLayerArgs<T> &p, int sms, cudaStream_t s) {
+    auto *fn = k_gnn_layer<T, DIN, TR, HEADS, STORE>;
+    constexpr int smem = gnn_layer_smem<DIN, TR, HEADS>();
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+    }
+    const int64_t tiles = (g.rows + TR - 1) / TR;
+    const int per = DIN == kGnnHid && TR == 128 ? 2 : 4;  // resident CTAs per multiprocessor
+    fn<<<int(std::max<int64_t>(1, std::min<int64_t>(tiles, int64_t(sms) * per))), 256, smem, s>>>(g, p);
+    return cudaGetLastError();
+}
+
+template <typename T, int TR, bool STORE>
+static cudaError_t layers_launch(const GnnGraph &g, const GnnParams &p, GnnActs<T> &a, float *rhat, float *yhat,
+                                 int sms, cudaStream_t s) {
+    for (int l = 0; l < kGnnLayers; ++l) {
+        const GnnLayerArgs<T> q{p.Ws[l], p.Wn[l], p.b[l], p.WR, p.wy, p.by, a.H[l], a.AGG[l], a.H[l + 1], rhat, yhat};
+        const cudaError_t e = l == 0              ? layer_launch<T, kGnnFeat, TR, false, STORE>(g, q, sms, s)
+                              : l + 1 < kGnnLayers ? layer_launch<T, kGnnHid, TR, false, STORE>(g, q, sms, s)
+                                                   : layer_launch<T, kGnnHid, TR, true, STORE>(g, q, sms, s);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 template <typename T>
 cudaError_t gnn_forward(const GnnGraph &g, const GnnParams &p, uint64_t feat_seed, GnnActs<T> &a, float *rhat,
-                        float *yhat, int sms, cudaStream_t s) {
-    const int grid = warp_grid(g.rows, sms);
+                        float *yhat, bool store, int sms, cudaStream_t s) {
     k_gnn_features<T><<<std::max<int64_t>(1, std::min<int64_t>((g.rows + 255) / 256, int64_t(sms) * 8)), 256, 0, s>>>(
         g, feat_seed, a.H[0]);
-    k_gnn_layer_fwd<T, kGnnFeat><<<grid, 256, 0, s>>>(g, p.Ws[0], p.Wn[0], p.b[0], a.H[0], a.AGG[0], a.H[1]);
-    for (int l = 1; l < kGnnLayers; ++l)
-        k_gnn_layer_fwd<T, kGnnHid><<<grid, 256, 0, s>>>(g, p.Ws[l], p.Wn[l], p.b[l], a.H[l], a.AGG[l], a.H[l + 1]);
-    k_gnn_heads<T><<<grid, 256, 0, s>>>(g, p.WR, p.wy, p.by, a.H[kGnnLayers], rhat, yhat);
-    return cudaGetLastError();
+    if (g.rows >= int64_t(128) * sms)
+        return store ? layers_launch<T, 128, true>(g, p, a, rhat, yhat, sms, s)
+                     : layers_launch<T, 128, false>(g, p, a, rhat, yhat, sms, s);
+    return store ? layers_launch<T, 32, true>(g, p, a, rhat, yhat, sms, s)
+                 : layers_launch<T, 32, false>(g, p, a, rhat, yhat, sms, s);
 }
 
 cudaError_t gnn_warm(const GnnGraph &g, const float *rhat, const float *yhat, const double *cbar, float mix,
@@ -447,53 +846,30 @@ cudaError_t gnn_warm(const GnnGraph &g, const float *rhat, const float *yhat, co
 }
 
 template <typename T>
-static void outer_launch(const float *A, const T *B, int64_t rows, int M, int K, int colsum, float *part, int64_t ldp,
-                         int nblk, cudaStream_t s) {
-    if (M == 64 && K == 64) k_gnn_outer<T, 64, 64><<<nblk, 256, 0, s>>>(A, B, rows, colsum, part, ldp);
-    else if (M == 64 && K == 8) k_gnn_outer<T, 64, 8><<<nblk, 256, 0, s>>>(A, B, rows, colsum, part, ldp);
-    else if (M == 32 && K == 64) k_gnn_outer<T, 32, 64><<<nblk, 256, 0, s>>>(A, B, rows, colsum, part, ldp);
-    else if (M == 1 && K == 64) k_gnn_outer<T, 1, 64><<<nblk, 256, 0, s>>>(A, B, rows, colsum, part, ldp);
-}
-
-template <typename T>
-cudaError_t gnn_loss_grad(const GnnGraph &g, const GnnParams &p, const GnnParams &grad, GnnActs<T> &a,
-                          const float *rhat, const float *yhat, const float *Rs, const double *ys, const double *cbar,
-                          double lam, double n_pattern, double n_rows, double *loss_dev, int sms, cudaStream_t s) {
-    const int grid = warp_grid(g.rows, sms);
-    k_gnn_loss<<<grid, 256, 0, s>>>(g, rhat, yhat, Rs, ys, cbar, p.WR, p.wy, float(1.0 / n_pattern),
-                                    float(lam / n_rows), a.dR, a.dY, a.dH, a.lpart);
-    k_gnn_sum_loss<<<1, 32, 0, s>>>(a.lpart, grid, loss_dev);
-    const int nblk = a.nblk;
-    const int64_t ldp = a.ldp;
-    auto reduce = [&](float *dst, int cnt) {
-        k_gnn_reduce<<<(cnt + 255) / 256, 256, 0, s>>>(a.part, nblk, ldp, cnt, dst);
-    };
-    const T *H3 = a.H[kGnnLayers];
-    // heads: dWR = dR^T H3, dwy = dY^T H3, dby = sum dY
-    outer_launch<T>(a.dR, H3, g.rows, kGnnRank, kGnnHid, 0, a.part, ldp, nblk, s);
-    reduce(grad.WR, kGnnRank * kGnnHid);
-    outer_launch<T>(a.dY, H3, g.rows, 1, kGnnHid, 1, a.part, ldp, nblk, s);
-    reduce(grad.wy, kGnnHid);
-    k_gnn_reduce<<<1, 32, 0, s>>>(a.part + kGnnHid, nblk, ldp, 1, grad.by);
-    float *dH = a.dH;
-    for (int l = kGnnLayers - 1; l >= 0; --l) {
-        const int din = l == 0 ? kGnnFeat : kGnnHid;
-        const bool prev = l > 0;
-        if (din == kGnnHid)
-            k_gnn_layer_bwd<T, kGnnHid><<<grid, 256, 0, s>>>(g, p.Ws[l], p.Wn[l], a.H[l + 1], dH, a.dZ, a.dHp, a.U, prev);
-        else
-            k_gnn_layer_bwd<T, kGnnFeat><<<grid, 256, 0, s>>>(g, p.Ws[l], p.Wn[l], a.H[l + 1], dH, a.dZ, a.dHp, a.U, prev);
-        outer_launch<T>(a.dZ, a.H[l], g.rows, kGnnHid, din, 1, a.part, ldp, nblk, s);
-        reduce(grad.Ws[l], kGnnHid * din);
-        k_gnn_reduce<<<1, 64, 0, s>>>(a.part + kGnnHid * din, nblk, ldp, kGnnHid, grad.b[l]);
-        outer_launch<T>(a.dZ, a.AGG[l], g.rows, kGnnHid, din, 0, a.part, ldp, nblk, s);
-        reduce(grad.Wn[l], kGnnHid * din);
-        if (prev) {
-            k_gnn_agg_t<kGnnHid><<<grid, 256, 0, s>>>(g, a.U, a.dHp);
-            std::swap(a.dH, a.dHp);
-            dH = a.dH;
-        }
+cudaError_t gnn_loss_grad(const GnnGraph &g, const GnnParams &p, float *grad, GnnActs<T> &a, const float *rhat,
+                          const float *yhat, const float *Rs, const double *ys, const double *cbar, double lam,
+                          double n_pattern, double n_rows, double *loss_dev, int sms, cudaStream_t s) {
+    const GnnParams at = gnn_views(grad);
+    auto off = [grad](const float *q) { return int(q - grad); };  // in the parameter vector
+    const int lgrid = int(std::max<int64_t>(1, std::min<int64_t>((g.rows + 31) / 32, int64_t(sms) * 8)));
+    k_gnn_loss<<<lgrid, 256, 0, s>>>(g, rhat, yhat, Rs, ys, cbar, float(1.0 / n_pattern), float(lam / n_rows),
+                                     reinterpret_cast<uintptr_t>(Rs) % 16 == 0, a.dR, a.dY, a.lpart);
+    const int nblk = int(std::min<int64_t>(a.nblk, (g.rows + kBwdRows - 1) / kBwdRows));
+    k_gnn_heads_bwd<T><<<nblk, 256, 0, s>>>(g.rows, a.dR, a.dY, a.H[kGnnLayers], p.WR, p.wy, a.dZ, a.part, a.ldp,
+                                            off(at.WR), off(at.wy), off(at.by));
+    cudaError_t e = cudaFuncSetAttribute(k_gnn_layer_bwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         gnn_bwd_smem<T>());
+    if (e != cudaSuccess) return e;
+    for (int l = kGnnLayers - 1; l > 0; --l) {
+        k_gnn_layer_bwd<T><<<nblk, 256, gnn_bwd_smem<T>(), s>>>(g, p.Ws[l], p.Wn[l], a.H[l], a.AGG[l], a.dZ, a.dHp,
+                                                               a.U, a.part, a.ldp, off(at.Ws[l]), off(at.Wn[l]),
+                                                               off(at.b[l]));
+        k_gnn_agg_t<T><<<warp_grid(g.rows, sms), 256, 0, s>>>(g, a.U, a.dHp, a.H[l], a.dZ);
     }
+    k_gnn_first_bwd<T><<<nblk, 256, 0, s>>>(g.rows, a.H[0], a.AGG[0], a.dZ, a.part, a.ldp, off(at.Ws[0]),
+                                            off(at.Wn[0]), off(at.b[0]));
+    const int np = gnn_num_params();
+    k_gnn_reduce<<<(np + 31) / 32 + 1, 256, 0, s>>>(a.part, nblk, a.ldp, np, grad, a.lpart, lgrid, loss_dev);
     return cudaGetLastError();
 }
 
@@ -508,8 +884,8 @@ cudaError_t gnn_adam(float *theta, const float *grad, float *m, float *v, int cn
 
 #define ALM_GNN_INST(T)                                                                                             \
     template cudaError_t gnn_forward<T>(const GnnGraph &, const GnnParams &, uint64_t, GnnActs<T> &, float *,      \
-                                        float *, int, cudaStream_t);                                                \
-    template cudaError_t gnn_loss_grad<T>(const GnnGraph &, const GnnParams &, const GnnParams &, GnnActs<T> &,    \
+                                        float *, bool, int, cudaStream_t);                                                \
+    template cudaError_t gnn_loss_grad<T>(const GnnGraph &, const GnnParams &, float *, GnnActs<T> &,              \
                                           const float *, const float *, const float *, const double *,             \
                                           const double *, double, double, double, double *, int, cudaStream_t);
 ALM_GNN_INST(float)
