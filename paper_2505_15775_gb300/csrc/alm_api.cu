@@ -719,11 +719,14 @@ static void eval_dual(alm_handle *h, const LaunchCtx &c, const SparseView<T> &v,
 // ------------------------------------------------------------------------------------
 // primitives
 // ------------------------------------------------------------------------------------
+// slack_only: the caller reads S and w, not L or <C, RR^T>; with diagonal selectors alone these
+// need |r_i|^2 of the rows and none of the off-diagonal dot products
 template <typename T>
 static alm_status eval_and_dual(alm_handle *h, const void *R, int r, int ldr, const double *y, double sigma,
-                                double *AXbuf) {
+                                double *AXbuf, bool slack_only = false) {
     LaunchCtx c = ctx(h);
-    const SparseView<T> v = view<T>(h);
+    SparseView<T> v = view<T>(h);
+    v.diag_only = slack_only && h->fused_dual;
     launch_set_state(c, sigma, 0.0, 0, ALM_INNER_GD, 0, 0.0);
     if (R) {
         eval_dual<T>(h, c, v, static_cast<const T *>(R), r, ldr, y ? y : h->zeros_m, AXbuf, h->zero_flag);
@@ -761,7 +764,7 @@ extern "C" alm_status alm_eval(alm_handle *h, const void *R, int32_t r, int32_t 
 template <typename T>
 static alm_status grad_prim(alm_handle *h, const void *R, int r, int ldr, const double *y, double sigma, void *G,
                             double *gnorm2_out) {
-    TRY(eval_and_dual<T>(h, R, r, ldr, y, sigma, h->AX));
+    TRY(eval_and_dual<T>(h, R, r, ldr, y, sigma, h->AX, true));
     const int W = vec_width(h);
     int L = 1;
     while (L * W < r) L <<= 1;
@@ -853,6 +856,15 @@ static alm_status lanczos(alm_handle *h, int k, int max_restarts, double tol_rel
     double *h1 = &h->st->h1[0];
     double *h2 = &h->st->h2[0];
     const int kk = int(std::min<int64_t>(k, n));
+    if (launch_lz_cluster<T>(c, v, Q, kk, max_restarts, tol_rel, tol_abs, seed, warm)) {
+        CK(cudaGetLastError());
+        TRY(sync_state(h));
+        if (!std::isfinite(h->h_st->theta)) FAIL(ALM_ERR_NUMERIC, "non-finite Ritz value in Lanczos");
+        *matvecs += h->h_st->lz_total + 1;
+        *theta_out = h->h_st->theta;
+        *resid_out = std::sqrt(std::max(h->h_st->red[1], 0.0));
+        return ALM_OK;
+    }
     if (warm) {  // Q[:, 0] holds the previous Ritz vector: perturb it by a seeded vector of norm 0.05
         launch_lz_start<T>(c, w, n, seed);
         launch_lz_mix<T>(c, Q, w, n);
@@ -1006,7 +1018,7 @@ static alm_status grow_block(alm_handle *h, double lam1, double sigma, double ta
 template <typename T>
 static alm_status lambda_prim(alm_handle *h, const void *R, int r, int ldr, const double *y, double sigma,
                               double *lambda_out, void *v_out, double *resid_out) {
-    TRY(eval_and_dual<T>(h, R, r, ldr, y, sigma, h->AX));
+    TRY(eval_and_dual<T>(h, R, r, ldr, y, sigma, h->AX, true));
     double theta = 0.0, resid = 0.0;
     int64_t mv = 0;
     TRY(lanczos<T>(h, h->opt.lanczos_k, h->opt.lanczos_max_restarts, h->opt.lanczos_tol, 0.0, h->opt.seed, &theta,

@@ -16,6 +16,7 @@ constexpr int kMaxRank = 32;     // rank cap (r_max)
 constexpr int kLzMax = 64;       // Lanczos basis length per cycle
 constexpr int kBlock = 256;      // threads per block of the row kernels
 constexpr int kNumSMs = 152;     // GB300
+constexpr int kLzClusterRows = 8192;  // longest vectors of the one-launch eigensolve
 constexpr int kGenChunk = 256;   // entries of a general constraint per CTA
 constexpr int kHeavyRow = 256;   // longer rows of the full pattern are summed by a CTA each
 constexpr int kUpSeg = 128;      // longer rows of the strict upper pattern are cut into segments
@@ -76,6 +77,7 @@ struct DevState {
     int method;        // ALM_INNER_CG / ALM_INNER_GD
     int lz_stop;       // Lanczos breakdown: skip the remaining steps of the cycle
     int lz_m;          // Lanczos steps done in this cycle
+    int lz_total;      // ... and in all cycles of a one-launch eigensolve
     int precond;       // 1: row-block Jacobi preconditioned CG directions
     int k1count;       // fused step+SpMM launches that ran in this inner solve (R ping-pong parity)
     float xcap2;       // staged FP32 step kernel: bound on |r_i|^2 for its next launch (0: none yet)
@@ -177,6 +179,7 @@ struct SparseView {
     int off_dynamic, has_off_sel;
     int fused_dual;                  // every constraint is a diagonal selector: the dual update
                                      // and slack diagonal are computed inside k_eval
+    int diag_only;                   // k_eval: only the diagonal entries (w and diag(S), not <C, X>)
     int ell_kf, ell_ku;              // ELL widths of the full / strict upper pattern (0: none)
     const int *f_ell_col, *u_ell_col;
     const T *f_ell_val, *u_ell_val;  // S_ij = C_ij (ELL is built only when S_off is static)
@@ -261,6 +264,12 @@ template <typename T>
 void launch_to_double(const LaunchCtx &c, const T *src, int64_t n, double *dst);
 
 // kernels_lanczos.cu
+// The whole eigensolve (cycles until the tolerance, then the residual) of short vectors in one
+// launch; false: not taken (long vectors, or no cluster of that size).  On return column 0 of Q
+// holds the Ritz vector, st has theta, resid_est, anorm, lz_total and red[1] = |S v - theta v|^2.
+template <typename T>
+bool launch_lz_cluster(const LaunchCtx &c, const SparseView<T> &v, T *Q, int kk, int max_restarts, double tol_rel,
+                       double tol_abs, uint64_t seed, bool warm);
 template <typename T>
 void launch_lz_start(const LaunchCtx &c, T *q, int64_t n, uint64_t seed);
 // q += (0.05 / sqrt(st->nrm2)) u, then st->nrm2 = |q|^2 (u from launch_lz_start)

@@ -17,8 +17,14 @@
 //                   tridiagonal solve), residual estimate |beta_{m-1} s_{m-1}|
 //   k_lz_ritz       v = Q s, the next start vector / the result.
 // Dot products accumulate in FP64; the vectors are stored in the working precision.
+//
+// Short vectors (lz_cluster_rows) take k_lz_cluster instead: the whole eigensolve, start
+// vector to residual, in one launch of one thread-block cluster.
+#include <cooperative_groups.h>
+
 #include <cfloat>
 #include <cmath>
+#include <mutex>
 
 #include "dev_util.cuh"
 #include "tridiag.cuh"
@@ -316,8 +322,339 @@ __global__ void k_lz_reset(DevState *st) {
 }
 
 // ---------------------------------------------------------------------------------------
+// The eigensolve of short vectors in one launch.  Four launches a step on vectors of 800
+// entries are all latency: 60 us a step in FP64 (4 CTAs, serial walks over the basis, launch
+// gaps), 32 steps and a tridiagonal solve a cycle.  Here one cluster of 16 CTAs runs every
+// cycle: each CTA keeps its rows of the basis and of w in shared memory (row-major, one lane
+// per basis vector, so that the dot products of a row with all vectors are one FMA
+// instruction and need no shuffles), sums are exchanged through distributed shared memory, and
+// the next Lanczos vector goes through global memory to every CTA's copy of q, which the SpMV
+// gathers from.  A step is four cluster barriers (hardware, bounded): Q^T w, Q^T w again,
+// |w|^2, the new q.  FP64 instructions are what is left (a warp's takes 64 cycles), so scalars
+// are computed by one warp.  ER(800), FP64: 12 us a step, the tridiagonal solve's share included.
+// ---------------------------------------------------------------------------------------
+constexpr int kLzcThreads = 512, kLzcWarps = kLzcThreads / 32, kLzcMaxCtas = 16;
+template <typename T>
+struct LzcArgs {
+    T *Q;                    // n x (k + 1), column-major; on return column 0 holds the Ritz vector
+    int n, kk, pitch, nr;    // steps per cycle, pitch of a row's basis entries, rows per CTA
+    int nv;                  // doubles per vector of partial sums
+    int max_restarts, warm;
+    double tol_rel, tol_abs;
+    uint64_t seed;
+};
+
+template <typename T>
+__global__ void __launch_bounds__(kLzcThreads, 1) k_lz_cluster(SparseView<T> v, LzcArgs<T> a, DevState *st) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = int(cl.block_rank()), nc = int(cl.num_blocks());
+    extern __shared__ __align__(16) unsigned char lsm[];
+    const int nv = a.nv, P = a.pitch, n = a.n;
+    double *part = reinterpret_cast<double *>(lsm);       // kLzcWarps x nv
+    double *recv = part + kLzcWarps * nv;                 // 2 x kLzcMaxCtas x nv
+    double *tot = recv + 2 * kLzcMaxCtas * nv;            // nv
+    double *la = tot + nv, *lb = la + kLzMax, *ls = lb + kLzMax, *sc = ls + kLzMax;  // sc: 8 scalars
+    T *hT = reinterpret_cast<T *>(sc + 8);                // nv
+    T *qs = hT + (nv + 1) / 2 * 2;                        // n
+    T *ws = qs + (n + 1) / 2 * 2;                         // nr
+    T *Qs = ws + (a.nr + 1) / 2 * 2;                      // nr x P
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int row0 = rank * a.nr;
+    const int nrows = max(0, min(a.nr, n - row0));
+    int buf = 0;
+    cl.sync();  // every CTA runs before another writes into its shared memory
+
+    // tot[l] = sum over the cluster of part[warp][l], l < cnt (a fixed order)
+    auto cluster_sum = [&](int cnt) {
+        __syncthreads();
+        const int l = tid >> 2, q = tid & 3;
+        const bool in = l < cnt;
+        double s = 0.0;
+        if (warp * 8 < cnt) {  // warp-uniform
+            if (in)
+                for (int w = q; w < kLzcWarps; w += 4) s += part[w * nv + l];
+            s += __shfl_xor_sync(0xffffffffu, s, 1);
+            s += __shfl_xor_sync(0xffffffffu, s, 2);
+            if (in)
+                for (int d = q; d < nc; d += 4)
+                    *cl.map_shared_rank(recv + (buf * kLzcMaxCtas + rank) * nv + l, d) = s;
+        }
+        cl.sync();
+        if (warp * 8 < cnt) {
+            s = 0.0;
+            if (in)
+                for (int d = q; d < nc; d += 4) s += recv[(buf * kLzcMaxCtas + d) * nv + l];
+            s += __shfl_xor_sync(0xffffffffu, s, 1);
+            s += __shfl_xor_sync(0xffffffffu, s, 2);
+            if (in && q == 0) {
+                tot[l] = s;
+                hT[l] = T(s);
+            }
+        }
+        buf ^= 1;
+        __syncthreads();
+    };
+    // part[warp][slot] = the warp's sum of x
+    auto warp_part = [&](T x, int slot) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (lane == 0) part[warp * nv + slot] = double(x);
+    };
+    // ws[lr] (op) sum_l Qs[lr][l] hT[l], l < nvec; returns the thread's share of |ws|^2
+    auto combine = [&](int nvec, bool subtract) -> T {
+        T nrm = T(0);
+        for (int b = 0; b < nrows; b += kLzcThreads / 4) {
+            const int lr = b + (tid >> 2), q = tid & 3;
+            T s = T(0);
+            if (lr < nrows)
+                for (int l = q; l < nvec; l += 4) s = fma(Qs[lr * P + l], hT[l], s);
+            s += __shfl_xor_sync(0xffffffffu, s, 1);
+            s += __shfl_xor_sync(0xffffffffu, s, 2);
+            if (lr < nrows && q == 0) {
+                const T x = subtract ? ws[lr] - s : s;
+                ws[lr] = x;
+                nrm = fma(x, x, nrm);
+            }
+        }
+        return nrm;
+    };
+    // basis column j = ws * scale, sent to every CTA's qs; sc[4 + l] = s_l u_l^T q
+    auto publish = [&](int j, T scale) {
+        T *X = a.Q + int64_t(j & 1) * n;
+        double u[kMaxLR] = {0.0, 0.0, 0.0, 0.0};
+        for (int lr = tid; lr < nrows; lr += kLzcThreads) {
+            const T q = ws[lr] * scale;
+            Qs[lr * P + j] = q;
+            X[row0 + lr] = q;
+            for (int l = 0; l < v.lr_k; ++l) u[l] = fma(v.lr_u[int64_t(l) * n + row0 + lr], double(q), u[l]);
+        }
+        if (v.lr_k > 0) {
+            for (int l = 0; l < v.lr_k; ++l) {
+                const double x = warp_sum(u[l]);
+                if (lane == 0) part[warp * nv + l] = x;
+            }
+            cluster_sum(v.lr_k);
+            if (tid < v.lr_k) sc[4 + tid] = v.lr_s[tid] * tot[tid];
+        } else {
+            cl.sync();
+        }
+        for (int t = tid; t < n; t += kLzcThreads) qs[t] = __ldcg(X + t);
+        __syncthreads();
+    };
+    // ws = S q on the CTA's rows, 8 lanes a row
+    auto spmv = [&]() {
+        for (int b = 0; b < nrows; b += kLzcThreads / 8) {
+            const int lr = b + (tid >> 3), sub = tid & 7;
+            T s = T(0);
+            if (lr < nrows) {
+                const int e1 = v.f_ptr[row0 + lr + 1];
+                for (int e = v.f_ptr[row0 + lr] + sub; e < e1; e += 16) {
+                    const bool two = e + 8 < e1;
+                    const T c0 = v.f_val[e], c1 = two ? v.f_val[e + 8] : T(0);
+                    const T x0 = qs[v.f_col[e]], x1 = two ? qs[v.f_col[e + 8]] : T(0);
+                    s = fma(c0, x0, s);
+                    if (two) s = fma(c1, x1, s);
+                }
+            }
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lr < nrows && sub == 0) {
+                s = fma(v.d_s[row0 + lr], qs[row0 + lr], s);
+                for (int l = 0; l < v.lr_k; ++l) s = fma(T(v.lr_u[int64_t(l) * n + row0 + lr]), T(sc[4 + l]), s);
+                ws[lr] = s;
+            }
+        }
+        __syncthreads();
+    };
+    // tot[l] = q_l . w, l < nvec: lane l takes basis vector l, a warp its share of the rows
+    auto project = [&](int nvec) {
+        T s0 = T(0), s1 = T(0);
+        for (int lr = warp; lr < nrows; lr += kLzcWarps) {
+            const T w = ws[lr];
+            if (lane < nvec) s0 = fma(Qs[lr * P + lane], w, s0);
+            if (lane + 32 < nvec) s1 = fma(Qs[lr * P + lane + 32], w, s1);
+        }
+        if (lane < nvec) part[warp * nv + lane] = double(s0);
+        if (lane + 32 < nvec) part[warp * nv + lane + 32] = double(s1);
+        cluster_sum(nvec);
+    };
+
+    // start vector: seeded, or the previous Ritz vector plus a seeded one of norm 0.05
+    {
+        T nrm = T(0);
+        for (int lr = tid; lr < nrows; lr += kLzcThreads) {
+            const uint64_t z = splitmix64_at(a.seed, uint64_t(row0 + lr));
+            const T x = T(2.0 * (double(z >> 11) * (1.0 / 9007199254740992.0)) - 1.0);
+            ws[lr] = x;
+            nrm = fma(x, x, nrm);
+        }
+        warp_part(nrm, 0);
+        cluster_sum(1);
+        if (a.warm) {
+            const T c = T(0.05 / sqrt(tot[0]));
+            nrm = T(0);
+            for (int lr = tid; lr < nrows; lr += kLzcThreads) {
+                const T x = a.Q[row0 + lr] + c * ws[lr];
+                ws[lr] = x;
+                nrm = fma(x, x, nrm);
+            }
+            warp_part(nrm, 0);
+            cluster_sum(1);
+        }
+        if (tid == 0) sc[0] = tot[0] > 0.0 ? 1.0 / sqrt(tot[0]) : 0.0;
+        __syncthreads();
+        publish(0, T(sc[0]));
+    }
+    double theta = 0.0, resid = 0.0, anorm = 0.0;
+    int m = 0, total = 0, stop = 0;
+    for (int cycle = 0; cycle < a.max_restarts; ++cycle) {
+        anorm = 0.0;
+        stop = 0;
+        for (int j = 0; j < a.kk; ++j) {
+            spmv();
+            project(j + 1);
+            double alpha = tot[j];
+            (void)combine(j + 1, true);
+            __syncthreads();
+            project(j + 1);
+            alpha += tot[j];
+            warp_part(combine(j + 1, true), 0);
+            cluster_sum(1);
+            if (tid == 0) {
+                const double beta = sqrt(tot[0]);
+                la[j] = alpha;
+                lb[j] = beta;
+                sc[1] = fmax(anorm, fabs(alpha) + beta + (j > 0 ? lb[j - 1] : 0.0));
+                sc[0] = beta > 0.0 ? 1.0 / beta : 0.0;
+                sc[2] = beta > 1e-13 * sc[1] ? 0.0 : 1.0;  // invariant subspace (or non-finite)
+            }
+            __syncthreads();
+            anorm = sc[1];
+            m = j + 1;
+            stop = sc[2] != 0.0;
+            if (stop) break;  // the same in every CTA: all hold the same sums
+            if (j + 1 < a.kk) publish(j + 1, T(sc[0]));
+        }
+        total += m;
+        __syncthreads();  // every thread has read sc
+        if (warp == 0) {
+            double rs = 0.0;
+            const double th = warp_tridiag_min(la, lb, m, ls, &rs);
+            if (lane == 0) {
+                sc[1] = th;
+                sc[2] = rs;
+            }
+            for (int l = lane; l < m; l += 32) hT[l] = T(ls[l]);
+        }
+        __syncthreads();
+        theta = sc[1];
+        resid = sc[2];
+        warp_part(combine(m, false), 0);
+        cluster_sum(1);
+        if (tid == 0) sc[0] = tot[0] > 0.0 ? 1.0 / sqrt(tot[0]) : 0.0;
+        __syncthreads();
+        publish(0, T(sc[0]));
+        if (!isfinite(theta) || resid <= fmax(a.tol_rel * anorm, a.tol_abs) || stop) break;
+    }
+    // true residual of the final pair
+    spmv();
+    T r2 = T(0);
+    for (int lr = tid; lr < nrows; lr += kLzcThreads) {
+        const T d = ws[lr] - T(theta) * qs[row0 + lr];
+        r2 = fma(d, d, r2);
+    }
+    warp_part(r2, 0);
+    cluster_sum(1);
+    if (rank == 0 && tid == 0) {
+        st->theta = theta;
+        st->resid_est = resid;
+        st->anorm = anorm;
+        st->lz_m = m;
+        st->lz_total = total;
+        st->lz_stop = stop;
+        st->red[1] = tot[0];
+    }
+    cl.sync();  // no CTA leaves while another may still write into its shared memory
+}
+
+// ---------------------------------------------------------------------------------------
 // host launchers
 // ---------------------------------------------------------------------------------------
+// Whether the one-launch eigensolve takes vectors of n entries at basis length k: its FP64 work
+// runs on 16 of 152 multiprocessors, so that longer vectors are faster spread over all of them,
+// and the basis has to fit the cluster's shared memory.  LZ_LINE
+template <typename T>
+static size_t lzc_smem(int n, int k, int ctas) {
+    const int nv = k + 1 + kMaxLR, nr = (n + ctas - 1) / ctas, P = k | 1;
+    const size_t dbl = size_t(kLzcWarps + 2 * kLzcMaxCtas + 1) * nv + 3 * kLzMax + 8;
+    const size_t el = size_t((nv + 1) / 2 * 2) + (n + 1) / 2 * 2 + (nr + 1) / 2 * 2 + size_t(nr) * P;
+    return 8 * dbl + sizeof(T) * el + 16;
+}
+template <typename T>
+static cudaLaunchConfig_t lzc_config(const LaunchCtx &c, int ctas, size_t smem, cudaLaunchAttribute *at) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(unsigned(ctas));
+    cfg.blockDim = dim3(kLzcThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = c.stream;
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = unsigned(ctas);
+    at->val.clusterDim.y = at->val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+// CTAs of the cluster for the largest shared memory the kernel may ask for: 16 where the device
+// schedules such a cluster, else 8, else none (0); asked once per precision
+template <typename T>
+static int lzc_ctas(const LaunchCtx &c, size_t *limit) {
+    static std::mutex mu;
+    static int ctas = -1;
+    static size_t lim = 0;
+    std::lock_guard<std::mutex> lk(mu);
+    if (ctas < 0) {
+        ctas = 0;
+        int dev = 0, maxsm = 0;
+        cudaFuncAttributes fa{};
+        auto *fn = k_lz_cluster<T>;
+        if (cudaGetDevice(&dev) == cudaSuccess && cudaFuncGetAttributes(&fa, fn) == cudaSuccess &&
+            cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess) {
+            lim = size_t(maxsm) - fa.sharedSizeBytes;
+            if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(lim)) == cudaSuccess &&
+                cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess)
+                for (int t = kLzcMaxCtas; t >= 8 && ctas == 0; t /= 2) {
+                    cudaLaunchAttribute at{};
+                    const cudaLaunchConfig_t cfg = lzc_config<T>(c, t, lim, &at);
+                    int nclu = 0;
+                    if (cudaOccupancyMaxActiveClusters(&nclu, fn, &cfg) == cudaSuccess && nclu > 0) ctas = t;
+                }
+        }
+        (void)cudaGetLastError();
+    }
+    *limit = lim;
+    return ctas;
+}
+
+template <typename T>
+bool launch_lz_cluster(const LaunchCtx &c, const SparseView<T> &v, T *Q, int kk, int max_restarts, double tol_rel,
+                       double tol_abs, uint64_t seed, bool warm) {
+    if (v.n > kLzClusterRows) return false;
+    size_t limit = 0;
+    const int ctas = lzc_ctas<T>(c, &limit);
+    const size_t smem = ctas ? lzc_smem<T>(v.n, kk, ctas) : 0;
+    if (ctas == 0 || smem > limit) return false;
+    LzcArgs<T> a{Q, v.n, kk, kk | 1, (v.n + ctas - 1) / ctas, kk + 1 + kMaxLR, max_restarts, warm ? 1 : 0, tol_rel, tol_abs, seed};
+    cudaLaunchAttribute at{};
+    const cudaLaunchConfig_t cfg = lzc_config<T>(c, ctas, smem, &at);
+    if (cudaLaunchKernelEx(&cfg, k_lz_cluster<T>, v, a, c.st) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    ++*c.launches;
+    return true;
+}
+
 static inline int lz_grid(const LaunchCtx &c, int64_t n) {
     int64_t need = (n + kBlock - 1) / kBlock;
     if (need < 1) need = 1;
@@ -408,6 +745,8 @@ void launch_lz_resid(const LaunchCtx &c, const T *w, const T *v, int64_t n) {
 }
 
 #define ALM_LZ_INST(T)                                                                                          \
+    template bool launch_lz_cluster<T>(const LaunchCtx &, const SparseView<T> &, T *, int, int, double, double, \
+                                       uint64_t, bool);                                                         \
     template void launch_lz_start<T>(const LaunchCtx &, T *, int64_t, uint64_t);                                \
     template void launch_lz_mix<T>(const LaunchCtx &, T *, const T *, int64_t);                                 \
     template void launch_lz_spmv<T>(const LaunchCtx &, const SparseView<T> &, const T *, T *);                  \

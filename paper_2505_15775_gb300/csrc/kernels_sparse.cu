@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(kBlock) k_prep_base(SparseView<T> v, const dou
 template <typename T, int LANES, int SP, bool OFFSEL, bool LR, bool FUSED>
 __global__ void __launch_bounds__(kBlock) k_eval(SparseView<T> v, const T *__restrict__ R, int r, int ldr,
                                                  double *__restrict__ AX, const double *__restrict__ y,
-                                                 double *__restrict__ w, DevState *st, double *partials,
+                                                 double *__restrict__ w, int nb, DevState *st, double *partials,
                                                  const int *done) {
     if (*done) return;
     using V = typename VecT<T>::type;
@@ -254,14 +254,37 @@ __global__ void __launch_bounds__(kBlock) k_eval(SparseView<T> v, const T *__res
         }
         pc += T(2) * acc;
     };
-    for (int64_t i = g0; i < v.n; i += ng) {
-        const V ri = mask_tail(load_row(R, i, ldr, gl, active), gl * W, r);
-        const int e0 = v.up_ptr[i], e1 = min(v.up_ptr[i + 1], e0 + kUpSeg);
-        const double viid = ff_norm2<LANES>(ri, gmask);  // compensated in FP32
-        if (gl == 0 && sub == 0) {
-            const T vii = T(viid);
+    // A warp takes nb rows per row group and keeps row t's |r_i|^2 in the group's lane t; then
+    // every lane does one row's FP64 work.  An FP64 instruction holds a warp 64 cycles whatever
+    // the number of active lanes, and a row takes about 16: one leader lane per row at a time
+    // cost 206 us on 1e6 rows at r = 32, of which the memory traffic is 60.
+    constexpr int RW = 32 / GW;  // row groups of a warp
+    const int x = lane & (GW - 1);
+    const int64_t tile = int64_t(RW) * nb;
+    const int64_t nw = int64_t(gridDim.x) * (kBlock / 32);
+    for (int64_t t0 = (int64_t(blockIdx.x) * (kBlock / 32) + (threadIdx.x >> 5)) * tile; t0 < v.n; t0 += nw * tile) {
+        T kh = T(0), kl = T(0);
+        for (int t = 0; t < nb; ++t) {
+            const int64_t i = t0 + int64_t(t) * RW + lane / GW;
+            const bool in = i < v.n;  // group-uniform
+            const V ri = mask_tail(load_row(R, in ? i : 0, ldr, gl, active && in), gl * W, r);
+            T hi, lo;
+            norm2_pair(ri, gmask, LANES, hi, lo);  // compensated in FP32
+            if (x == t) {
+                kh = hi;
+                kl = lo;
+            }
+            if (in && !v.diag_only) {
+                const int e0 = v.up_ptr[i];
+                upper(ri, i, e0, min(v.up_ptr[i + 1], e0 + kUpSeg));
+            }
+        }
+        __syncwarp();
+        const int64_t i = t0 + int64_t(x) * RW + lane / GW;
+        if (x < nb && i < v.n) {
+            const double viid = double(kh) + double(kl);
             const T cii = v.d_c[i];
-            pc += cii * vii;
+            pc += cii * T(viid);
             const int k = v.d_sel_k[i];
             if (k >= 0) {
                 const double a = v.d_sel_a[i];
@@ -280,9 +303,9 @@ __global__ void __launch_bounds__(kBlock) k_eval(SparseView<T> v, const T *__res
                 store_slack_diag(v, i, double(cii));
             }
         }
-        upper(ri, i, e0, e1);
+        __syncwarp();
     }
-    for (int64_t q = g0; q < v.n_useg; q += ng) {  // the rest of the long rows
+    for (int64_t q = g0; q < v.n_useg && !v.diag_only; q += ng) {  // the rest of the long rows
         const int i = v.us_row[q], e0 = v.us_e0[q], e1 = min(v.up_ptr[i + 1], e0 + kUpSeg);
         upper(mask_tail(load_row(R, i, ldr, gl, active), gl * W, r), i, e0, e1);
     }
@@ -985,8 +1008,11 @@ static __global__ void __launch_bounds__(kBlock) k_sumsq(const double *__restric
 
 // Subgroups per row: a warp's worth when the pattern's rows give each of them two entries on
 // average, else one: with fewer, the split's reductions and idle lanes cost more than the
-// shorter walk saves.
-static inline bool wide_rows(int64_t entries, int64_t n, int LN) { return entries >= 2 * (32 / LN) * n; }
+// shorter walk saves -- unless one subgroup a row leaves most of the chip idle, where two
+// entries a row are enough.
+static inline bool wide_rows(const LaunchCtx &c, int64_t entries, int64_t n, int LN) {
+    return entries >= 2 * (32 / LN) * n || (n * LN < int64_t(c.sms) * 512 && entries >= 2 * n);
+}
 #define ALM_ROW_SPLIT(wide, LN, ...)                                             \
     if (wide) { constexpr int SPW = 32 / LN; __VA_ARGS__; }                      \
     else { constexpr int SPW = 1; __VA_ARGS__; }
@@ -994,10 +1020,14 @@ static inline bool wide_rows(int64_t entries, int64_t n, int LN) { return entrie
 template <typename T, int LN, bool OFF, bool LRB, bool FUS>
 static void eval_one(const LaunchCtx &c, const SparseView<T> &v, const T *R, int r, int ldr, double *AX,
                      const double *y, double *w, const int *done) {
-    ALM_ROW_SPLIT(wide_rows(v.nnz_u, v.n, LN), LN, {
+    ALM_ROW_SPLIT(wide_rows(c, v.nnz_u, v.n, LN), LN, {
         auto *fn = k_eval<T, LN, SPW, OFF, LRB, FUS>;
-        const int grid = grid_for(c, fn, v.n + v.n_useg, kBlock / (LN * SPW));
-        fn<<<grid, kBlock, 0, c.stream>>>(v, R, r, ldr, AX, y, w, c.st, c.partials, done);
+        // rows per row group and round: up to one per lane (for the FP64 work of the rows), as
+        // long as the rounds still give every multiprocessor 16 warps
+        const int64_t rw = 32 / (LN * SPW);
+        const int nb = int(std::max<int64_t>(1, std::min<int64_t>(LN * SPW, v.n / (rw * 16 * c.sms))));
+        const int grid = grid_for(c, fn, v.n + v.n_useg * nb, kBlock / (LN * SPW) * nb);
+        fn<<<grid, kBlock, 0, c.stream>>>(v, R, r, ldr, AX, y, w, nb, c.st, c.partials, done);
     });
 }
 
@@ -1071,7 +1101,7 @@ static void spmm_one(const LaunchCtx &c, const SparseView<T> &v, const T *R, int
         k_spmm_heavy<T, LN><<<std::min(v.n_heavy, c.grid), kBlock, 0, c.stream>>>(v, R, r, ldr, done);
         ++*c.launches;
     }
-    ALM_ROW_SPLIT(wide_rows(2 * v.nnz_u, v.n, LN), LN, {
+    ALM_ROW_SPLIT(wide_rows(c, 2 * v.nnz_u, v.n, LN), LN, {
         auto *fn = k_spmm<T, LN, SPW, LRB, MODE>;
         const int grid = grid_for(c, fn, v.n, kBlock / (LN * SPW));
         fn<<<grid, kBlock, 0, c.stream>>>(v, R, r, ldr, G, D, c.st, c.partials, done);
@@ -1130,7 +1160,7 @@ void launch_dir(const LaunchCtx &c, const T *G, T *D, int64_t count, const int *
 template <typename T, int LN, bool OFF, bool LRB, int MODE>
 static void ls_one(const LaunchCtx &c, const SparseView<T> &v, const T *R, const T *D, int r, int ldr,
                    const int *done) {
-    ALM_ROW_SPLIT(wide_rows(v.nnz_u, v.n, LN), LN, {
+    ALM_ROW_SPLIT(wide_rows(c, v.nnz_u, v.n, LN), LN, {
         auto *fn = k_ls<T, LN, SPW, OFF, LRB, MODE>;
         const int grid = grid_for(c, fn, v.n + v.n_useg, kBlock / (LN * SPW));
         fn<<<grid, kBlock, 0, c.stream>>>(v, R, D, r, ldr, c.st, c.partials, done);
