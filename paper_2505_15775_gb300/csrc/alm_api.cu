@@ -87,6 +87,10 @@ struct alm_handle {
     bool fused_dual = false;
     int sms = 0;
     double *up_sel_a = nullptr, *d_sel_a = nullptr, *gd_a = nullptr, *gu_a = nullptr, *g_a = nullptr;
+    double2 *pc_rec = nullptr;   // FP64 form: per-row factors of the preconditioner
+    bool off_fast = false;       // inner slack update without FP64 for off-diagonal selectors
+    void *up_sel_a2 = nullptr, *up_sel_t = nullptr, *ob_hi = nullptr, *ob_lo = nullptr, *obb_hi = nullptr,
+         *obb_lo = nullptr;
     int n_heavy = 0;             // rows above kHeavyRow entries, and segments of long upper rows
     int64_t n_useg = 0;
     int *hv_row = nullptr, *us_row = nullptr, *us_e0 = nullptr;
@@ -288,6 +292,15 @@ static SparseView<T> view(const alm_handle *h) {
     v.g_a = h->g_a;
     v.g_a1 = h->g_a1;
     v.g_a2 = h->g_a2;
+    v.pc_rec = h->pc_rec;
+    v.up_sel_a2 = static_cast<const T *>(h->up_sel_a2);
+    v.up_slot = h->up_slot;
+    v.ob_hi = static_cast<T *>(h->ob_hi);
+    v.ob_lo = static_cast<T *>(h->ob_lo);
+    v.obb_hi = static_cast<const T *>(h->obb_hi);
+    v.obb_lo = static_cast<const T *>(h->obb_lo);
+    v.up_sel_t = static_cast<const T *>(h->up_sel_t);
+    v.off_fast = h->off_fast ? 1 : 0;
     v.n_heavy = h->n_heavy;
     v.hv_row = h->hv_row;
     v.hv_sum = static_cast<T *>(h->hv_sum);
@@ -532,6 +545,46 @@ static alm_status create_impl(alm_handle *h, const alm_problem *p, const alm_opt
         int32_t *slot = nullptr;
         TRY(upload(h, &slot, hp.up_slot));
         h->up_slot = reinterpret_cast<int2 *>(slot);
+    }
+    if (h->fused_dual && h->prec == ALM_FP64) {
+        void *p = nullptr;
+        TRY(dalloc(h, &p, sizeof(double2) * size_t(h->n)));
+        h->pc_rec = static_cast<double2 *>(p);
+    }
+    if (hp.has_off_sel) {
+        TRY(upload_T(h, &h->up_sel_a2, hp.up_sel_a, 2.0));
+        // off_fast: all constraints are selectors, and the FP32 form holds their coefficients exactly
+        bool fast = hp.m_gen == 0 && hp.lr_k == 0;
+        if (h->prec == ALM_FP32) {
+            for (double a : hp.up_sel_a) fast = fast && double(float(a)) == a;
+            for (double a : hp.d_sel_a) fast = fast && double(float(a)) == a;
+        }
+        h->off_fast = fast;
+        if (fast) {
+            auto pairs = [&](void **hi, void **lo, size_t cnt, auto value) -> alm_status {
+                std::vector<double> vh(cnt, 0.0), vl(cnt, 0.0);
+                for (size_t e = 0; e < cnt; ++e) {
+                    const double x = value(e);
+                    vh[e] = h->prec == ALM_FP32 ? double(float(x)) : x;
+                    vl[e] = x - vh[e];
+                }
+                TRY(upload_T(h, hi, vh, 1.0));
+                return upload_T(h, lo, vl, 1.0);
+            };
+            const size_t nu = size_t(h->nnz_u), nn = size_t(h->n);
+            TRY(upload_T(h, &h->up_sel_t, hp.up_sel_a, 1.0));
+            TRY(pairs(&h->obb_hi, &h->obb_lo, nu, [&](size_t e) {
+                return hp.up_sel_k[e] >= 0 ? hp.b[size_t(hp.up_sel_k[e])] : 0.0;
+            }));
+            TRY(dalloc(h, &h->ob_hi, h->esz * nu));
+            TRY(dalloc(h, &h->ob_lo, h->esz * nu));
+            // the diagonal's, as in the fused form
+            TRY(pairs(&h->b_hi, &h->b_lo, nn, [&](size_t i) {
+                return hp.d_sel_k[i] >= 0 ? hp.b[size_t(hp.d_sel_k[i])] : 0.0;
+            }));
+            TRY(dalloc(h, &h->base_hi, h->esz * nn));
+            TRY(dalloc(h, &h->base_lo, h->esz * nn));
+        }
     }
     if (hp.ell_kf == 0) {  // the CSR kernels' long rows
         std::vector<int32_t> hv;
@@ -830,7 +883,7 @@ static alm_status ensure_lanczos(alm_handle *h, int k) {
     if (h->lzw) cudaFree(h->lzw);
     h->Q = h->lzw = nullptr;
     CK(cudaMalloc(&h->Q, h->esz * size_t(h->n) * size_t(k + 1)));
-    CK(cudaMalloc(&h->lzw, h->esz * size_t(h->n)));
+    CK(cudaMalloc(&h->lzw, 2 * h->esz * size_t(h->n)));
     h->Q_cols = k + 1;
     return ALM_OK;
 }
@@ -852,7 +905,7 @@ static alm_status lanczos(alm_handle *h, int k, int max_restarts, double tol_rel
     }
     const int64_t n = h->n;
     T *Q = static_cast<T *>(h->Q);
-    T *w = static_cast<T *>(h->lzw);
+    T *w = static_cast<T *>(h->lzw), *w2 = w + n;
     double *h1 = &h->st->h1[0];
     double *h2 = &h->st->h2[0];
     const int kk = int(std::min<int64_t>(k, n));
@@ -872,16 +925,19 @@ static alm_status lanczos(alm_handle *h, int k, int max_restarts, double tol_rel
         launch_lz_start<T>(c, Q, n, seed);
     }
     launch_lz_normalize<T>(c, v, Q, Q, n, 0, 0);
-    // one restart cycle: kk steps (SpMV, CGS2 in three passes, normalisation), the tridiagonal
+    // one restart cycle: kk steps (normalisation and SpMV, CGS2 in three passes), the tridiagonal
     // eigensolve and the Ritz vector; captured once as a CUDA graph (its launches are many
     // and, at small n, short)
     auto cycle_launches = [&]() {
         launch_lz_reset(c);
+        T *wa = w, *wb = w2;  // this step's w, the next one's
         for (int j = 0; j < kk; ++j) {
-            launch_lz_spmv_reorth<T>(c, v, Q + int64_t(j) * n, Q, n, j + 1, w, h1, j);
-            launch_lz_reorth<T>(c, Q, n, j + 1, w, n, h1, h2, j, 1);
-            launch_lz_reorth<T>(c, Q, n, j + 1, w, n, h2, nullptr, j, 2);
-            launch_lz_normalize<T>(c, v, w, Q + int64_t(j + 1) * n, n, 1, j);
+            const bool fuse = v.lr_k == 0 && j > 0;  // the normalisation of the step before
+            launch_lz_spmv_reorth<T>(c, v, fuse ? wb : nullptr, Q, n, wa, h1, j);
+            launch_lz_reorth<T>(c, Q, n, j + 1, wa, n, h1, h2, j, 1);
+            launch_lz_reorth<T>(c, Q, n, j + 1, wa, n, h2, nullptr, j, 2);
+            if (v.lr_k > 0) launch_lz_normalize<T>(c, v, wa, Q + int64_t(j + 1) * n, n, 1, j);
+            else std::swap(wa, wb);
         }
         launch_lz_tridiag(c, kk);
         launch_lz_ritz<T>(c, Q, n, kk, w, n);
@@ -1105,6 +1161,7 @@ static void enqueue_inner_chunk(alm_handle *h, T *R, T *Rpart, int r, int ldr, i
         // slack diagonal only (y is fixed during the inner solve), after applying the step of
         // the previous line search
         if (h->fused_dual) launch_inner_slack<T>(c, v, R, Dc, r, ldr, done);
+        else if (h->off_fast) launch_inner_off<T>(c, v, R, r, ldr, done);
         else eval_dual<T>(h, c, v, R, r, ldr, h->y, h->AX, done);
         mark(it, 1);
         launch_spmm<T>(c, v, R, r, ldr, G, Dc, 1, done);
@@ -1201,8 +1258,9 @@ static alm_status solve_impl(alm_handle *h, void *R_user, int ldr_user, int *r_i
         T *Rpart = static_cast<T *>(h->Rb[1 - cur]);  // ping-pong partner of the fused inner step
         launch_set_state(c, sigma, tau_in * (1.0 + h->norm_C), o.max_inner, o.inner_method, o.inner_precond,
                          h->pc_floor);
-        if (h->fused_dual)
+        if (h->fused_dual || h->off_fast)
             launch_prep_base<T>(c, v, h->y, static_cast<T *>(h->base_hi), static_cast<T *>(h->base_lo));
+        if (h->off_fast) launch_prep_off<T>(c, v, h->y);
         // ---- inner solve: chunks of `chunk` steps, each step a fixed kernel sequence that
         //      turns into no-ops once the device sets `done` --------------------------------
         int iters = 0;

@@ -151,6 +151,14 @@ struct SparseView {
     const double *d_sel_a;
     const int *f_ptr, *f_col;
     T *f_val;                        // S_ij on the full pattern
+    double2 *pc_rec;                 // FP64 form: per row 1 / (2 s_i) and ka_i / (2 s_i + ka_i |r_i|^2)
+                                     // of the preconditioner (written with the slack diagonal)
+    const T *up_sel_a2;              // 2 a of the upper entries' selectors
+    const int2 *up_slot;             // full slots of each upper entry (off_dynamic)
+    T *ob_hi, *ob_lo;                // C_ij - a y_k of the upper entries, per outer iteration, and
+    const T *obb_hi, *obb_lo;        // b_k (both pairs; null unless off_fast)
+    const T *up_sel_t;               // a in the working precision
+    int off_fast;                    // the inner loop's slack update needs no FP64 (k_inner_off)
     int n_heavy;                     // rows of more than kHeavyRow entries in the full pattern:
     const int *hv_row;               // ascending
     T *hv_sum;                       // their off-diagonal sums (k_spmm_heavy)
@@ -221,6 +229,12 @@ void launch_dual_slack(const LaunchCtx &c, const SparseView<T> &v, const double 
 template <typename T>
 void launch_inner_slack(const LaunchCtx &c, const SparseView<T> &v, T *R, const T *D, int r, int ldr,
                         const int *done);
+// S on the whole pattern at R for problems whose constraints are all selectors, some of them
+// off the diagonal (SparseView::off_fast); prep: its per-outer-iteration base values from y
+template <typename T>
+void launch_inner_off(const LaunchCtx &c, const SparseView<T> &v, const T *R, int r, int ldr, const int *done);
+template <typename T>
+void launch_prep_off(const LaunchCtx &c, const SparseView<T> &v, const double *y);
 template <typename T>
 void launch_prep_base(const LaunchCtx &c, const SparseView<T> &v, const double *y, T *base_hi, T *base_lo);
 template <typename T>
@@ -281,8 +295,9 @@ template <typename T>
 void launch_lz_reorth(const LaunchCtx &c, const T *Q, int64_t ldq, int nvec, T *w, int64_t n,
                       const double *h_in, double *h_out, int j, int stage);
 template <typename T>
-void launch_lz_spmv_reorth(const LaunchCtx &c, const SparseView<T> &v, const T *q, const T *Q, int64_t ldq, int nvec,
-                           T *w, double *h_out, int j);
+// src: the step before's w, normalised into column j on the way (null: column j is there already)
+void launch_lz_spmv_reorth(const LaunchCtx &c, const SparseView<T> &v, const T *src, T *Q, int64_t ldq, T *w,
+                           double *h_out, int j);
 template <typename T>
 void launch_lz_normalize(const LaunchCtx &c, const SparseView<T> &v, const T *src, T *dst, int64_t n,
                          int mode, int j);

@@ -38,6 +38,12 @@ __device__ __forceinline__ void stv(double *p, double2 v) { *reinterpret_cast<do
 __device__ __forceinline__ float dot(float4 a, float4 b) { return a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w; }
 __device__ __forceinline__ double dot(double2 a, double2 b) { return a.x * b.x + a.y * b.y; }
 
+// acc + a . b in one FMA per component
+__device__ __forceinline__ float dot_add(float4 a, float4 b, float acc) {
+    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, acc))));
+}
+__device__ __forceinline__ double dot_add(double2 a, double2 b, double acc) { return fma(a.y, b.y, fma(a.x, b.x, acc)); }
+
 __device__ __forceinline__ float4 fma4(float s, float4 a, float4 c) {
     return make_float4(fmaf(s, a.x, c.x), fmaf(s, a.y, c.y), fmaf(s, a.z, c.z), fmaf(s, a.w, c.w));
 }
@@ -46,6 +52,9 @@ __device__ __forceinline__ double2 fma4(double s, double2 a, double2 c) {
 }
 __device__ __forceinline__ float4 scale4(float s, float4 a) { return make_float4(s * a.x, s * a.y, s * a.z, s * a.w); }
 __device__ __forceinline__ double2 scale4(double s, double2 a) { return make_double2(s * a.x, s * a.y); }
+
+__device__ __forceinline__ float4 neg4(float4 a) { return make_float4(-a.x, -a.y, -a.z, -a.w); }
+__device__ __forceinline__ double2 neg4(double2 a) { return make_double2(-a.x, -a.y); }
 
 __device__ __forceinline__ float comp(float4 v, int k) { return k == 0 ? v.x : k == 1 ? v.y : k == 2 ? v.z : v.w; }
 __device__ __forceinline__ double comp(double2 v, int k) { return k == 0 ? v.x : v.y; }

@@ -564,7 +564,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_ls_dir_pipe(SparseView<T> v, c
             }
         }
     };
-    auto dir_of = [&](V z, V d) { return fma4(beta, use_old ? d : vzero(T()), scale4(T(-1), z)); };
+    auto dir_of = [&](V z, V d) { return fma4(beta, use_old ? d : vzero(T()), neg4(z)); };
     T p2 = T(0), p11 = T(0), p12 = T(0), p22 = T(0);
     for (int s = 0; s < stages - 1; ++s) {
         fetch_cols(row0 + s * ng);
@@ -597,17 +597,29 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_ls_dir_pipe(SparseView<T> v, c
             if (!FULL) di = mask_tail(di, col, r);
             if (writer) stv(Dnew + off(i), di);
             const T rdi = dot(ri, di), ddi = dot(di, di);
-            T l2 = ds * ddi;
+            T l2 = sizeof(T) == 4 ? ds * ddi : T(0);
 #pragma unroll
             for (int k = 0; k < KU; ++k) {
                 const V zj = active ? sl[(3 + k) * NT] : vzero(T());
                 const V dj = (active && use_old) ? sl[(3 + KU + k) * NT] : vzero(T());
-                l2 += T(2) * sv[k] * dot(di, dir_of(zj, dj));
+                if (sizeof(T) == 4) l2 += T(2) * sv[k] * dot(di, dir_of(zj, dj));
+                else l2 = fma(sv[k], dot(di, dir_of(zj, dj)), l2);
             }
-            p2 += l2;
+            // FP64: every instruction counts (64 cycles a warp), one FMA each for what follows
+            if (sizeof(T) == 4) p2 += l2;
+            else p2 = fma(T(2), l2, fma(ds, ddi, p2));
             if (rec.k >= 0) {  // group-uniform
-                const T a1 = T(2) * group_sum<LANES>(rdi, gmask);
-                const T a2 = group_sum<LANES>(ddi, gmask);
+                T a1, a2;
+                if constexpr (sizeof(T) == 4 || LANES < 2) {
+                    a1 = T(2) * group_sum<LANES>(rdi, gmask);
+                    a2 = group_sum<LANES>(ddi, gmask);
+                } else {  // both sums share the butterfly: half of the lanes carry each
+                    const bool up = gl & (LANES / 2);
+                    T x = (up ? ddi : rdi) + __shfl_xor_sync(gmask, up ? rdi : ddi, LANES / 2);
+                    x = group_sum<LANES / 2>(x, gmask);
+                    a2 = __shfl_xor_sync(gmask, x, LANES / 2);  // lane 0 holds the other sum
+                    a1 = x + x;
+                }
                 if (gl == 0) {
                     const T aa = rec.a;
                     const T A1 = aa * a1, A2 = aa * a2;

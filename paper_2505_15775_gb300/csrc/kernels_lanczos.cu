@@ -3,13 +3,14 @@
 // Sec. 6: lambda_min(C - A^* y) is the dual term of the KKT error)  [hot path (d)].
 //
 // One restart cycle builds an orthonormal basis Q = [q_0 .. q_m] (column-major,
-// each q_l contiguous) of the Krylov space of S.  Step j (four launches):
-//   k_lz_reorth<SPMV>  w = S q_j (sparse part, diagonal, low-rank part of C), formed in
-//                      registers and stored, then h1 = Q^T w
+// each q_l contiguous) of the Krylov space of S.  Step j (three launches; four with a low-rank
+// part of C, whose products u_l^T q need the normalised vector):
+//   k_lz_reorth<SPMV>  q_j = w / beta_{j-1}, w = S q_j (sparse part, diagonal, low-rank part of
+//                      C), formed in registers and stored, then h1 = Q^T w
 //   k_lz_reorth x2     the rest of classical Gram-Schmidt against q_0..q_j, applied twice:
 //                      w -= Q h1; h2 = Q^T w; w -= Q h2; beta_j = ||w||
 //                      (alpha_j = h1_j + h2_j)
-//   k_lz_normalize     q_{j+1} = w / beta_j
+//   k_lz_normalize     q_{j+1} = w / beta_j (only with a low-rank part)
 // (k_lz_spmv alone serves the residual check of the final Ritz pair)
 // and at the end of a cycle
 //   k_lz_tridiag    smallest eigenpair (theta, s) of the m x m tridiagonal T in FP64
@@ -109,9 +110,20 @@ __global__ void __launch_bounds__(kBlock) k_lz_spmv(SparseView<T> v, const T *__
 // SPMV (stage 0 only): the SpMV of the step is fused in -- each thread forms its rows of
 // w = S q (as k_lz_spmv, same order of operations), stores them and keeps them in
 // registers for the dot products, so w is not read back and the step has one launch less.
+// With src the normalisation of the step before is fused in too: q = src / beta_{j-1} is formed
+// where it is read (one product, as k_lz_normalize stores it) and the rows' owner stores it as
+// basis column j; w then goes to the other buffer, as neighbours still read src.
+//
+// Bound: with 1 MB vectors and a basis in L2 the passes are latency, one warp's chain over the
+// basis vectors.  Hence kLzUnroll vectors at a time: their loads are in flight together, and
+// their warp sums share the shuffles -- in the first three rounds of the butterfly each lane
+// keeps half of its vectors and hands over the other half, so eight vectors take 9 shuffles
+// instead of 40, each sum over the same tree (the bits are those of one sum at a time).
+// 251,001 rows, FP32: alm_lambda_min over two cycles 3.85 -> 2.95 ms.
+constexpr int kLzUnroll = 8;
 template <typename T, int RPT, bool SPMV>
-__global__ void __launch_bounds__(kBlock) k_lz_reorth(SparseView<T> v, const T *__restrict__ q,
-                                                      const T *__restrict__ Q, int64_t ldq, int nvec, T *__restrict__ w,
+__global__ void __launch_bounds__(kBlock) k_lz_reorth(SparseView<T> v, const T *__restrict__ src, T *qj,
+                                                      const T *Q, int64_t ldq, int nvec, T *__restrict__ w,
                                                       int64_t n, const double *__restrict__ h_in, double *h_out, int j,
                                                       int stage, DevState *st, double *partials) {
     if (st->lz_stop) return;
@@ -119,30 +131,44 @@ __global__ void __launch_bounds__(kBlock) k_lz_reorth(SparseView<T> v, const T *
     if constexpr (SPMV)
         for (int l = 0; l < v.lr_k; ++l) qu[l] = T(v.lr_s[l] * st->qu[l]);
     constexpr int NW = kBlock / 32;
-    __shared__ T hs[kLzMax + 1];
+    constexpr int K = kLzUnroll;
+    __shared__ T hs[kLzMax + K];
     __shared__ double wsum[NW][kLzMax + 2];
-    __shared__ double shm[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int l = threadIdx.x; l < nvec; l += blockDim.x) hs[l] = stage > 0 ? T(h_in[l]) : T(0);
+    for (int l = threadIdx.x; l < kLzMax + K; l += blockDim.x) hs[l] = stage > 0 && l < nvec ? T(h_in[l]) : T(0);
     for (int t = threadIdx.x; t < NW * (kLzMax + 2); t += blockDim.x) (&wsum[0][0])[t] = 0.0;
     __syncthreads();
+    // the scale of q = scale * src (src null: q is column j, normalised already)
+    T scale = T(1);
+    if constexpr (SPMV)
+        if (src) {
+            const double beta = st->lz_beta[j - 1];
+            scale = T(beta > 0.0 ? 1.0 / beta : 0.0);
+        }
+    const T *qin = SPMV ? (src ? src : qj) : nullptr;
     const int64_t tile = int64_t(kBlock) * RPT;
     T nrm = T(0);
     for (int64_t base = int64_t(blockIdx.x) * tile; base < n; base += int64_t(gridDim.x) * tile) {
-        T x[RPT];
+        T x[RPT], own[RPT];
         int64_t idx[RPT];
 #pragma unroll
         for (int k = 0; k < RPT; ++k) {
             idx[k] = base + threadIdx.x + int64_t(k) * kBlock;
+            own[k] = T(0);
             if constexpr (SPMV) {
                 T acc = T(0);
                 if (idx[k] < n) {
                     const int64_t i = idx[k];
-                    acc = v.d_s[i] * q[i];
+                    own[k] = src ? qin[i] * scale : qin[i];
+                    acc = v.d_s[i] * own[k];
                     const int e1 = v.f_ptr[i + 1];
-                    for (int e = v.f_ptr[i]; e < e1; ++e) acc += v.f_val[e] * q[v.f_col[e]];
+                    for (int e = v.f_ptr[i]; e < e1; ++e) {
+                        const T q = qin[v.f_col[e]];
+                        acc += v.f_val[e] * (src ? q * scale : q);
+                    }
                     for (int l = 0; l < v.lr_k; ++l) acc += T(v.lr_u[int64_t(l) * v.n + i]) * qu[l];
                     w[i] = acc;
+                    if (src) qj[i] = own[k];
                 }
                 x[k] = acc;
             } else {
@@ -150,27 +176,59 @@ __global__ void __launch_bounds__(kBlock) k_lz_reorth(SparseView<T> v, const T *
             }
         }
         if (stage > 0) {
-            for (int l = 0; l < nvec; ++l) {
-                const T hl = hs[l];
-                const T *ql = Q + int64_t(l) * ldq;
+            for (int l0 = 0; l0 < nvec; l0 += K) {
+                T q[K][RPT];
 #pragma unroll
-                for (int k = 0; k < RPT; ++k)
-                    if (idx[k] < n) x[k] -= ql[idx[k]] * hl;
+                for (int u = 0; u < K; ++u)
+#pragma unroll
+                    for (int k = 0; k < RPT; ++k)
+                        q[u][k] = l0 + u < nvec && idx[k] < n ? Q[int64_t(l0 + u) * ldq + idx[k]] : T(0);
+#pragma unroll
+                for (int u = 0; u < K; ++u)
+#pragma unroll
+                    for (int k = 0; k < RPT; ++k) x[k] -= q[u][k] * hs[l0 + u];  // 0 past nvec
             }
 #pragma unroll
             for (int k = 0; k < RPT; ++k)
                 if (idx[k] < n) w[idx[k]] = x[k];
         }
         if (stage < 2) {
-            for (int l = 0; l < nvec; ++l) {
-                const T *ql = Q + int64_t(l) * ldq;
-                T a = T(0);
+            for (int l0 = 0; l0 < nvec; l0 += K) {
+                T a[K];
 #pragma unroll
-                for (int k = 0; k < RPT; ++k)
-                    if (idx[k] < n) a += ql[idx[k]] * x[k];
+                for (int u = 0; u < K; ++u) {
+                    const int l = l0 + u;
+                    a[u] = T(0);
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-                if (lane == 0) wsum[warp][l] += double(a);
+                    for (int k = 0; k < RPT; ++k) {
+                        // column j itself is this thread's own value when it was formed here
+                        T q = T(0);
+                        if (l < nvec && idx[k] < n) q = SPMV && src && l == j ? own[k] : Q[int64_t(l) * ldq + idx[k]];
+                        a[u] += q * x[k];
+                    }
+                }
+                // lane bits 4, 3, 2 pick the vector that the lane ends up with
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const bool up = lane & 16;
+                    const T give = up ? a[u] : a[u + 4], keep = up ? a[u + 4] : a[u];
+                    a[u] = keep + __shfl_xor_sync(0xffffffffu, give, 16);
+                }
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const bool up = lane & 8;
+                    const T give = up ? a[u] : a[u + 2], keep = up ? a[u + 2] : a[u];
+                    a[u] = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+                }
+                {
+                    const bool up = lane & 4;
+                    const T give = up ? a[0] : a[1], keep = up ? a[1] : a[0];
+                    a[0] = keep + __shfl_xor_sync(0xffffffffu, give, 4);
+                }
+                a[0] += __shfl_xor_sync(0xffffffffu, a[0], 2);
+                a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
+                const int l = l0 + ((lane & 16) ? 4 : 0) + ((lane & 8) ? 2 : 0) + ((lane & 4) ? 1 : 0);
+                if ((lane & 3) == 0 && l < nvec) wsum[warp][l] += double(a[0]);
             }
         }
 #pragma unroll
@@ -183,9 +241,9 @@ __global__ void __launch_bounds__(kBlock) k_lz_reorth(SparseView<T> v, const T *
     double *part = partials + size_t(blockIdx.x) * kPartStride;
     const int nslots = stage < 2 ? nvec : 0;
     for (int t = threadIdx.x; t <= nslots; t += blockDim.x) {
-        const int src = t == 0 ? kLzMax + 1 : t - 1;
+        const int from = t == 0 ? kLzMax + 1 : t - 1;
         double sacc = 0.0;
-        for (int ww = 0; ww < NW; ++ww) sacc += wsum[ww][src];
+        for (int ww = 0; ww < NW; ++ww) sacc += wsum[ww][from];
         part[t] = sacc;  // slot 0: ||w||^2, slot 1 + l: (Q^T w)_l
     }
     if (!last_block(&st->counter[CNT_LZ])) return;
@@ -194,6 +252,7 @@ __global__ void __launch_bounds__(kBlock) k_lz_reorth(SparseView<T> v, const T *
     __shared__ double tot[kLzMax + 2];
     for (int t = warp; t <= nslots; t += NW) {
         double a = 0.0;
+#pragma unroll 8
         for (int b = lane; b < int(gridDim.x); b += 32) a += __ldcg(partials + size_t(b) * kPartStride + t);
         a = warp_sum(a);
         if (lane == 0) tot[t] = a;
@@ -202,7 +261,6 @@ __global__ void __launch_bounds__(kBlock) k_lz_reorth(SparseView<T> v, const T *
     if (stage < 2)
         for (int l = threadIdx.x; l < nvec; l += blockDim.x) h_out[l] = tot[1 + l];
     const double nrm2 = tot[0];
-    (void)shm;
     if (threadIdx.x == 0) {
         st->nrm2 = nrm2;
         if (stage == 0) st->lz_alpha[j] = tot[1 + j];
@@ -696,22 +754,24 @@ void launch_lz_reorth(const LaunchCtx &c, const T *Q, int64_t ldq, int nvec, T *
                       double *h_out, int j, int stage) {
     if (lz_one_row(c, n))
         k_lz_reorth<T, 1, false><<<lz_tiles_grid(c, n, 1), kBlock, 0, c.stream>>>(
-            SparseView<T>{}, nullptr, Q, ldq, nvec, w, n, h_in, h_out, j, stage, c.st, c.partials);
+            SparseView<T>{}, nullptr, nullptr, Q, ldq, nvec, w, n, h_in, h_out, j, stage, c.st, c.partials);
     else
         k_lz_reorth<T, 4, false><<<lz_tiles_grid(c, n, 4), kBlock, 0, c.stream>>>(
-            SparseView<T>{}, nullptr, Q, ldq, nvec, w, n, h_in, h_out, j, stage, c.st, c.partials);
+            SparseView<T>{}, nullptr, nullptr, Q, ldq, nvec, w, n, h_in, h_out, j, stage, c.st, c.partials);
     ++*c.launches;
 }
 
 template <typename T>
-void launch_lz_spmv_reorth(const LaunchCtx &c, const SparseView<T> &v, const T *q, const T *Q, int64_t ldq, int nvec,
-                           T *w, double *h_out, int j) {
+void launch_lz_spmv_reorth(const LaunchCtx &c, const SparseView<T> &v, const T *src, T *Q, int64_t ldq, T *w,
+                           double *h_out, int j) {
+    T *qj = Q + int64_t(j) * ldq;
+    const int nvec = j + 1;
     if (lz_one_row(c, v.n))
         k_lz_reorth<T, 1, true><<<lz_tiles_grid(c, v.n, 1), kBlock, 0, c.stream>>>(
-            v, q, Q, ldq, nvec, w, v.n, nullptr, h_out, j, 0, c.st, c.partials);
+            v, src, qj, Q, ldq, nvec, w, v.n, nullptr, h_out, j, 0, c.st, c.partials);
     else
         k_lz_reorth<T, 4, true><<<lz_tiles_grid(c, v.n, 4), kBlock, 0, c.stream>>>(
-            v, q, Q, ldq, nvec, w, v.n, nullptr, h_out, j, 0, c.st, c.partials);
+            v, src, qj, Q, ldq, nvec, w, v.n, nullptr, h_out, j, 0, c.st, c.partials);
     ++*c.launches;
 }
 
@@ -752,8 +812,8 @@ void launch_lz_resid(const LaunchCtx &c, const T *w, const T *v, int64_t n) {
     template void launch_lz_spmv<T>(const LaunchCtx &, const SparseView<T> &, const T *, T *);                  \
     template void launch_lz_reorth<T>(const LaunchCtx &, const T *, int64_t, int, T *, int64_t, const double *, \
                                       double *, int, int);                                                      \
-    template void launch_lz_spmv_reorth<T>(const LaunchCtx &, const SparseView<T> &, const T *, const T *, int64_t, \
-                                           int, T *, double *, int);                                            \
+    template void launch_lz_spmv_reorth<T>(const LaunchCtx &, const SparseView<T> &, const T *, T *, int64_t, T *, \
+                                           double *, int);                                                      \
     template void launch_lz_normalize<T>(const LaunchCtx &, const SparseView<T> &, const T *, T *, int64_t, int, \
                                          int);                                                                  \
     template void launch_lz_ritz<T>(const LaunchCtx &, const T *, int64_t, int, T *, int64_t);                  \

@@ -178,6 +178,64 @@ __global__ void __launch_bounds__(kBlock, 4) k_inner_slack(SparseView<T> v, T *_
     }
 }
 
+// FP64 form of k_inner_slack.  FP64 instructions bound it (a warp's takes 64 cycles, and a row's
+// scalar work cost as many on a leader lane as the row's 32 elements): a warp takes LANES rows
+// per row group, its lanes' partial squares are reduced for all of them at once (LANES - 1
+// additions instead of LANES log2 LANES), which leaves lane t with row t's sum, and every lane
+// then does one row's scalars, the two divisions of the preconditioner among them (k_spmm_ell
+// reads them back).  201,601 rows, r = 32: 188 -> 60 us.
+template <int LANES, bool STEP>
+__global__ void __launch_bounds__(kBlock) k_inner_slack64(SparseView<double> v, double *__restrict__ R,
+                                                          const double *__restrict__ D, int r, int ldr,
+                                                          const DevState *st, const int *done) {
+    if (*done) return;
+    constexpr int RW = 32 / LANES;
+    const int lane = threadIdx.x & 31;
+    const int gl = lane & (LANES - 1);
+    const bool writer = gl * 2 < ldr;
+    const double sigma = st->sigma;
+    const double alpha = STEP ? st->alpha : 0.0;
+    const bool step = STEP && alpha != 0.0;
+    const int64_t nw = int64_t(gridDim.x) * (kBlock / 32);
+    for (int64_t t0 = (int64_t(blockIdx.x) * (kBlock / 32) + (threadIdx.x >> 5)) * 32; t0 < v.n; t0 += nw * 32) {
+        double p[LANES];
+#pragma unroll
+        for (int t = 0; t < LANES; ++t) {
+            const int64_t i = t0 + t * RW + lane / LANES;
+            double2 x = make_double2(0.0, 0.0);
+            if (writer && i < v.n) {
+                x = ld(R + i * ldr + gl * 2);
+                if (step) {
+                    x = fma4(alpha, ld(D + i * ldr + gl * 2), x);
+                    stv(R + i * ldr + gl * 2, x);
+                }
+            }
+            x = mask_tail(x, gl * 2, r);
+            p[t] = fma(x.x, x.x, x.y * x.y);
+        }
+#pragma unroll
+        for (int s = LANES / 2; s > 0; s >>= 1) {
+            const bool up = gl & s;
+#pragma unroll
+            for (int u = 0; u < s; ++u) {
+                const double give = up ? p[u] : p[u + s], keep = up ? p[u + s] : p[u];
+                p[u] = keep + __shfl_xor_sync(0xffffffffu, give, s);
+            }
+        }
+        const int64_t i = t0 + gl * RW + lane / LANES;
+        if (i < v.n) {
+            slack_row<double, LANES>(v, i, p[0], 0.0, sigma);
+            if (v.pc_rec) {
+                double sdi = v.d_s[i];
+                sdi = sdi > st->pc_floor ? sdi : st->pc_floor;
+                const double a = v.d_sel_k[i] >= 0 ? v.d_sel_a[i] : 0.0;
+                const double ka = 4.0 * sigma * a * a;
+                v.pc_rec[i] = make_double2(1.0 / (2.0 * sdi), ka / (2.0 * sdi + ka * p[0]));
+            }
+        }
+    }
+}
+
 // base_i = C_ii - a_i y_k(i) (rows without a diagonal selector: C_ii), as a float pair
 template <typename T>
 __global__ void __launch_bounds__(kBlock) k_prep_base(SparseView<T> v, const double *__restrict__ y,
@@ -492,6 +550,89 @@ __global__ void __launch_bounds__(kBlock) k_dual_slack(SparseView<T> v, const do
     }
 }
 
+// Per outer iteration: C_ij - a y_k of every strict upper entry as a pair
+template <typename T>
+__global__ void __launch_bounds__(kBlock) k_prep_off(SparseView<T> v, const double *__restrict__ y) {
+    for (int64_t e = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; e < v.nnz_u; e += int64_t(gridDim.x) * blockDim.x) {
+        double d = double(v.up_c[e]);
+        const int k = v.up_sel_k[e];
+        if (k >= 0) d -= v.up_sel_a[e] * y[k];
+        T hi, lo;
+        split_pair(d, hi, lo);
+        v.ob_hi[e] = hi;
+        v.ob_lo[e] = lo;
+    }
+}
+
+// Slack update of the inner loop when every constraint is a selector and some are off the
+// diagonal (matrix completion): S_ij = (C_ij - a y_k) + sigma a (2 a r_i.r_j - b_k) in float
+// pairs, as slack_row has it for the diagonal, in one pass over the upper pattern.  k_eval and
+// k_dual_slack (still what ends an inner solve) put the values through FP64 A(X) and w, some 15
+// FP64 instructions an entry at 64 cycles a warp: together 85 us on 829,000 entries
+// at rank 3 (cold caches), this 18 us; 32 inner steps there 4.49 -> 3.00 ms with it.
+template <typename T, int LANES, int SP>
+__global__ void __launch_bounds__(kBlock) k_inner_off(SparseView<T> v, const T *__restrict__ R, int r, int ldr,
+                                                      const DevState *st, const int *done) {
+    if (*done) return;
+    using V = typename VecT<T>::type;
+    constexpr int W = VecT<T>::W;
+    constexpr int GW = LANES * SP;
+    constexpr int U = 2;
+    const int lane = threadIdx.x & 31;
+    const int gl = lane & (LANES - 1), sub = (lane & (GW - 1)) / LANES;
+    const unsigned gmask = group_mask<GW>(lane);
+    const int64_t g0 = int64_t(blockIdx.x) * (kBlock / GW) + threadIdx.x / GW;
+    const int64_t ng = int64_t(gridDim.x) * (kBlock / GW);
+    const bool active = gl * W < r;
+    const T sigma = T(st->sigma);
+    auto upper = [&](V ri, int64_t i, int e0, int e1) {
+        for (int e = e0 + sub; e < e1 + sub; e += U * SP) {  // group-uniform trip count
+            int j[U];
+            V x[U];
+#pragma unroll
+            for (int k = 0; k < U; ++k) j[k] = e + k * SP < e1 ? v.up_col[e + k * SP] : int(i);
+#pragma unroll
+            for (int k = 0; k < U; ++k) x[k] = load_row(R, j[k], ldr, gl, active);
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+                T xh, xl;
+                dot_pair(ri, x[k], xh, xl);
+                pair_group_sum<LANES>(xh, xl, gmask);
+                const int q = e + k * SP;
+                if (gl == 0 && q < e1) {
+                    T s = v.ob_hi[q];
+                    const T a = v.up_sel_t[q];  // 0 without a selector
+                    const T a2 = a + a;
+                    const T ph = a2 * xh;
+                    const T pe = fma(a2, xh, -ph) + a2 * xl;
+                    const T bh = v.obb_hi[q];
+                    const T s0 = ph - bh;
+                    const T bb = s0 - ph;
+                    const T err = (ph - (s0 - bb)) + (-bh - bb);
+                    const T corr = sigma * a * (s0 + (err + pe - v.obb_lo[q]));
+                    s = s + (corr + v.ob_lo[q]);
+                    v.up_s[q] = s;
+                    const int2 sl = v.up_slot[q];
+                    v.f_val[sl.x] = s;
+                    v.f_val[sl.y] = s;
+                }
+            }
+        }
+    };
+    for (int64_t i = g0; i < v.n; i += ng) {
+        const V ri = mask_tail(load_row(R, i, ldr, gl, active), gl * W, r);
+        const int e0 = v.up_ptr[i], e1 = min(v.up_ptr[i + 1], e0 + kUpSeg);
+        T xh, xl;
+        norm2_pair(ri, gmask, LANES, xh, xl);
+        if (gl == 0 && sub == 0) slack_row<T, LANES>(v, i, xh, xl, sigma);
+        upper(ri, i, e0, e1);
+    }
+    for (int64_t q = g0; q < v.n_useg; q += ng) {
+        const int i = v.us_row[q], e0 = v.us_e0[q], e1 = min(v.up_ptr[i + 1], e0 + kUpSeg);
+        upper(mask_tail(load_row(R, i, ldr, gl, active), gl * W, r), i, e0, e1);
+    }
+}
+
 // ---------------------------------------------------------------------------------------
 // (b) G = 2 S R
 //   MODE 0: gradient only (and ||G||^2)
@@ -705,14 +846,18 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 3 : 4) k_spmm_ell(Spa
         Acc acc;
         acc.init();
         acc.add(dsi, ri);
-        acc.add_lo(dlo, ri);
+        if (sizeof(T) == 4) acc.add_lo(dlo, ri);
 #pragma unroll
         for (int k = 0; k < KF; ++k) acc.add(sc[k], gth[k]);
         const V g = mask_tail(scale4(T(2), acc.value()), gl * W, r);
-        pgg += dot(g, g);
+        pgg = dot_add(g, g, pgg);
         if (MODE == 1) {
             V z = g;
-            if (pc) {
+            if (pc && sizeof(T) == 8 && v.pc_rec) {  // the row's divisions come with its slack diagonal
+                const T rg = group_sum<LANES>(dot(ri, g), gmask);
+                const double2 q = v.pc_rec[i];
+                z = scale4(T(q.x), fma4(T(-q.y) * rg, ri, g));
+            } else if (pc) {
                 const T rg = group_sum<LANES>(dot(ri, g), gmask), rr = group_sum<LANES>(dot(ri, ri), gmask);
                 T sdi = dsi + dlo;
                 sdi = sdi > pc_floor ? sdi : pc_floor;
@@ -722,9 +867,9 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 3 : 4) k_spmm_ell(Spa
                 const T coef = ka * rg / (T(2) * sdi + ka * rr);
                 z = scale4(T(1) / (T(2) * sdi), fma4(-coef, ri, g));
             }
-            pzg += dot(z, g);
-            pgo += dot(g, gold);
-            pgd += dot(g, dold);
+            pzg = dot_add(z, g, pzg);
+            pgo = dot_add(g, gold, pgo);
+            pgd = dot_add(g, dold, pgd);
             if (writer) stv(G + i * ldr + gl * W, z);
         } else if (writer) {
             stv(G + i * ldr + gl * W, g);
@@ -791,9 +936,8 @@ __global__ void __launch_bounds__(kBlock, 3) k_ls(SparseView<T> v, const T *__re
     const int64_t ng = int64_t(gridDim.x) * (kBlock / GW);
     const bool active = gl * W < r;
     T p1 = T(0), p2 = T(0), p11 = T(0), p12 = T(0), p22 = T(0);
-    auto sel_terms = [&](int k, double a_k, T x1, T x2) {
+    auto sel_terms = [&](int k, T a, T x1, T x2) {
         if (k >= 0) {
-            const T a = T(a_k);
             const T A1 = a * x1, A2 = a * x2;
             p11 += A1 * A1;
             p12 += A1 * A2;
@@ -827,7 +971,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_ls(SparseView<T> v, const T *__re
                 if (OFFSEL) {
                     x1 = group_sum<LANES>(x1, gmask);
                     x2 = group_sum<LANES>(x2, gmask);
-                    if (gl == 0 && e + k * SP < e1) sel_terms(v.up_sel_k[e + k * SP], 2.0 * v.up_sel_a[e + k * SP], x1, x2);
+                    if (gl == 0 && e + k * SP < e1) sel_terms(v.up_sel_k[e + k * SP], v.up_sel_a2[e + k * SP], x1, x2);
                 }
             }
         }
@@ -846,7 +990,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_ls(SparseView<T> v, const T *__re
         if (ksel >= 0) {  // group-uniform
             const T a1 = group_sum<LANES>(rdi, gmask);
             const T a2 = group_sum<LANES>(ddi, gmask);
-            if (gl == 0 && sub == 0) sel_terms(ksel, v.d_sel_a[i], a1, a2);
+            if (gl == 0 && sub == 0) sel_terms(ksel, sizeof(T) == 4 ? T(v.d_sel_af[i]) : T(v.d_sel_a[i]), a1, a2);
         }
         upper(ri, di, i, e0, e1);
     }
@@ -1008,10 +1152,10 @@ static __global__ void __launch_bounds__(kBlock) k_sumsq(const double *__restric
 
 // Subgroups per row: a warp's worth when the pattern's rows give each of them two entries on
 // average, else one: with fewer, the split's reductions and idle lanes cost more than the
-// shorter walk saves -- unless one subgroup a row leaves most of the chip idle, where two
-// entries a row are enough.
+// shorter walk saves -- unless one subgroup a row leaves most of the chip idle, where half
+// an entry each is enough.
 static inline bool wide_rows(const LaunchCtx &c, int64_t entries, int64_t n, int LN) {
-    return entries >= 2 * (32 / LN) * n || (n * LN < int64_t(c.sms) * 512 && entries >= 2 * n);
+    return entries >= 2 * (32 / LN) * n || (n * LN < int64_t(c.sms) * 512 && entries >= (16 / LN) * n);
 }
 #define ALM_ROW_SPLIT(wide, LN, ...)                                             \
     if (wide) { constexpr int SPW = 32 / LN; __VA_ARGS__; }                      \
@@ -1061,6 +1205,15 @@ void launch_inner_slack(const LaunchCtx &c, const SparseView<T> &v, T *R, const 
                         const int *done) {
     constexpr int W = VecT<T>::W;
     const int L = lanes_for(r, W);
+    if constexpr (sizeof(T) == 8) {
+        ALM_DISPATCH_LANES(L, {
+            auto *fn = D ? k_inner_slack64<LN, true> : k_inner_slack64<LN, false>;
+            const int grid = grid_for(c, fn, v.n, kBlock);
+            fn<<<grid, kBlock, 0, c.stream>>>(v, R, D, r, ldr, c.st, done);
+        });
+        ++*c.launches;
+        return;
+    }
     ALM_DISPATCH_LANES(L, {
         if (D) {
             auto *fn = k_inner_slack<T, LN, true>;
@@ -1072,6 +1225,26 @@ void launch_inner_slack(const LaunchCtx &c, const SparseView<T> &v, T *R, const 
             fn<<<grid, kBlock, 0, c.stream>>>(v, R, D, r, ldr, c.st, done);
         }
     });
+    ++*c.launches;
+}
+
+template <typename T>
+void launch_inner_off(const LaunchCtx &c, const SparseView<T> &v, const T *R, int r, int ldr, const int *done) {
+    const int L = lanes_for(r, VecT<T>::W);
+    ALM_DISPATCH_LANES(L, {
+        ALM_ROW_SPLIT(wide_rows(c, v.nnz_u, v.n, LN), LN, {
+            auto *fn = k_inner_off<T, LN, SPW>;
+            const int grid = grid_for(c, fn, v.n + v.n_useg, kBlock / (LN * SPW));
+            fn<<<grid, kBlock, 0, c.stream>>>(v, R, r, ldr, c.st, done);
+        });
+    });
+    ++*c.launches;
+}
+
+template <typename T>
+void launch_prep_off(const LaunchCtx &c, const SparseView<T> &v, const double *y) {
+    auto *fn = k_prep_off<T>;
+    fn<<<grid_for(c, fn, v.nnz_u, kBlock * 4), kBlock, 0, c.stream>>>(v, y);
     ++*c.launches;
 }
 
@@ -1248,6 +1421,8 @@ void launch_sumsq(const LaunchCtx &c, const double *x, int64_t m) {
                                        double *, const int *, const int2 *);                                     \
     template void launch_inner_slack<T>(const LaunchCtx &, const SparseView<T> &, T *, const T *, int, int,      \
                                         const int *);                                                             \
+    template void launch_inner_off<T>(const LaunchCtx &, const SparseView<T> &, const T *, int, int, const int *); \
+    template void launch_prep_off<T>(const LaunchCtx &, const SparseView<T> &, const double *);                  \
     template void launch_prep_base<T>(const LaunchCtx &, const SparseView<T> &, const double *, T *, T *);      \
     template void launch_spmm<T>(const LaunchCtx &, const SparseView<T> &, const T *, int, int, T *, const T *,  \
                                  int, const int *);                                                              \
