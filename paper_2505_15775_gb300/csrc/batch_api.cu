@@ -55,7 +55,7 @@ alm_status upload(alm_batch *hb, T **dst, const std::vector<T> &src) {
 // relative to the instance's first entry.
 struct InstPattern {
     std::vector<int32_t> ptr, col;
-    std::vector<float> val;
+    std::vector<float> val, rabs;
     std::vector<double> diag;
     double norm_c = 0.0, pc_floor = 0.0;
     double dbar = 1.0, cbar = 1.0, sbar = 1.0;  // scales of the warm-start network's inputs
@@ -95,9 +95,10 @@ void build_instance(const alm_batch_problem *p, int b, InstPattern *out) {
         ent[size_t(pos[size_t(j)]++)] = {i, p->c_v[e]};
     }
     out->ptr.assign(size_t(n) + 1, 0);
+    out->rabs.assign(size_t(n), 0.f);
     double nc = 0.0, acd = 0.0, asum = 0.0, arow = 0.0;
     for (int64_t i = 0; i < n; ++i) {
-        double srow = 0.0;
+        double srow = 0.0, rabs = 0.0;
         auto first = ent.begin() + cnt[size_t(i)], last = ent.begin() + cnt[size_t(i) + 1];
         std::sort(first, last, [](const auto &x, const auto &y) { return x.first < y.first; });
         for (auto it = first; it != last;) {
@@ -109,7 +110,9 @@ void build_instance(const alm_batch_problem *p, int b, InstPattern *out) {
             nc += v * v;  // each off-diagonal pair appears twice: 2 C_ij^2 in total
             asum += std::fabs(v);
             srow += v;
+            rabs += std::fabs(v);
         }
+        out->rabs[size_t(i)] = float(rabs * (1.0 + 1e-6));
         arow += std::fabs(srow);
         out->ptr[size_t(i) + 1] = int32_t(out->col.size());
         nc += out->diag[size_t(i)] * out->diag[size_t(i)];
@@ -162,7 +165,7 @@ alm_status create_impl(alm_batch *hb, const alm_batch_problem *p) {
     if (nnz >= (int64_t(1) << 31)) BFAIL(ALM_ERR_INVALID_ARG, "the batch has more than 2^31 - 1 off-diagonal entries");
     hb->nnz = nnz;
     std::vector<int32_t> rowptr(static_cast<size_t>(hb->rows) + 1), col(static_cast<size_t>(nnz));
-    std::vector<float> val(static_cast<size_t>(nnz));
+    std::vector<float> val(static_cast<size_t>(nnz)), rabs(static_cast<size_t>(hb->rows));
     std::vector<double> cdiag(static_cast<size_t>(hb->rows)), norm_c(static_cast<size_t>(count)),
         pcf(static_cast<size_t>(count)), work(static_cast<size_t>(count)), cbar(static_cast<size_t>(count));
     std::vector<int32_t> row_inst(static_cast<size_t>(hb->rows));
@@ -176,6 +179,7 @@ alm_status create_impl(alm_batch *hb, const alm_batch_problem *p) {
         std::copy(q.col.begin(), q.col.end(), col.begin() + base);
         std::copy(q.val.begin(), q.val.end(), val.begin() + base);
         std::copy(q.diag.begin(), q.diag.end(), cdiag.begin() + r0);
+        std::copy(q.rabs.begin(), q.rabs.end(), rabs.begin() + r0);
         norm_c[size_t(b)] = q.norm_c;
         pcf[size_t(b)] = q.pc_floor;
         work[size_t(b)] = double(q.col.size()) + 8.0 * double(n);  // row passes touch n x 32 floats
@@ -195,6 +199,7 @@ alm_status create_impl(alm_batch *hb, const alm_batch_problem *p) {
     BTRY(upload(hb, &hb->col, col));
     BTRY(upload(hb, &hb->val, val));
     BTRY(upload(hb, &hb->cdiag, cdiag));
+    BTRY(upload(hb, &hb->rabs, rabs));
     BTRY(upload(hb, &hb->norm_c, norm_c));
     BTRY(upload(hb, &hb->pc_floor, pcf));
     BTRY(upload(hb, &hb->order, hb->h_order));
@@ -249,6 +254,7 @@ BatchArgs args_for(alm_batch *hb, float *R, int32_t *rank, double *y, const int3
     a.col = hb->col;
     a.val = hb->val;
     a.cdiag = hb->cdiag;
+    a.rabs = hb->rabs;
     a.norm_c = hb->norm_c;
     a.pc_floor = hb->pc_floor;
     a.order = order;
@@ -343,7 +349,7 @@ extern "C" void alm_batch_destroy(alm_batch *hb) {
     if (hb->graph) cudaGraphExecDestroy(hb->graph);
     for (cudaEvent_t e : hb->ev)
         if (e) cudaEventDestroy(e);
-    void *ptrs[] = {hb->row_off, hb->rowptr, hb->col, hb->order, hb->sample, hb->queue, hb->val, hb->cdiag,
+    void *ptrs[] = {hb->row_off, hb->rowptr, hb->col, hb->order, hb->sample, hb->queue, hb->val, hb->cdiag, hb->rabs,
                     hb->norm_c, hb->pc_floor, hb->out, hb->scr_f, hb->scr_d, hb->row_inst, hb->gnn_scal,
                     hb->cbar};
     for (void *ptr : ptrs)

@@ -27,6 +27,7 @@ struct BatchArgs {
     const int32_t *col;        // local column index
     const float *val;          // C_ij
     const double *cdiag;       // C_ii, per global row
+    const float *rabs;         // sum of |C_ij| over the row's off-diagonal entries, rounded up
     const double *norm_c;      // ||C_b||_F
     const double *pc_floor;    // preconditioner floor of S_ii, per instance
     const int32_t *order;      // queue position -> instance
@@ -84,6 +85,7 @@ struct alm_batch {
     double *cbar = nullptr;       // per instance: mean |C_ij| over the off-diagonal entries
     float *val = nullptr;
     double *cdiag = nullptr, *norm_c = nullptr, *pc_floor = nullptr;
+    float *rabs = nullptr;
     alm_instance_stats *out = nullptr;
     float *scr_f = nullptr;
     double *scr_d = nullptr;

@@ -36,6 +36,7 @@ struct BShared {
     double wpart[32 * 4];
     double sigma, tau_abs, alpha, beta, zg, zg_prev, gd, gg;
     int done, iters, status, restart, inst;
+    float rmaxw[32];  // per warp: the largest |r_i|^2 of the pending step's pass
     double lz_a[kLzMax + 1], lz_b[kLzMax + 1], lz_s[kLzMax + 1], h1[kLzMax + 1], h2[kLzMax + 1];
     float h1f[kLzMax + 1], h2f[kLzMax + 1], lz_sf[kLzMax + 1];  // FP32 copies for the row loops
     double theta, resid;
@@ -92,32 +93,37 @@ __device__ __forceinline__ float4 gather_rows(const int32_t *__restrict__ col, c
     for (; e + 4 <= e1; e += 4) {
         const int j0 = col[e], j1 = col[e + 1], j2 = col[e + 2], j3 = col[e + 3];
         const float s0 = val[e], s1 = val[e + 1], s2 = val[e + 2], s3 = val[e + 3];
-        const float4 x0 = ld(X + int64_t(j0) * kMaxRank + c0), x1 = ld(X + int64_t(j1) * kMaxRank + c0);
-        const float4 x2 = ld(X + int64_t(j2) * kMaxRank + c0), x3 = ld(X + int64_t(j3) * kMaxRank + c0);
+        const float4 x0 = ld(X + j0 * kMaxRank + c0), x1 = ld(X + j1 * kMaxRank + c0);
+        const float4 x2 = ld(X + j2 * kMaxRank + c0), x3 = ld(X + j3 * kMaxRank + c0);
         acc = fma4(s0, x0, acc);
         acc = fma4(s1, x1, acc);
         acc = fma4(s2, x2, acc);
         acc = fma4(s3, x3, acc);
     }
-    for (; e < e1; ++e) acc = fma4(val[e], ld(X + int64_t(col[e]) * kMaxRank + c0), acc);
+    for (; e < e1; ++e) acc = fma4(val[e], ld(X + col[e] * kMaxRank + c0), acc);
     return acc;
 }
 
-// the compensated form of the same sum for the gradient (its terms cancel near a solution)
-__device__ __forceinline__ void gather_rows_acc(const int32_t *__restrict__ col, const float *__restrict__ val,
-                                                int e0, int e1, const float *X, int c0, AccF &acc) {
+// The compensated form of the same sum for the gradient (its terms cancel near a solution):
+// error-free extraction against the row's power-of-two bias (ext_fma: four operations an element
+// and entry; a product error plus a two-sum took ten and kept the FP32 pipe of a multiprocessor
+// with a large instance at 85% of its peak).  The loads of the next four entries go out before
+// the arithmetic of these.
+__device__ __forceinline__ void gather_rows_ext(const int32_t *__restrict__ col, const float *__restrict__ val,
+                                                int e0, int e1, const float *X, int c0, float (&sg)[4],
+                                                float (&lo)[4]) {
     int e = e0;
     for (; e + 4 <= e1; e += 4) {
         const int j0 = col[e], j1 = col[e + 1], j2 = col[e + 2], j3 = col[e + 3];
         const float s0 = val[e], s1 = val[e + 1], s2 = val[e + 2], s3 = val[e + 3];
-        const float4 x0 = ld(X + int64_t(j0) * kMaxRank + c0), x1 = ld(X + int64_t(j1) * kMaxRank + c0);
-        const float4 x2 = ld(X + int64_t(j2) * kMaxRank + c0), x3 = ld(X + int64_t(j3) * kMaxRank + c0);
-        acc.add(s0, x0);
-        acc.add(s1, x1);
-        acc.add(s2, x2);
-        acc.add(s3, x3);
+        const float4 x0 = ld(X + j0 * kMaxRank + c0), x1 = ld(X + j1 * kMaxRank + c0);
+        const float4 x2 = ld(X + j2 * kMaxRank + c0), x3 = ld(X + j3 * kMaxRank + c0);
+        ext_term(sg, lo, s0, x0);
+        ext_term(sg, lo, s1, x1);
+        ext_term(sg, lo, s2, x2);
+        ext_term(sg, lo, s3, x3);
     }
-    for (; e < e1; ++e) acc.add(val[e], ld(X + int64_t(col[e]) * kMaxRank + c0));
+    for (; e < e1; ++e) ext_term(sg, lo, val[e], ld(X + col[e] * kMaxRank + c0));
 }
 
 // the GPU's global nanosecond timer (PTX special register %globaltimer)
@@ -149,6 +155,7 @@ __device__ void solve_instance(const BatchArgs &a, const int b, float *scr, doub
     float *R = a.R + row0 * kMaxRank;
     double *y = a.y + row0;
     const double *cd = a.cdiag + row0;
+    const float *rabs = a.rabs + row0;
     const int64_t nm = a.nmax;
     float *Z = scr;
     float *D = scr + nm * kMaxRank;
@@ -390,6 +397,7 @@ __device__ void solve_instance(const BatchArgs &a, const int b, float *scr, doub
         for (;;) {
             // (1) pending step R += alpha D, then S_ii = base_i + sigma (|r_i|^2 - 1) (float pair)
             const float alpha = float(sh.alpha);
+            float rmax = 0.f;
             for (int i = grp; i < n; i += NG) {
                 float4 rv = ld(R + int64_t(i) * kMaxRank + c0);
                 if (alpha != 0.f) {
@@ -398,6 +406,7 @@ __device__ void solve_instance(const BatchArgs &a, const int b, float *scr, doub
                 }
                 float xh, xl;
                 norm2_pair(rv, gmask, L, xh, xl);
+                rmax = fmaxf(rmax, xh + xl);
                 if (gl == 0) {
                     // res = (xh - 1) + xl with the first difference by two-sum
                     const float s0 = xh - 1.f;
@@ -412,19 +421,34 @@ __device__ void solve_instance(const BatchArgs &a, const int b, float *scr, doub
                     slo[i] = blo[i] + ((dh - (s1 - b1)) + (corr - b1));
                 }
             }
+            __syncwarp();
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
+            if (lane == 0) sh.rmaxw[warp] = rmax;
             __syncthreads();
+            rmax = lane < NW ? sh.rmaxw[lane] : 0.f;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
+            // every entry of R is below xc: G's partial sums are below (|S_ii| + sum_j |C_ij|) xc
+            // (rounded up; a non-finite row is caught by the CG sums)
+            const float xc = rmax < 1e30f ? 1.0001f * sqrtf(rmax) + 1e-18f : 1e15f;
             // (2) G = 2 S R, Z = P^{-1} G (row-block Jacobi), CG inner products
             {
                 float h[4] = {0.f, 0.f, 0.f, 0.f}, l[4] = {0.f, 0.f, 0.f, 0.f};
                 for (int i = grp; i < n; i += NG) {
                     const float4 ri = ld(R + int64_t(i) * kMaxRank + c0);
                     const float dh = shi[i], dl = slo[i];
-                    AccF acc;
-                    acc.init();
-                    acc.add(dh, ri);
-                    acc.add_lo(dl, ri);
-                    gather_rows_acc(col, val, rp[i], rp[i + 1], R, c0, acc);
-                    const float4 g = mask_tail(scale4(2.f, acc.value()), c0, r);
+                    const float gb = ext_bias((fabsf(dh) + rabs[i]) * xc);
+                    float sg4[4] = {gb, gb, gb, gb}, lo4[4] = {0.f, 0.f, 0.f, 0.f};
+                    ext_term(sg4, lo4, dh, ri);
+                    lo4[0] = fmaf(dl, ri.x, lo4[0]);
+                    lo4[1] = fmaf(dl, ri.y, lo4[1]);
+                    lo4[2] = fmaf(dl, ri.z, lo4[2]);
+                    lo4[3] = fmaf(dl, ri.w, lo4[3]);
+                    gather_rows_ext(col, val, rp[i], rp[i + 1], R, c0, sg4, lo4);
+                    const float4 g = mask_tail(make_float4(2.f * ((sg4[0] - gb) + lo4[0]), 2.f * ((sg4[1] - gb) + lo4[1]),
+                                                           2.f * ((sg4[2] - gb) + lo4[2]), 2.f * ((sg4[3] - gb) + lo4[3])),
+                                               c0, r);
                     float4 zz = g;
                     if (a.precond) {
                         const float rg = group_sum<L>(dot(ri, g), gmask), rr = group_sum<L>(dot(ri, ri), gmask);

@@ -264,35 +264,6 @@ __device__ __forceinline__ void cpa_wait(int pending) {
 // thread ([stage][slot][thread], consecutive threads on consecutive 16-byte words), then
 // one block of per-row data (ELL values and the row's record) per row group.
 
-// Error-free accumulation against a power-of-two bias (the extraction step of Rump, Ogita and
-// Oishi, "Accurate floating-point summation", SIAM J. Sci. Comput. 31, 2008).  `sg` starts at
-// bias = 1.5 * 2^e with 2^e above twice every partial sum, so sg stays in (2^e, 2^(e+1)).  One
-// FMA rounds the exact sum sg + c x; q = s - sg is then exact (Sterbenz: s and sg lie within a
-// factor of two) and c x - q, the part of c x that the rounding dropped, is exact when c x is
-// a float (c a power of two) and otherwise off by 2^-24 of a unit in the last place of sg:
-// it goes to `lo`.  Four operations per term, the product included, against eight to ten for a
-// product error plus a two-sum.  If a bound is exceeded the sum loses only the exactness of
-// that step (plain FP32 rounding).
-__device__ __forceinline__ void ext_fma(float &sg, float &lo, float c, float x) {
-    const float s = fmaf(c, x, sg);
-    const float q = s - sg;
-    lo += fmaf(c, x, -q);
-    sg = s;
-}
-// 1.5 * 2^e with 2^e the power of two just above 2 b (b >= 0), capped below the overflow range
-__device__ __forceinline__ float ext_bias(float b) {
-    unsigned u = __float_as_uint(2.f * b) & 0x7f800000u;
-    u = u < 0x7e000000u ? u : 0x7e000000u;
-    return __uint_as_float(u + 0x00c00000u);
-}
-// c x accumulated into (sg, lo) per component
-__device__ __forceinline__ void ext_term(float (&sg)[4], float (&lo)[4], float c, float4 x) {
-    ext_fma(sg[0], lo[0], c, x.x);
-    ext_fma(sg[1], lo[1], c, x.y);
-    ext_fma(sg[2], lo[2], c, x.z);
-    ext_fma(sg[3], lo[3], c, x.w);
-}
-
 template <int KF>
 constexpr int step_aux_bytes() { return KF * 4 + int(sizeof(StepRec)); }  // ELL values, record
 template <int KF>
