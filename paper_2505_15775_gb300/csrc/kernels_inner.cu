@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_spmm_ell_step(SparseView<T> v, co
     if (*done) return;
     using V = typename VecT<T>::type;
     constexpr int W = VecT<T>::W;
-    __shared__ double shm[32];
+    __shared__ double shm[64];
     const int lane = threadIdx.x & 31;
     const int gl = lane & (LANES - 1);
     const unsigned gmask = group_mask<LANES>(lane);
@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_ls_ell_dir(SparseView<T> v, const
     if (*done) return;
     using V = typename VecT<T>::type;
     constexpr int W = VecT<T>::W;
-    __shared__ double shm[32];
+    __shared__ double shm[64];
     const int lane = threadIdx.x & 31;
     const int gl = lane & (LANES - 1);
     const unsigned gmask = group_mask<LANES>(lane);
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_spmm_step_pipe(SparseView<floa
     constexpr int GPB = NT / LANES;
     static_assert(NAUX <= LANES, "a row's per-row data is copied by one lane per 16 bytes");
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ double shm[32];
+    __shared__ double shm[64];
     const int tid = threadIdx.x;
     const int lane = tid & 31;
     const int gl = lane & (LANES - 1);
@@ -481,7 +481,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_ls_dir_pipe(SparseView<T> v, c
     constexpr int GPB = NT / LANES;
     static_assert(NITEM <= LANES, "a row's per-row data is copied by one lane per 16 bytes");
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ double shm[32];
+    __shared__ double shm[64];
     const int tid = threadIdx.x;
     const int lane = tid & 31;
     const int gl = lane & (LANES - 1);

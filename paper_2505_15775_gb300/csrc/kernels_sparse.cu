@@ -424,7 +424,7 @@ __global__ void __launch_bounds__(kBlock) k_gen(SparseView<T> v, const T *__rest
     if (*done) return;
     using V = typename VecT<T>::type;
     constexpr int W = VecT<T>::W;
-    __shared__ double shm[32];
+    __shared__ double shm[64];
     __shared__ bool last;
     const int gl = threadIdx.x & (LANES - 1);
     const bool active = gl * W < r;
@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(kBlock) k_dual_slack(SparseView<T> v, const do
                                                        const int2 *__restrict__ up_slot, DevState *st,
                                                        double *partials, const int *done) {
     if (*done) return;
-    __shared__ double shm[32];
+    __shared__ double shm[64];
     const double sigma = st->sigma;
     const int64_t tid = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     const int64_t nt = int64_t(gridDim.x) * blockDim.x;
@@ -696,7 +696,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 3 : 4) k_spmm(SparseV
     constexpr int W = VecT<T>::W;
     constexpr int GW = LANES * SP;
     constexpr int U = 4;  // entries per subgroup and round
-    __shared__ double shm[32];
+    __shared__ double shm[64];
     const int lane = threadIdx.x & 31;
     const int gl = lane & (LANES - 1), sub = (lane & (GW - 1)) / LANES;
     const unsigned gmask = group_mask<GW>(lane);
@@ -810,7 +810,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 3 : 4) k_spmm_ell(Spa
     if (*done) return;
     using V = typename VecT<T>::type;
     constexpr int W = VecT<T>::W;
-    __shared__ double shm[32];
+    __shared__ double shm[64];
     const int lane = threadIdx.x & 31;
     const int gl = lane & (LANES - 1);
     const unsigned gmask = group_mask<LANES>(lane);
@@ -1032,7 +1032,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_ls_ell(SparseView<T> v, const T *
     if (*done) return;
     using V = typename VecT<T>::type;
     constexpr int W = VecT<T>::W;
-    __shared__ double shm[32];
+    __shared__ double shm[64];
     const int lane = threadIdx.x & 31;
     const int gl = lane & (LANES - 1);
     const unsigned gmask = group_mask<LANES>(lane);
@@ -1135,7 +1135,7 @@ __global__ void __launch_bounds__(kBlock) k_relayout(const T *__restrict__ src, 
 // st->red[0] = sum_k x_k^2
 static __global__ void __launch_bounds__(kBlock) k_sumsq(const double *__restrict__ x, int64_t m, DevState *st,
                                                   double *partials) {
-    __shared__ double shm[32];
+    __shared__ double shm[64];
     double acc = 0.0;
     for (int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; k < m; k += int64_t(gridDim.x) * blockDim.x)
         acc += x[k] * x[k];
