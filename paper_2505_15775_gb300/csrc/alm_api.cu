@@ -1467,7 +1467,9 @@ static alm_status solve_impl(alm_handle *h, void *R_user, int ldr_user, int *r_i
         q.lanczos_matvecs = S.lanczos_matvecs;
     }
     // ---- outputs ------------------------------------------------------------------------
-    launch_eval<T>(c, v, static_cast<T *>(h->Rb[cur]), r, ldr, h->AX, h->zero_flag);
+    // <C, RR^T> at this factor is there from the last outer iteration, if one ran
+    if (outer_first > o.max_outer)
+        launch_eval<T>(c, v, static_cast<T *>(h->Rb[cur]), r, ldr, h->AX, h->zero_flag);
     launch_relayout<T>(c, static_cast<const T *>(h->Rb[cur]), ldr, static_cast<T *>(R_user), ldr_user, r, h->n,
                        nullptr, 0.0);
     CK(cudaMemcpyAsync(y_user, h->y, sizeof(double) * size_t(h->m), cudaMemcpyDeviceToDevice, h->stream));
