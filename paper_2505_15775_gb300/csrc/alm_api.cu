@@ -112,6 +112,7 @@ struct alm_handle {
     int work_rmax = 0;
     // host mirrors
     DevState *h_st = nullptr;  // pinned
+    HostResult *h_res = nullptr, *d_res = nullptr;  // mapped pinned memory: host and device address
     cudaEvent_t prof_ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     cudaGraphExec_t graph = nullptr;
     int graph_r = -1, graph_ldr = -1, graph_cur = -1;
@@ -651,6 +652,8 @@ static alm_status create_impl(alm_handle *h, const alm_problem *p, const alm_opt
     TRY(dalloc(h, reinterpret_cast<void **>(&h->zeros_m), sizeof(double) * size_t(h->m)));
     CK(cudaMemsetAsync(h->zeros_m, 0, sizeof(double) * size_t(h->m), h->stream));
     CK(cudaMallocHost(reinterpret_cast<void **>(&h->h_st), sizeof(DevState)));
+    CK(cudaHostAlloc(reinterpret_cast<void **>(&h->h_res), sizeof(HostResult), cudaHostAllocMapped));
+    CK(cudaHostGetDevicePointer(reinterpret_cast<void **>(&h->d_res), h->h_res, 0));
     for (auto &e : h->prof_ev) CK(cudaEventCreate(&e));
     CK(cudaStreamSynchronize(h->stream));
     (void)o;
@@ -734,6 +737,7 @@ extern "C" void alm_destroy(alm_handle *h) {
     for (auto e : h->prof_ev)
         if (e) cudaEventDestroy(e);
     if (h->h_st) cudaFreeHost(h->h_st);
+    if (h->h_res) cudaFreeHost(h->h_res);
     delete h;
 }
 
@@ -778,8 +782,16 @@ template <typename T>
 static alm_status eval_and_dual(alm_handle *h, const void *R, int r, int ldr, const double *y, double sigma,
                                 double *AXbuf, bool slack_only = false) {
     LaunchCtx c = ctx(h);
-    SparseView<T> v = view<T>(h);
-    v.diag_only = slack_only && h->fused_dual;
+    if (h->fused_dual && R) {  // one kernel, which takes sigma and sets the state itself
+        SparseView<T> v = view<T>(h);
+        v.diag_only = slack_only;
+        c.sigma = sigma;
+        c.res = h->d_res;
+        eval_dual<T>(h, c, v, static_cast<const T *>(R), r, ldr, y ? y : h->zeros_m, AXbuf, h->zero_flag);
+        CK(cudaGetLastError());
+        return ALM_OK;
+    }
+    const SparseView<T> v = view<T>(h);
     launch_set_state(c, sigma, 0.0, 0, ALM_INNER_GD, 0, 0.0);
     if (R) {
         eval_dual<T>(h, c, v, static_cast<const T *>(R), r, ldr, y ? y : h->zeros_m, AXbuf, h->zero_flag);
@@ -797,10 +809,12 @@ static alm_status eval_prim(alm_handle *h, const void *R, int r, int ldr, const 
                             double *AX_out, double *CX_out) {
     TRY(eval_and_dual<T>(h, R, r, ldr, y, sigma, AX_out ? AX_out : h->AX));
     if (L_out || CX_out) {
-        TRY(sync_state(h));
-        if (L_out) *L_out = h->h_st->L;
-        if (CX_out) *CX_out = h->h_st->c0;
-        if (h->h_st->status) FAIL(alm_status(h->h_st->status), "non-finite value in the augmented Lagrangian");
+        if (h->fused_dual) CK(cudaStreamSynchronize(h->stream));  // the kernel has written *h_res
+        else TRY(sync_state(h));
+        if (L_out) *L_out = h->fused_dual ? h->h_res->L : h->h_st->L;
+        if (CX_out) *CX_out = h->fused_dual ? h->h_res->c0 : h->h_st->c0;
+        const int status = h->fused_dual ? h->h_res->status : h->h_st->status;
+        if (status) FAIL(alm_status(status), "non-finite value in the augmented Lagrangian");
     }
     return ALM_OK;
 }
@@ -822,12 +836,13 @@ static alm_status grad_prim(alm_handle *h, const void *R, int r, int ldr, const 
     int L = 1;
     while (L * W < r) L <<= 1;
     if (ldr > L * W) CK(cudaMemsetAsync(G, 0, h->esz * size_t(h->n) * size_t(ldr), h->stream));
-    launch_spmm<T>(ctx(h), view<T>(h), static_cast<const T *>(R), r, ldr, static_cast<T *>(G), nullptr, 0,
-                   h->zero_flag);
+    LaunchCtx c = ctx(h);
+    c.res = h->d_res;
+    launch_spmm<T>(c, view<T>(h), static_cast<const T *>(R), r, ldr, static_cast<T *>(G), nullptr, 0, h->zero_flag);
     CK(cudaGetLastError());
     if (gnorm2_out) {
-        TRY(sync_state(h));
-        *gnorm2_out = h->h_st->gg;
+        CK(cudaStreamSynchronize(h->stream));
+        *gnorm2_out = h->h_res->gg;
     }
     return ALM_OK;
 }
@@ -847,15 +862,17 @@ template <typename T>
 static alm_status ls_prim(alm_handle *h, const void *R, const void *D, int r, int ldr, const double *y, double sigma,
                           double *coeffs_out, double *alpha_out) {
     TRY(eval_and_dual<T>(h, R, r, ldr, y, sigma, h->AX));
-    launch_ls<T>(ctx(h), view<T>(h), static_cast<const T *>(R), static_cast<const T *>(D), r, ldr, h->w, 0,
-                 h->zero_flag);
+    LaunchCtx c = ctx(h);
+    c.res = h->d_res;
+    launch_ls<T>(c, view<T>(h), static_cast<const T *>(R), static_cast<const T *>(D), r, ldr, h->w, 0, h->zero_flag);
     CK(cudaGetLastError());
-    TRY(sync_state(h));
+    CK(cudaStreamSynchronize(h->stream));
+    const HostResult &s = *h->h_res;
     if (coeffs_out)
-        for (int k = 0; k < 5; ++k) coeffs_out[k] = h->h_st->q[k];
-    if (alpha_out) *alpha_out = h->h_st->alpha;
-    if (h->h_st->status == ALM_ERR_UNBOUNDED) FAIL(ALM_ERR_UNBOUNDED, "phi(alpha) is unbounded below on alpha >= 0");
-    if (h->h_st->status) FAIL(alm_status(h->h_st->status), "non-finite value in the line search");
+        for (int k = 0; k < 5; ++k) coeffs_out[k] = s.q[k];
+    if (alpha_out) *alpha_out = s.alpha;
+    if (s.status == ALM_ERR_UNBOUNDED) FAIL(ALM_ERR_UNBOUNDED, "phi(alpha) is unbounded below on alpha >= 0");
+    if (s.status) FAIL(alm_status(s.status), "non-finite value in the line search");
     return ALM_OK;
 }
 

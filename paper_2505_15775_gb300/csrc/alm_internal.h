@@ -209,7 +209,16 @@ struct InnerCfg {
     int threads = 128; // variant 1: threads per CTA (128 or 256)
 };
 
+// What a primitive returns to the host, in mapped pinned memory: the last block of its last
+// kernel writes it there, so that the call ends with a stream synchronisation and no copy.
+struct HostResult {
+    double L, c0, gg, q[5], alpha;
+    int status;
+};
+
 struct LaunchCtx {
+    HostResult *res = nullptr;  // device address of the handle's result (null: inside a solve)
+    double sigma = -1.0;        // penalty of a primitive (below 0: DevState::sigma)
     cudaStream_t stream;
     int sms;                  // multiprocessors of the device
     int grid;                 // upper bound on blocks (partials hold grid * kPartStride)

@@ -261,8 +261,8 @@ __global__ void __launch_bounds__(kBlock) k_prep_base(SparseView<T> v, const dou
 template <typename T, int LANES, int SP, bool OFFSEL, bool LR, bool FUSED>
 __global__ void __launch_bounds__(kBlock) k_eval(SparseView<T> v, const T *__restrict__ R, int r, int ldr,
                                                  double *__restrict__ AX, const double *__restrict__ y,
-                                                 double *__restrict__ w, int nb, DevState *st, double *partials,
-                                                 const int *done) {
+                                                 double *__restrict__ w, int nb, double sigma_arg, HostResult *res,
+                                                 DevState *st, double *partials, const int *done) {
     if (*done) return;
     using V = typename VecT<T>::type;
     constexpr int W = VecT<T>::W;
@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(kBlock) k_eval(SparseView<T> v, const T *__res
     const int64_t g0 = int64_t(blockIdx.x) * (kBlock / GW) + threadIdx.x / GW;
     const int64_t ng = int64_t(gridDim.x) * (kBlock / GW);
     const bool active = gl * W < r;
-    const double sigma = FUSED ? st->sigma : 0.0;
+    const double sigma = FUSED ? (sigma_arg >= 0.0 ? sigma_arg : st->sigma) : 0.0;
     T pc = T(0);
     double pyres = 0.0, pres2 = 0.0, pbw = 0.0;
 
@@ -398,8 +398,18 @@ __global__ void __launch_bounds__(kBlock) k_eval(SparseView<T> v, const T *__res
             st->yres = tot[1];
             st->res2 = tot[2];
             st->bw = tot[3];
-            st->L = c - tot[1] + 0.5 * sigma * tot[2];
-            if (!isfinite(st->L)) {
+            const double L = c - tot[1] + 0.5 * sigma * tot[2];
+            st->L = L;
+            if (sigma_arg >= 0.0) {  // a primitive: the state that k_set_state prepares for a solve
+                st->sigma = sigma;
+                st->status = isfinite(L) ? 0 : ALM_ERR_NUMERIC;
+                if (res) {
+                    res->L = L;
+                    res->c0 = c;
+                    res->status = st->status;
+                    __threadfence_system();
+                }
+            } else if (!isfinite(L)) {
                 st->status = ALM_ERR_NUMERIC;
                 st->done = 1;
             }
@@ -688,8 +698,8 @@ __global__ void __launch_bounds__(kBlock) k_spmm_heavy(SparseView<T> v, const T 
 
 template <typename T, int LANES, int SP, bool LR, int MODE>
 __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 3 : 4) k_spmm(SparseView<T> v, const T *__restrict__ R,
-                                                                      int r, int ldr, T *G, const T *D, DevState *st,
-                                                                      double *partials, const int *done) {
+                                                                      int r, int ldr, T *G, const T *D, HostResult *res,
+                                                                      DevState *st, double *partials, const int *done) {
     if (*done) return;
     using V = typename VecT<T>::type;
     using Acc = typename AccOf<T>::type;
@@ -797,16 +807,23 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 3 : 4) k_spmm(SparseV
     double tot[4];
     sum_partials_n<4>(partials, tot, shm);
     if (threadIdx.x == 0) {
-        if (MODE == 1) spmm_finish(st, tot[0], tot[1], tot[2], tot[3]);
-        else st->gg = tot[0];
+        if (MODE == 1) {
+            spmm_finish(st, tot[0], tot[1], tot[2], tot[3]);
+        } else {
+            st->gg = tot[0];
+            if (res) {
+                res->gg = tot[0];
+                __threadfence_system();
+            }
+        }
     }
 }
 
 
 template <typename T, int LANES, int KF, int MODE>
 __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 3 : 4) k_spmm_ell(SparseView<T> v, const T *__restrict__ R, int r, int ldr,
-                                                     T *G, const T *D, DevState *st, double *partials,
-                                                     const int *done) {
+                                                     T *G, const T *D, HostResult *res, DevState *st,
+                                                     double *partials, const int *done) {
     if (*done) return;
     using V = typename VecT<T>::type;
     constexpr int W = VecT<T>::W;
@@ -887,8 +904,15 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 3 : 4) k_spmm_ell(Spa
     double tot[4];
     sum_partials_n<4>(partials, tot, shm);
     if (threadIdx.x == 0) {
-        if (MODE == 1) spmm_finish(st, tot[0], tot[1], tot[2], tot[3]);
-        else st->gg = tot[0];
+        if (MODE == 1) {
+            spmm_finish(st, tot[0], tot[1], tot[2], tot[3]);
+        } else {
+            st->gg = tot[0];
+            if (res) {
+                res->gg = tot[0];
+                __threadfence_system();
+            }
+        }
     }
 }
 
@@ -922,7 +946,8 @@ __global__ void __launch_bounds__(kBlock) k_dir(const T *__restrict__ G, T *__re
 // ---------------------------------------------------------------------------------------
 template <typename T, int LANES, int SP, bool OFFSEL, bool LR, int MODE>
 __global__ void __launch_bounds__(kBlock, 3) k_ls(SparseView<T> v, const T *__restrict__ R, const T *__restrict__ D,
-                                               int r, int ldr, DevState *st, double *partials, const int *done) {
+                                               int r, int ldr, HostResult *res, DevState *st, double *partials,
+                                               const int *done) {
     if (*done) return;
     using V = typename VecT<T>::type;
     constexpr int W = VecT<T>::W;
@@ -1019,7 +1044,10 @@ __global__ void __launch_bounds__(kBlock, 3) k_ls(SparseView<T> v, const T *__re
         tot[3] += block_sum(g12, shm);
         tot[4] += block_sum(g22, shm);
     }
-    if (threadIdx.x == 0) ls_finish<T, MODE, LR>(v, st, r, tot);
+    if (threadIdx.x == 0) {
+        ls_finish<T, MODE, LR>(v, st, r, tot);
+        if (res) ls_result(res, st);
+    }
 }
 
 // ELL form of the line-search SDDMM (static S_off: no off-diagonal selector constraints,
@@ -1027,8 +1055,8 @@ __global__ void __launch_bounds__(kBlock, 3) k_ls(SparseView<T> v, const T *__re
 // ahead of the current row's gathers of R and D
 template <typename T, int LANES, int KU, int MODE>
 __global__ void __launch_bounds__(kBlock, 4) k_ls_ell(SparseView<T> v, const T *__restrict__ R,
-                                                   const T *__restrict__ D, int r, int ldr, DevState *st,
-                                                   double *partials, const int *done) {
+                                                   const T *__restrict__ D, int r, int ldr, HostResult *res,
+                                                   DevState *st, double *partials, const int *done) {
     if (*done) return;
     using V = typename VecT<T>::type;
     constexpr int W = VecT<T>::W;
@@ -1094,7 +1122,10 @@ __global__ void __launch_bounds__(kBlock, 4) k_ls_ell(SparseView<T> v, const T *
     if (!last_block(&st->counter[CNT_LS])) return;
     double tot[5];
     sum_partials_n<5>(partials, tot, shm);
-    if (threadIdx.x == 0) ls_finish<T, MODE, false>(v, st, r, tot);
+    if (threadIdx.x == 0) {
+        ls_finish<T, MODE, false>(v, st, r, tot);
+        if (res) ls_result(res, st);
+    }
 }
 
 
@@ -1171,7 +1202,7 @@ static void eval_one(const LaunchCtx &c, const SparseView<T> &v, const T *R, int
         const int64_t rw = 32 / (LN * SPW);
         const int nb = int(std::max<int64_t>(1, std::min<int64_t>(LN * SPW, v.n / (rw * 16 * c.sms))));
         const int grid = grid_for(c, fn, v.n + v.n_useg * nb, kBlock / (LN * SPW) * nb);
-        fn<<<grid, kBlock, 0, c.stream>>>(v, R, r, ldr, AX, y, w, nb, c.st, c.partials, done);
+        fn<<<grid, kBlock, 0, c.stream>>>(v, R, r, ldr, AX, y, w, nb, c.sigma, c.res, c.st, c.partials, done);
     });
 }
 
@@ -1277,7 +1308,7 @@ static void spmm_one(const LaunchCtx &c, const SparseView<T> &v, const T *R, int
     ALM_ROW_SPLIT(wide_rows(c, 2 * v.nnz_u, v.n, LN), LN, {
         auto *fn = k_spmm<T, LN, SPW, LRB, MODE>;
         const int grid = grid_for(c, fn, v.n, kBlock / (LN * SPW));
-        fn<<<grid, kBlock, 0, c.stream>>>(v, R, r, ldr, G, D, c.st, c.partials, done);
+        fn<<<grid, kBlock, 0, c.stream>>>(v, R, r, ldr, G, D, c.res, c.st, c.partials, done);
     });
 }
 
@@ -1286,10 +1317,12 @@ static void spmm_ell_one(const LaunchCtx &c, const SparseView<T> &v, const T *R,
                          int mode, const int *done) {
     if (mode == 1) {
         auto *fn = k_spmm_ell<T, LN, KF, 1>;
-        fn<<<grid_for(c, fn, v.n, kBlock / LN), kBlock, 0, c.stream>>>(v, R, r, ldr, G, D, c.st, c.partials, done);
+        fn<<<grid_for(c, fn, v.n, kBlock / LN), kBlock, 0, c.stream>>>(v, R, r, ldr, G, D, c.res, c.st, c.partials,
+                                                                             done);
     } else {
         auto *fn = k_spmm_ell<T, LN, KF, 0>;
-        fn<<<grid_for(c, fn, v.n, kBlock / LN), kBlock, 0, c.stream>>>(v, R, r, ldr, G, D, c.st, c.partials, done);
+        fn<<<grid_for(c, fn, v.n, kBlock / LN), kBlock, 0, c.stream>>>(v, R, r, ldr, G, D, c.res, c.st, c.partials,
+                                                                             done);
     }
 }
 
@@ -1336,7 +1369,7 @@ static void ls_one(const LaunchCtx &c, const SparseView<T> &v, const T *R, const
     ALM_ROW_SPLIT(wide_rows(c, v.nnz_u, v.n, LN), LN, {
         auto *fn = k_ls<T, LN, SPW, OFF, LRB, MODE>;
         const int grid = grid_for(c, fn, v.n + v.n_useg, kBlock / (LN * SPW));
-        fn<<<grid, kBlock, 0, c.stream>>>(v, R, D, r, ldr, c.st, c.partials, done);
+        fn<<<grid, kBlock, 0, c.stream>>>(v, R, D, r, ldr, c.res, c.st, c.partials, done);
     });
 }
 
@@ -1345,10 +1378,10 @@ static void ls_ell_one(const LaunchCtx &c, const SparseView<T> &v, const T *R, c
                        const int *done) {
     if (mode == 1) {
         auto *fn = k_ls_ell<T, LN, KU, 1>;
-        fn<<<grid_for(c, fn, v.n, kBlock / LN), kBlock, 0, c.stream>>>(v, R, D, r, ldr, c.st, c.partials, done);
+        fn<<<grid_for(c, fn, v.n, kBlock / LN), kBlock, 0, c.stream>>>(v, R, D, r, ldr, c.res, c.st, c.partials, done);
     } else {
         auto *fn = k_ls_ell<T, LN, KU, 0>;
-        fn<<<grid_for(c, fn, v.n, kBlock / LN), kBlock, 0, c.stream>>>(v, R, D, r, ldr, c.st, c.partials, done);
+        fn<<<grid_for(c, fn, v.n, kBlock / LN), kBlock, 0, c.stream>>>(v, R, D, r, ldr, c.res, c.st, c.partials, done);
     }
 }
 

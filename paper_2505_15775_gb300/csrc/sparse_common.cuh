@@ -227,6 +227,14 @@ __device__ __forceinline__ void ls_finish(const SparseView<T> &v, DevState *st, 
         }
     }
 
+// the line search's scalars to the host
+__device__ __forceinline__ void ls_result(HostResult *res, const DevState *st) {
+    for (int k = 0; k < 5; ++k) res->q[k] = st->q[k];
+    res->alpha = st->alpha;
+    res->status = st->status;
+    __threadfence_system();
+}
+
 // blocks of kBlock threads per SM that the kernel can keep resident (cached per kernel)
 static int resident_blocks(const void *fn) {
     static std::mutex mu;
