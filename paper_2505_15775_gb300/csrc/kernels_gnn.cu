@@ -117,9 +117,10 @@ __device__ __forceinline__ void lds_vec(const float *p, float (&x)[N]) {
 // One layer over tiles of TR rows: agg_i, h'_i = relu(Ws h_i + Wn agg_i + b), and with HEADS
 // (the last layer) rhat_i = W_R h'_i, yhat_i = w_y . h'_i + b_y from the tile in shared memory.
 // STORE: keep agg and, in the last layer, h' for the backward pass (inference needs neither).
-//   gather   64 channels: a warp takes four rows at once, a lane two channels of each; the rows'
-//            columns and weights are loaded by the lanes beforehand, so that the gathers of up
-//            to eight neighbour rows (two per row) are in flight.  8 channels: two threads a row.
+//   gather   64 channels: a warp loads the places of all its rows and their first 32 entries at
+//            once (a lane per row, then a lane per entry: the dependent loads are paid once a
+//            tile), then takes four rows at a time, a lane two channels of each, with the gathers
+//            of sixteen neighbour rows in flight.  8 channels: two threads a row.
 //   product  thread (rg, og) holds TR / 16 rows x 4 outputs; inputs lie transposed in shared
 //            memory ([channel][row]), so an input costs TR / 16 x 4 FMAs per 16-byte load.
 //            Per output the FMAs run over k in order, Wn's before Ws's, from the bias on.
@@ -127,7 +128,7 @@ __device__ __forceinline__ void lds_vec(const float *p, float (&x)[N]) {
 // such tile per multiprocessor take tiles of 32, to use more of them.
 // Bound: the FP32 pipe (8192 FMAs a row: 0.21 ms per million rows) and the gathers.  One warp
 // per row with both operands of every FMA from shared memory took 1.25 ms a layer on 1e6 torus
-// rows and 0.37 ms for the heads: alm_gnn_warm_start 3.60 -> 1.56 ms.
+// rows and 0.37 ms for the heads: alm_gnn_warm_start 3.60 -> 1.50 ms.
 template <int DIN, int TR, bool HEADS>
 constexpr int gnn_layer_smem() {
     return 4 * (DIN * (2 * kGnnHid + 4) + kGnnHid + 2 * DIN * (TR + 4) +
@@ -158,63 +159,76 @@ __global__ void __launch_bounds__(256, 2) k_gnn_layer(GnnGraph g, GnnLayerArgs<T
     const int og = tid & 15, rg = tid >> 4;
     for (int64_t r0 = int64_t(blockIdx.x) * TR; r0 < g.rows; r0 += int64_t(gridDim.x) * TR) {
         if constexpr (DIN == kGnnHid) {
-            for (int q4 = 0; q4 < TR / 8; q4 += 4) {  // four rows at once
-                const int lr = wid * (TR / 8) + q4;
-                int64_t base = 0;
-                int e0 = 0, e1 = 0;
-                float icb = 0.f;
-                if (lane < 4 && r0 + lr + lane < g.rows) {
-                    const int64_t r = r0 + lr + lane;
-                    const int b = g.row_inst[r];
-                    base = g.row_off[b];
-                    icb = g.scal[b].y;
-                    e0 = g.rowptr[r];
-                    e1 = g.rowptr[r + 1];
-                }
+            constexpr int RW = TR / 8;  // rows of a warp: their places and first 32 entries in one go
+            int64_t base = 0;
+            int e0 = 0, dg = 0;
+            float icb = 0.f;
+            if (lane < RW && r0 + wid * RW + lane < g.rows) {
+                const int64_t r = r0 + wid * RW + lane;
+                const int b = g.row_inst[r];
+                base = g.row_off[b];
+                icb = g.scal[b].y;
+                e0 = g.rowptr[r];
+                dg = g.rowptr[r + 1] - e0;
+            }
+            int jc[RW];
+            float ac[RW];
+#pragma unroll
+            for (int q = 0; q < RW; ++q) {
+                const int eq = __shfl_sync(0xffffffffu, e0, q), dq = __shfl_sync(0xffffffffu, dg, q);
+                const float iq = __shfl_sync(0xffffffffu, icb, q);
+                jc[q] = lane < dq ? g.col[eq + lane] : 0;
+                ac[q] = lane < dq ? g.val[eq + lane] * iq : 0.f;
+            }
+#pragma unroll
+            for (int q4 = 0; q4 < RW; q4 += 4) {  // four rows at once
+                const int lr = wid * RW + q4;
                 float a0[4] = {0.f, 0.f, 0.f, 0.f}, a1[4] = {0.f, 0.f, 0.f, 0.f};
                 int deg[4];
+                const T *hb[4];
                 int most = 0;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    deg[q] = __shfl_sync(0xffffffffu, e1 - e0, q);
-                    most = max(most, deg[q]);
-                }
                 float2 own[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
+                    deg[q] = __shfl_sync(0xffffffffu, dg, q4 + q);
+                    most = max(most, deg[q]);
+                    hb[q] = p.H + __shfl_sync(0xffffffffu, base, q4 + q) * DIN + 2 * lane;
                     const int64_t r = r0 + lr + q;
                     own[q] = r < g.rows ? ld2(p.H + r * DIN + 2 * lane) : make_float2(0.f, 0.f);
                 }
                 for (int c0 = 0; c0 < most; c0 += 32) {  // 32 entries of each row at a time
-                    int64_t jr[4];
+                    int jr[4];
                     float aw[4];
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
-                        const int64_t bq = __shfl_sync(0xffffffffu, base, q);
-                        const int eq = __shfl_sync(0xffffffffu, e0, q) + c0 + lane;
-                        const float iq = __shfl_sync(0xffffffffu, icb, q);
-                        const bool in = c0 + lane < deg[q];
-                        jr[q] = in ? bq + g.col[eq] : 0;
-                        aw[q] = in ? g.val[eq] * iq : 0.f;
+                        jr[q] = jc[q4 + q];
+                        aw[q] = ac[q4 + q];
+                        if (c0 > 0) {
+                            const int eq = __shfl_sync(0xffffffffu, e0, q4 + q) + c0 + lane;
+                            const float iq = __shfl_sync(0xffffffffu, icb, q4 + q);
+                            const bool in = c0 + lane < deg[q];
+                            jr[q] = in ? g.col[eq] : 0;
+                            aw[q] = in ? g.val[eq] * iq : 0.f;
+                        }
                     }
                     const int lim = min(32, most - c0);
-                    for (int t = 0; t < lim; t += 2) {
-                        float2 x[2][4];
-                        float a[2][4];
+                    for (int t = 0; t < lim; t += 4) {
+                        float2 x[4][4];
+                        float a[4][4];
 #pragma unroll
-                        for (int u = 0; u < 2; ++u)
+                        for (int u = 0; u < 4; ++u)
 #pragma unroll
                             for (int q = 0; q < 4; ++q) {
-                                const int64_t j = __shfl_sync(0xffffffffu, jr[q], (t + u) & 31);
-                                a[u][q] = __shfl_sync(0xffffffffu, aw[q], (t + u) & 31);
+                                const int j = __shfl_sync(0xffffffffu, jr[q], t + u);
+                                a[u][q] = __shfl_sync(0xffffffffu, aw[q], t + u);
                                 x[u][q] = make_float2(0.f, 0.f);
-                                if (t + u < 32 && c0 + t + u < deg[q]) x[u][q] = ld2(p.H + j * DIN + 2 * lane);
+                                if (c0 + t + u < deg[q]) x[u][q] = ld2(hb[q] + int64_t(j) * DIN);
                             }
 #pragma unroll
-                        for (int u = 0; u < 2; ++u)
+                        for (int u = 0; u < 4; ++u)
 #pragma unroll
                             for (int q = 0; q < 4; ++q)
-                                if (t + u < 32 && c0 + t + u < deg[q]) {  // warp-uniform
+                                if (c0 + t + u < deg[q]) {  // warp-uniform
                                     a0[q] = fmaf(a[u][q], x[u][q].x, a0[q]);
                                     a1[q] = fmaf(a[u][q], x[u][q].y, a1[q]);
                                 }
