@@ -66,7 +66,7 @@ struct alm_handle {
     int64_t launches = 0;
     std::vector<DevBuf> bufs;
     // pattern
-    int *up_row = nullptr, *up_col = nullptr, *up_sel_k = nullptr, *d_sel_k = nullptr;
+    int *up_col = nullptr, *up_sel_k = nullptr, *d_sel_k = nullptr;
     int *f_ptr = nullptr, *f_col = nullptr;
     int2 *up_slot = nullptr;
     int *gd_ptr = nullptr, *gd_k = nullptr, *gu_ptr = nullptr, *gu_k = nullptr;
@@ -244,7 +244,6 @@ static SparseView<T> view(const alm_handle *h) {
     v.n = int(h->n);
     v.m = int(h->m);
     v.nnz_u = h->nnz_u;
-    v.up_row = h->up_row;
     v.up_col = h->up_col;
     v.up_ptr = h->up_ptr;
     v.d_s_lo = static_cast<T *>(h->d_s_lo);
@@ -452,7 +451,6 @@ static alm_status create_impl(alm_handle *h, const alm_problem *p, const alm_opt
     // all constraints are diagonal selectors (MaxCut-like): the dual update is fused into k_eval
     h->fused_dual = hp.m_gen == 0 && !hp.has_off_sel && hp.n_sel == hp.m;
 
-    TRY(upload(h, &h->up_row, hp.up_row));
     h->ell_kf = hp.ell_kf;
     h->ell_ku = hp.ell_ku;
     if (hp.ell_kf > 0) {

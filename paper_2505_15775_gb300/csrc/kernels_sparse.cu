@@ -1242,20 +1242,13 @@ void launch_inner_slack(const LaunchCtx &c, const SparseView<T> &v, T *R, const 
             const int grid = grid_for(c, fn, v.n, kBlock);
             fn<<<grid, kBlock, 0, c.stream>>>(v, R, D, r, ldr, c.st, done);
         });
-        ++*c.launches;
-        return;
+    } else {
+        ALM_DISPATCH_LANES(L, {
+            auto *fn = D ? k_inner_slack<T, LN, true> : k_inner_slack<T, LN, false>;
+            const int grid = grid_for(c, fn, v.n, 4 * (kBlock / LN));
+            fn<<<grid, kBlock, 0, c.stream>>>(v, R, D, r, ldr, c.st, done);
+        });
     }
-    ALM_DISPATCH_LANES(L, {
-        if (D) {
-            auto *fn = k_inner_slack<T, LN, true>;
-            const int grid = grid_for(c, fn, v.n, 4 * (kBlock / LN));
-            fn<<<grid, kBlock, 0, c.stream>>>(v, R, D, r, ldr, c.st, done);
-        } else {
-            auto *fn = k_inner_slack<T, LN, false>;
-            const int grid = grid_for(c, fn, v.n, 4 * (kBlock / LN));
-            fn<<<grid, kBlock, 0, c.stream>>>(v, R, D, r, ldr, c.st, done);
-        }
-    });
     ++*c.launches;
 }
 
