@@ -91,10 +91,10 @@ struct alm_handle {
     bool off_fast = false;       // inner slack update without FP64 for off-diagonal selectors
     void *up_sel_a2 = nullptr, *up_sel_t = nullptr, *ob_hi = nullptr, *ob_lo = nullptr, *obb_hi = nullptr,
          *obb_lo = nullptr;
-    int n_heavy = 0;             // rows above kHeavyRow entries, and segments of long upper rows
+    int n_heavy = 0, n_hseg = 0; // rows above kHeavyRow entries, and segments of long upper rows
     int64_t n_useg = 0;
-    int *hv_row = nullptr, *us_row = nullptr, *us_e0 = nullptr;
-    void *hv_sum = nullptr;
+    int *hv_row = nullptr, *hv_ptr = nullptr, *hs_row = nullptr, *hs_e0 = nullptr, *us_row = nullptr, *us_e0 = nullptr;
+    void *hs_sum = nullptr;
     int n_gchunk = 0;
     int *gc_con = nullptr, *g_cptr = nullptr;
     double *g_part = nullptr;
@@ -303,7 +303,11 @@ static SparseView<T> view(const alm_handle *h) {
     v.off_fast = h->off_fast ? 1 : 0;
     v.n_heavy = h->n_heavy;
     v.hv_row = h->hv_row;
-    v.hv_sum = static_cast<T *>(h->hv_sum);
+    v.hv_ptr = h->hv_ptr;
+    v.n_hseg = h->n_hseg;
+    v.hs_row = h->hs_row;
+    v.hs_e0 = h->hs_e0;
+    v.hs_sum = static_cast<T *>(h->hs_sum);
     v.n_useg = h->n_useg;
     v.us_row = h->us_row;
     v.us_e0 = h->us_e0;
@@ -586,12 +590,24 @@ static alm_status create_impl(alm_handle *h, const alm_problem *p, const alm_opt
         }
     }
     if (hp.ell_kf == 0) {  // the CSR kernels' long rows
-        std::vector<int32_t> hv;
-        for (int64_t i = 0; i < h->n; ++i)
-            if (hp.f_ptr[size_t(i) + 1] - hp.f_ptr[size_t(i)] > kHeavyRow) hv.push_back(int32_t(i));
+        std::vector<int32_t> hv, first(1, 0), row, e0;
+        for (int64_t i = 0; i < h->n; ++i) {
+            const int64_t b = hp.f_ptr[size_t(i)], e = hp.f_ptr[size_t(i) + 1];
+            if (e - b <= kHeavyRow) continue;
+            hv.push_back(int32_t(i));
+            for (int64_t s = b; s < e; s += kHeavySeg) {
+                row.push_back(int32_t(i));
+                e0.push_back(int32_t(s));
+            }
+            first.push_back(int32_t(row.size()));
+        }
         h->n_heavy = int(hv.size());
+        h->n_hseg = int(row.size());
         TRY(upload(h, &h->hv_row, hv));
-        TRY(dalloc(h, &h->hv_sum, sizeof(double) * 2 * kMaxRank * hv.size()));
+        TRY(upload(h, &h->hv_ptr, first));
+        TRY(upload(h, &h->hs_row, row));
+        TRY(upload(h, &h->hs_e0, e0));
+        TRY(dalloc(h, &h->hs_sum, sizeof(double) * 2 * kMaxRank * row.size()));
         CK(cudaStreamSynchronize(h->stream));
     }
     {

@@ -18,7 +18,8 @@ constexpr int kBlock = 256;      // threads per block of the row kernels
 constexpr int kNumSMs = 152;     // GB300
 constexpr int kLzClusterRows = 8192;  // longest vectors of the one-launch eigensolve
 constexpr int kGenChunk = 256;   // entries of a general constraint per CTA
-constexpr int kHeavyRow = 256;   // longer rows of the full pattern are summed by a CTA each
+constexpr int kHeavyRow = 256;   // longer rows of the full pattern are summed beforehand, by CTAs
+constexpr int kHeavySeg = 512;   // ... of this many entries each
 constexpr int kUpSeg = 128;      // longer rows of the strict upper pattern are cut into segments
 constexpr int kPartStride = 160; // doubles of partial sums per block (>= kLzMax + 4, >= 1 + kMaxLR*kMaxRank)
 
@@ -158,8 +159,10 @@ struct SparseView {
     const T *up_sel_t;               // a in the working precision
     int off_fast;                    // the inner loop's slack update needs no FP64 (k_inner_off)
     int n_heavy;                     // rows of more than kHeavyRow entries in the full pattern:
-    const int *hv_row;               // ascending
-    T *hv_sum;                       // their off-diagonal sums (k_spmm_heavy)
+    const int *hv_row, *hv_ptr;      // ascending; their first segments (n_heavy + 1)
+    int n_hseg;                      // segments of kHeavySeg entries: row, first entry and
+    const int *hs_row, *hs_e0;
+    T *hs_sum;                       // off-diagonal sums (k_spmm_heavy)
     int64_t n_useg;                  // segments of kUpSeg entries of the strict upper rows beyond
     const int *us_row, *us_e0;       // their first kUpSeg: row and first entry
     T *d_s;                          // S_ii (FP32 form: the leading float of a float pair)

@@ -23,10 +23,10 @@
 // one (wide_rows): with one subgroup a row of 80 entries is a serial walk and 10,000 rows at
 // rank 3 fill 40 of 152 multiprocessors.  Rows above kHeavyRow entries
 // (heavy-tailed graphs) would still be one warp's serial walk: the SpMM's are summed
-// beforehand by a CTA each (k_spmm_heavy); the SDDMMs' sums are scalars, so their rows are
+// beforehand, kHeavySeg entries by a CTA (k_spmm_heavy); the SDDMMs' sums are scalars, so their rows are
 // cut into segments of kUpSeg entries that any row group takes.
 // In FP32, against one subgroup a row and two rows a group: alm_grad on a Kronecker graph of
-// 2^16 rows at r = 32 1.62 -> 0.36 ms; 32 inner steps of matrix completion (n = 1e4, 829,000
+// 2^16 rows at r = 32 1.62 -> 0.17 ms; 32 inner steps of matrix completion (n = 1e4, 829,000
 // entries, rank 3) 10.4 -> 4.5 ms.
 //
 // Precision.  FP64 arithmetic is scarce on GB300, so in the FP32 form every per-entry
@@ -649,8 +649,10 @@ __global__ void __launch_bounds__(kBlock) k_inner_off(SparseView<T> v, const T *
 //   MODE 1: inner CG step: also <G, G_old> (G is updated in place) and <G, D_old>, the
 //           stop test ||G|| <= tau and the Polak-Ribiere+ coefficient
 // ---------------------------------------------------------------------------------------
-// Off-diagonal sums of the rows above kHeavyRow entries, one CTA each, into hv_sum (the
-// accumulator's state per column vector; k_spmm adds it to the row's diagonal part).
+// Off-diagonal sums of the rows above kHeavyRow entries, segments of kHeavySeg of them by one CTA
+// each, into hs_sum (the accumulator's state per column vector; k_spmm adds a row's up).  With one
+// CTA per row the longest row set the time (129 us at 8.6% of the SM rate): alm_grad on a Kronecker
+// graph of 2^16 rows at r = 32, FP32, 268 -> 170 us.
 template <typename T, int LANES>
 __global__ void __launch_bounds__(kBlock) k_spmm_heavy(SparseView<T> v, const T *__restrict__ R, int r, int ldr,
                                                        const int *done) {
@@ -664,12 +666,12 @@ __global__ void __launch_bounds__(kBlock) k_spmm_heavy(SparseView<T> v, const T 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int gl = lane & (LANES - 1);
     const bool active = gl * W < r;
-    for (int q = blockIdx.x; q < v.n_heavy; q += gridDim.x) {
-        const int i = v.hv_row[q];
-        const int e1 = v.f_ptr[i + 1];
+    for (int q = blockIdx.x; q < v.n_hseg; q += gridDim.x) {
+        const int i = v.hs_row[q], e0 = v.hs_e0[q];
+        const int e1 = min(v.f_ptr[i + 1], e0 + kHeavySeg);
         Acc acc;
         acc.init();
-        for (int e = v.f_ptr[i] + threadIdx.x / LANES; e < e1; e += U * NSUB) {
+        for (int e = e0 + threadIdx.x / LANES; e < e1; e += U * NSUB) {
             int j[U];
             T c[U];
             V x[U];
@@ -690,7 +692,7 @@ __global__ void __launch_bounds__(kBlock) k_spmm_heavy(SparseView<T> v, const T 
         __syncthreads();
         if (threadIdx.x < LANES) {
             for (int ww = 1; ww < kBlock / 32; ++ww) acc.add_stored(sh[ww][lane]);
-            acc.store(v.hv_sum + (int64_t(q) * LANES + lane) * (Acc::kWords * W));
+            acc.store(v.hs_sum + (int64_t(q) * LANES + lane) * (Acc::kWords * W));
         }
         __syncthreads();
     }
@@ -725,7 +727,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 3 : 4) k_spmm(SparseV
             if constexpr (W == 4) zl[l] = make_float4(zz[0], zz[1], zz[2], zz[3]);
             else zl[l] = make_double2(zz[0], zz[1]);
         }
-    T pgg = T(0), pgo = T(0), pgd = T(0), pzg = T(0);
+    T pgg = T(0), pgg_lo = T(0), pgo = T(0), pgd = T(0), pzg = T(0);
     const bool pc = MODE == 1 && st->precond;
     const T sig = T(st->sigma);
     const T pc_floor = T(st->pc_floor);
@@ -753,7 +755,10 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 3 : 4) k_spmm(SparseV
                 if (v.hv_row[mid] < int(i)) a = mid + 1;
                 else b = mid;
             }
-            if (sub == 0) acc.add_stored(v.hv_sum + (int64_t(a) * LANES + gl) * (Acc::kWords * W));
+            const int q1 = v.hv_ptr[a + 1];
+#pragma unroll 4
+            for (int q = v.hv_ptr[a] + sub; q < q1; q += SP)
+                acc.add_stored(v.hs_sum + (int64_t(q) * LANES + gl) * (Acc::kWords * W));
         } else {
             for (int e = e0 + sub; e < e1; e += U * SP) {
                 int j[U];
@@ -770,11 +775,20 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 3 : 4) k_spmm(SparseV
 #pragma unroll
                 for (int k = 0; k < U; ++k) acc.add(c[k], x[k]);
             }
-            __syncwarp(gmask);
-            acc.template merge<LANES, GW>(gmask);
         }
+        __syncwarp(gmask);
+        acc.template merge<LANES, GW>(gmask);
         const V g = mask_tail(scale4(T(2), acc.value()), gl * W, r);
-        if (sub == 0) pgg += dot(g, g);
+        if constexpr (MODE == 0 && sizeof(T) == 4) {  // a few long rows can hold most of |G|^2: a float pair
+            if (sub == 0) {
+                T h, l;
+                dot_pair(g, g, h, l);
+                two_sum_acc(pgg, pgg_lo, h);
+                pgg_lo += l;
+            }
+        } else if (sub == 0) {
+            pgg += dot(g, g);
+        }
         if (MODE == 1) {
             // Row-block Jacobi preconditioner Z = P^{-1} G with P_i = 2 s_i I + 4 sigma a_i^2 r_i r_i^T
             // (the block of the Hessian of L in row i: the S_ii part and the penalty of the
@@ -801,7 +815,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 3 : 4) k_spmm(SparseV
         }
     }
     double *part = partials + size_t(blockIdx.x) * kPartStride;
-    const double vals[4] = {double(pgg), double(pgo), double(pgd), double(pzg)};
+    const double vals[4] = {double(pgg) + double(pgg_lo), double(pgo), double(pgd), double(pzg)};
     block_partials<4>(vals, part, shm);
     if (!last_block(&st->counter[CNT_SPMM])) return;
     double tot[4];
@@ -1295,7 +1309,7 @@ template <typename T, int LN, bool LRB, int MODE>
 static void spmm_one(const LaunchCtx &c, const SparseView<T> &v, const T *R, int r, int ldr, T *G, const T *D,
                      const int *done) {
     if (v.n_heavy > 0) {
-        k_spmm_heavy<T, LN><<<std::min(v.n_heavy, c.grid), kBlock, 0, c.stream>>>(v, R, r, ldr, done);
+        k_spmm_heavy<T, LN><<<std::min(v.n_hseg, c.grid), kBlock, 0, c.stream>>>(v, R, r, ldr, done);
         ++*c.launches;
     }
     ALM_ROW_SPLIT(wide_rows(c, 2 * v.nnz_u, v.n, LN), LN, {

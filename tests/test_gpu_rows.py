@@ -67,6 +67,14 @@ def test_row_lengths(degrees, n, r, prec):
 
 
 @pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("r", [1, 5, 32])
+@pytest.mark.parametrize("degrees,n", [((511, 512, 513), 700), ((1024, 1025, 257, 3), 1100), ((6000, 2049), 6500)])
+def test_long_rows_in_segments(degrees, n, r, prec):
+    """Rows summed by several CTAs (512 entries each)."""
+    _check_primitives(_hubs(degrees, n), r, prec)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
 @pytest.mark.parametrize("r", [3, 32])
 @pytest.mark.parametrize("count", [1, 255, 256, 257, 1000])
 def test_general_constraint_lengths(count, r, prec):
