@@ -192,8 +192,12 @@ __device__ __forceinline__ void ls_finish(const SparseView<T> &v, DevState *st, 
             }
         const double sigma = st->sigma;
         double q[5];
-        q[0] = st->L;
-        q[1] = (MODE == 1) ? (-st->zg + st->beta * st->g_dprev) : s1;  // <G, D>, D = -Z + beta D_old
+        // MODE 1: q0 has no part in the step, and L is not computed in the inner loop (st->L is some
+        // earlier call's); at a restart beta = 0 and <G, D_old> is of whatever D_old holds.  Neither may
+        // reach the test for non-finite coefficients below.
+        q[0] = MODE == 1 ? 0.0 : st->L;
+        if (MODE == 1) q[1] = -st->zg + (st->beta != 0.0 ? st->beta * st->g_dprev : 0.0);  // <G, D>, D = -Z + beta D_old
+        else q[1] = s1;
         q[2] = s2 + 0.5 * sigma * a11;
         q[3] = sigma * a12;
         q[4] = 0.5 * sigma * a22;
