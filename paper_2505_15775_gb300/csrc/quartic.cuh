@@ -47,7 +47,30 @@ __device__ inline int real_cubic_roots64(double c3, double c2, double c1, double
         }
         x[k] = t;
     }
-    return nr;
+    // The discriminant's sign is its rounding's when two roots lie some 1e8 times below the third: the
+    // quadratic that the largest root leaves over (divided out from the low end, which is the stable
+    // way for it) tells whether there are two more.
+    double xm = x[0];
+    for (int k = 1; k < nr; ++k)
+        if (fabs(x[k]) > fabs(xm)) xm = x[k];
+    const double g = -c0 / xm, b = (g - c1) / xm;  // (x - xm)(c3 x^2 + b x + g)
+    const double d2 = b * b - 4.0 * c3 * g;
+    if (!(d2 > 0.0) || !isfinite(d2)) return nr;
+    const double h = -0.5 * (b + copysign(sqrt(d2), b));
+    const double two[2] = {h / c3, g / h};
+    for (int k = 0; k < 2; ++k) {
+        double t = two[k];
+        for (int it = 0; it < 4; ++it) {
+            const double f = ((c3 * t + c2) * t + c1) * t + c0;
+            const double fp = (3.0 * c3 * t + 2.0 * c2) * t + c1;
+            const double nt = t - f / fp;
+            if (!isfinite(nt)) break;
+            t = nt;
+        }
+        x[k + 1] = t;
+    }
+    x[0] = xm;
+    return 3;
 }
 
 // FP64 on this part: 64 cycles an instruction for the one thread that runs this, 568 a division,
@@ -105,8 +128,13 @@ __device__ inline int real_cubic_roots(double c3, double c2, double c1, double c
         for (int k = 0; k < 3; ++k) t0[k] = 2.f * rr * cosf(ph - 2.0943951f * float(k)) + shift;
         nr = 3;
     }
-    bool ok = true;
-    double sum = B;
+    // The FP32 starts do for roots of similar size.  Where roots lie far below the largest (a cubic
+    // whose leading coefficient is small: -0.17 + 4.8e-6 a + 4.5 a^3 + 2e-8 a^4 has its minimum at 0.11
+    // and a stationary point at -1.7e8) they may not: a discriminant within rounding of its terms does not
+    // tell one real root from three, and two starts can end on one root.  Both are seen here, as is a
+    // Newton that has not converged, and FP64 throughout takes over.
+    bool ok = nr == 3 || disc > 0x1p-20 * fma(hq, hq, fabs(p3 * p3 * p3));
+    double t1[3];
     for (int k = 0; k < nr; ++k) {  // Newton on the scaled cubic
         double t = double(t0[k]);
         bool conv = false;
@@ -120,12 +148,11 @@ __device__ inline int real_cubic_roots(double c3, double c2, double c1, double c
             conv = fabs(d) <= 0x1p-30 * fabs(t);  // the error is now its square
         }
         ok = ok && conv;
-        sum += t;
+        t1[k] = t;
         x[k] = t * pow2(e);
+        for (int l = 0; l < k; ++l) ok = ok && fabs(t - t1[l]) > 0x1p-16 * fmax(fabs(t), fabs(t1[l]));
     }
-    // a root far below the others may lie under their FP32 rounding: not converged, or two starts
-    // that ended on one root (three roots sum to -B)
-    if (!ok || (nr == 3 && fabs(sum) > 1e-9)) return real_cubic_roots64(c3, c2, c1, c0, x);
+    if (!ok) return real_cubic_roots64(c3, c2, c1, c0, x);
     return nr;
 }
 
