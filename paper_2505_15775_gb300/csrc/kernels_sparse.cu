@@ -574,9 +574,35 @@ __global__ void __launch_bounds__(kBlock) k_prep_off(SparseView<T> v, const doub
     }
 }
 
+// (h + l) + sigma m (c x - b) as a normalised pair; x, b and sigma are pairs, m and c floats.  Every
+// product and sum keeps its rounding error, so that the result has its own relative accuracy also
+// where the two terms cancel (a multiplier close to sigma times a large residual).
+__device__ __forceinline__ void selector_slack(float h, float l, float m, float c, float xh, float xl, float bh,
+                                               float bl, float sh, float sl, float &oh, float &ol) {
+    const float ph = c * xh;
+    const float pe = fmaf(c, xh, -ph) + c * xl;
+    const float s0 = ph - bh;
+    const float bb = s0 - ph;
+    const float r0 = ((ph - (s0 - bb)) + (-bh - bb)) + (pe - bl);
+    const float kh = sh * m;
+    const float kl = fmaf(sh, m, -kh) + sl * m;
+    const float ch = kh * s0;
+    const float cl = fmaf(kh, s0, -ch) + fmaf(kh, r0, kl * s0);
+    const float s1 = h + ch;
+    const float b1 = s1 - h;
+    const float e1 = l + (cl + ((h - (s1 - b1)) + (ch - b1)));
+    oh = s1 + e1;
+    ol = e1 - (oh - s1);
+}
+__device__ __forceinline__ void selector_slack(double h, double, double m, double c, double x, double, double b, double,
+                                               double sigma, double, double &oh, double &ol) {
+    oh = fma(sigma * m, fma(c, x, -b), h);
+    ol = 0.0;
+}
+
 // Slack update of the inner loop when every constraint is a selector and some are off the
 // diagonal (matrix completion): S_ij = (C_ij - a y_k) + sigma a (2 a r_i.r_j - b_k) in float
-// pairs, as slack_row has it for the diagonal, in one pass over the upper pattern.  k_eval and
+// pairs (selector_slack), in one pass over the upper pattern.  k_eval and
 // k_dual_slack (still what ends an inner solve) put the values through FP64 A(X) and w, some 15
 // FP64 instructions an entry at 64 cycles a warp: together 85 us on 829,000 entries
 // at rank 3 (cold caches), this 18 us; 32 inner steps there 4.49 -> 3.00 ms with it.
@@ -594,7 +620,8 @@ __global__ void __launch_bounds__(kBlock) k_inner_off(SparseView<T> v, const T *
     const int64_t g0 = int64_t(blockIdx.x) * (kBlock / GW) + threadIdx.x / GW;
     const int64_t ng = int64_t(gridDim.x) * (kBlock / GW);
     const bool active = gl * W < r;
-    const T sigma = T(st->sigma);
+    T sh, sl;
+    split_pair(st->sigma, sh, sl);
     auto upper = [&](V ri, int64_t i, int e0, int e1) {
         for (int e = e0 + sub; e < e1 + sub; e += U * SP) {  // group-uniform trip count
             int j[U];
@@ -610,21 +637,13 @@ __global__ void __launch_bounds__(kBlock) k_inner_off(SparseView<T> v, const T *
                 pair_group_sum<LANES>(xh, xl, gmask);
                 const int q = e + k * SP;
                 if (gl == 0 && q < e1) {
-                    T s = v.ob_hi[q];
                     const T a = v.up_sel_t[q];  // 0 without a selector
-                    const T a2 = a + a;
-                    const T ph = a2 * xh;
-                    const T pe = fma(a2, xh, -ph) + a2 * xl;
-                    const T bh = v.obb_hi[q];
-                    const T s0 = ph - bh;
-                    const T bb = s0 - ph;
-                    const T err = (ph - (s0 - bb)) + (-bh - bb);
-                    const T corr = sigma * a * (s0 + (err + pe - v.obb_lo[q]));
-                    s = s + (corr + v.ob_lo[q]);
+                    T s, lo;
+                    selector_slack(v.ob_hi[q], v.ob_lo[q], a, a + a, xh, xl, v.obb_hi[q], v.obb_lo[q], sh, sl, s, lo);
                     v.up_s[q] = s;
-                    const int2 sl = v.up_slot[q];
-                    v.f_val[sl.x] = s;
-                    v.f_val[sl.y] = s;
+                    const int2 at = v.up_slot[q];
+                    v.f_val[at.x] = s;
+                    v.f_val[at.y] = s;
                 }
             }
         }
@@ -634,7 +653,15 @@ __global__ void __launch_bounds__(kBlock) k_inner_off(SparseView<T> v, const T *
         const int e0 = v.up_ptr[i], e1 = min(v.up_ptr[i + 1], e0 + kUpSeg);
         T xh, xl;
         norm2_pair(ri, gmask, LANES, xh, xl);
-        if (gl == 0 && sub == 0) slack_row<T, LANES>(v, i, xh, xl, sigma);
+        if (gl == 0 && sub == 0) {
+            T dh = v.base_hi[i], dl = v.base_lo ? v.base_lo[i] : T(0);
+            if (v.d_sel_k[i] >= 0) {
+                const T a = sizeof(T) == 8 ? T(v.d_sel_a[i]) : T(v.d_sel_af[i]);
+                selector_slack(dh, dl, a, a, xh, xl, v.b_hi[i], v.b_lo ? v.b_lo[i] : T(0), sh, sl, dh, dl);
+            }
+            v.d_s[i] = dh;
+            if (v.d_s_lo) v.d_s_lo[i] = dl;
+        }
         upper(ri, i, e0, e1);
     }
     for (int64_t q = g0; q < v.n_useg; q += ng) {
