@@ -453,8 +453,8 @@ __global__ void __launch_bounds__(kLzcThreads, 1) k_lz_cluster(SparseView<T> v, 
         buf ^= 1;
         __syncthreads();
     };
-    // part[warp][slot] = the warp's sum of x
-    auto warp_part = [&](T x, int slot) {
+    // part[warp][slot] = the warp's sum of x (in x's type)
+    auto warp_part = [&](auto x, int slot) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
         if (lane == 0) part[warp * nv + slot] = double(x);
@@ -540,22 +540,22 @@ __global__ void __launch_bounds__(kLzcThreads, 1) k_lz_cluster(SparseView<T> v, 
 
     // start vector: seeded, or the previous Ritz vector plus a seeded one of norm 0.05
     {
-        T nrm = T(0);
+        double nrm = 0.0;  // the norms of the start, the Ritz vector and the residual sum in FP64
         for (int lr = tid; lr < nrows; lr += kLzcThreads) {
             const uint64_t z = splitmix64_at(a.seed, uint64_t(row0 + lr));
             const T x = T(2.0 * (double(z >> 11) * (1.0 / 9007199254740992.0)) - 1.0);
             ws[lr] = x;
-            nrm = fma(x, x, nrm);
+            nrm = fma(double(x), double(x), nrm);
         }
         warp_part(nrm, 0);
         cluster_sum(1);
         if (a.warm) {
             const T c = T(0.05 / sqrt(tot[0]));
-            nrm = T(0);
+            nrm = 0.0;
             for (int lr = tid; lr < nrows; lr += kLzcThreads) {
                 const T x = a.Q[row0 + lr] + c * ws[lr];
                 ws[lr] = x;
-                nrm = fma(x, x, nrm);
+                nrm = fma(double(x), double(x), nrm);
             }
             warp_part(nrm, 0);
             cluster_sum(1);
@@ -608,7 +608,7 @@ __global__ void __launch_bounds__(kLzcThreads, 1) k_lz_cluster(SparseView<T> v, 
         __syncthreads();
         theta = sc[1];
         resid = sc[2];
-        warp_part(combine(m, false), 0);
+        warp_part(double(combine(m, false)), 0);
         cluster_sum(1);
         if (tid == 0) sc[0] = tot[0] > 0.0 ? 1.0 / sqrt(tot[0]) : 0.0;
         __syncthreads();
@@ -622,7 +622,7 @@ __global__ void __launch_bounds__(kLzcThreads, 1) k_lz_cluster(SparseView<T> v, 
         const T d = ws[lr] - T(theta) * qs[row0 + lr];
         r2 = fma(d, d, r2);
     }
-    warp_part(r2, 0);
+    warp_part(double(r2), 0);
     cluster_sum(1);
     if (rank == 0 && tid == 0) {
         st->theta = theta;
