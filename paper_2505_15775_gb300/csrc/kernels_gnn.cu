@@ -346,13 +346,15 @@ __global__ void __launch_bounds__(256, 2) k_gnn_layer(GnnGraph g, GnnLayerArgs<T
                         make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
             for (int lr = tid; lr < TR; lr += 256)
                 if (r0 + lr < g.rows) {
-                    float s0 = 0.f, s1 = 0.f;
-#pragma unroll 8
-                    for (int k = 0; k < kGnnHid; k += 2) {
-                        s0 = fmaf(wy[k], hx[k * TP + lr], s0);
-                        s1 = fmaf(wy[k + 1], hx[(k + 1) * TP + lr], s1);
-                    }
-                    p.yhat[r0 + lr] = (s0 + s1) + by;
+                    float t[kGnnHid / 2];  // pairs and then halves: 7 roundings deep, two chains would be 33
+#pragma unroll
+                    for (int k = 0; k < kGnnHid / 2; ++k)
+                        t[k] = fmaf(wy[k], hx[k * TP + lr], wy[k + kGnnHid / 2] * hx[(k + kGnnHid / 2) * TP + lr]);
+#pragma unroll
+                    for (int o = kGnnHid / 4; o > 0; o >>= 1)
+#pragma unroll
+                        for (int k = 0; k < o; ++k) t[k] += t[k + o];
+                    p.yhat[r0 + lr] = t[0] + by;
                 }
             __syncthreads();
         }
