@@ -66,7 +66,7 @@ struct alm_handle {
     int64_t launches = 0;
     std::vector<DevBuf> bufs;
     // pattern
-    int *up_col = nullptr, *up_sel_k = nullptr, *d_sel_k = nullptr;
+    int *up_row = nullptr, *up_col = nullptr, *up_sel_k = nullptr, *d_sel_k = nullptr;
     int *f_ptr = nullptr, *f_col = nullptr;
     int2 *up_slot = nullptr;
     int *gd_ptr = nullptr, *gd_k = nullptr, *gu_ptr = nullptr, *gu_k = nullptr;
@@ -245,6 +245,7 @@ static SparseView<T> view(const alm_handle *h) {
     v.m = int(h->m);
     v.nnz_u = h->nnz_u;
     v.up_col = h->up_col;
+    v.up_row = h->up_row;
     v.up_ptr = h->up_ptr;
     v.d_s_lo = static_cast<T *>(h->d_s_lo);
     v.base_hi = static_cast<const T *>(h->base_hi);
@@ -472,6 +473,7 @@ static alm_status create_impl(alm_handle *h, const alm_problem *p, const alm_opt
     }
     TRY(upload(h, &h->up_ptr, hp.up_ptr));
     TRY(upload(h, &h->up_col, hp.up_col));
+    TRY(upload(h, &h->up_row, hp.up_row));
     {
         std::vector<float> af(hp.d_sel_a.begin(), hp.d_sel_a.end());
         TRY(upload(h, &h->d_sel_af, af));

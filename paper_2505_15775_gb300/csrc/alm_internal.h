@@ -29,6 +29,7 @@ constexpr int kPartStride = 160; // doubles of partial sums per block (>= kLzMax
 struct HostPattern {
     int64_t n = 0, m = 0;
     std::vector<int32_t> up_ptr, up_col;     // strict upper CSR
+    std::vector<int32_t> up_row;             // row of each upper entry
     int ell_kf = 0, ell_ku = 0;              // ELL widths (0: no ELL layout)
     std::vector<int32_t> f_ell_col, u_ell_col;  // n x ell_kf / n x ell_ku, padded with the row itself
     std::vector<double> f_ell_val, u_ell_val;   // C_ij on them, 0 in the padding
@@ -141,6 +142,7 @@ struct SparseView {
     int n, m;
     int64_t nnz_u;
     const int *up_ptr, *up_col;     // strict upper pattern (CSR)
+    const int *up_row;              // ... and the row of each entry
     const T *up_c;                  // C_ij on it
     T *up_s;                        // S_ij on it (aliases up_c while S_off = C_off is static)
     const int *up_sel_k;            // may be null

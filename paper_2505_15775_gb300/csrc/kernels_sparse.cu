@@ -17,7 +17,7 @@
 //
 // Work decomposition.  LANES lanes hold one row of R (lane l the 16-byte vector of columns
 // [l W, l W + W), W = 4 floats or 2 doubles), so a gathered row is one coalesced
-// 16*LANES-byte read.  SP such subgroups share a row of the pattern (k_eval, k_spmm, k_ls):
+// 16*LANES-byte read.  SP such subgroups share a row of the pattern (k_spmm, k_ls, k_inner_off):
 // subgroup s takes its entries s, s + SP, .., and a row group is LANES x SP lanes.  SP is
 // a whole warp's worth when the rows are long enough to give each subgroup two entries, else
 // one (wide_rows): with one subgroup a row of 80 entries is a serial walk and 10,000 rows at
@@ -258,7 +258,14 @@ __global__ void __launch_bounds__(kBlock) k_prep_base(SparseView<T> v, const dou
 // ---------------------------------------------------------------------------------------
 // (a) constraint map + <C, RR^T> (+ fused dual update for diagonal-selector problems)
 // ---------------------------------------------------------------------------------------
-template <typename T, int LANES, int SP, bool OFFSEL, bool LR, bool FUSED>
+// The rows' FP64 work goes through a warp at a time; the strict upper entries are taken two per
+// row group and round from the whole pattern, whatever rows they lie in: four independent gathers
+// a lane, and no row sets the time.  Walking the entries by rows instead (subgroups of a warp sharing
+// the long ones) was slower nearly everywhere: ER(60,000) of degree 40, r = 32, FP32 151 us a call
+// against 102; a Kronecker graph of 2^13 rows, r = 1 110 against 64; matrix completion, n = 1e4, r = 3,
+// FP64 123 against 101.  BYROW is what is left of it: FP32 factors that do not stay in L2 and rows of at
+// most two upper entries, where it reads R twice instead of 2.5 times (eval_by_row has the line).
+template <typename T, int LANES, bool BYROW, bool OFFSEL, bool LR, bool FUSED>
 __global__ void __launch_bounds__(kBlock) k_eval(SparseView<T> v, const T *__restrict__ R, int r, int ldr,
                                                  double *__restrict__ AX, const double *__restrict__ y,
                                                  double *__restrict__ w, int nb, double sigma_arg, HostResult *res,
@@ -266,49 +273,35 @@ __global__ void __launch_bounds__(kBlock) k_eval(SparseView<T> v, const T *__res
     if (*done) return;
     using V = typename VecT<T>::type;
     constexpr int W = VecT<T>::W;
-    constexpr int GW = LANES * SP;
-    constexpr int U = 2;  // entries per subgroup and round
+    constexpr int U = 2;  // entries per row group and round
     __shared__ double shm[32 * 32];
     const int lane = threadIdx.x & 31;
-    const int gl = lane & (LANES - 1), sub = (lane & (GW - 1)) / LANES;
-    const unsigned gmask = group_mask<GW>(lane);
-    const int64_t g0 = int64_t(blockIdx.x) * (kBlock / GW) + threadIdx.x / GW;
-    const int64_t ng = int64_t(gridDim.x) * (kBlock / GW);
+    const int gl = lane & (LANES - 1);
+    const unsigned gmask = group_mask<LANES>(lane);
+    const int64_t g0 = int64_t(blockIdx.x) * (kBlock / LANES) + threadIdx.x / LANES;
+    const int64_t ng = int64_t(gridDim.x) * (kBlock / LANES);
     const bool active = gl * W < r;
     const double sigma = FUSED ? (sigma_arg >= 0.0 ? sigma_arg : st->sigma) : 0.0;
     T pc = T(0);
     double pyres = 0.0, pres2 = 0.0, pbw = 0.0;
 
-    // strict upper entries e0 .. e1-1 of a row (ri its masked vector)
+    // BYROW: strict upper entries e0 .. e1-1 of a row (ri its masked vector)
     auto upper = [&](V ri, int64_t i, int e0, int e1) {
         T acc = T(0);
-        for (int e = e0 + sub; e < e1 + sub; e += U * SP) {  // group-uniform trip count
+        for (int e = e0; e < e1; e += U) {
             int j[U];
             T c[U];
             V x[U];
 #pragma unroll
             for (int k = 0; k < U; ++k) {
-                const bool in = e + k * SP < e1;
-                j[k] = in ? v.up_col[e + k * SP] : int(i);
-                c[k] = in ? v.up_c[e + k * SP] : T(0);
+                const bool in = e + k < e1;
+                j[k] = in ? v.up_col[e + k] : int(i);
+                c[k] = in ? v.up_c[e + k] : T(0);
             }
 #pragma unroll
             for (int k = 0; k < U; ++k) x[k] = load_row(R, j[k], ldr, gl, active);
 #pragma unroll
-            for (int k = 0; k < U; ++k) {
-                if (OFFSEL) {
-                    T hi, lo;
-                    dot_pair(ri, x[k], hi, lo);
-                    acc += c[k] * hi;
-                    pair_group_sum<LANES>(hi, lo, gmask);
-                    if (gl == 0 && e + k * SP < e1) {
-                        const int q = v.up_sel_k[e + k * SP];
-                        if (q >= 0) AX[q] = 2.0 * v.up_sel_a[e + k * SP] * (double(hi) + double(lo));
-                    }
-                } else {
-                    acc += c[k] * dot(ri, x[k]);
-                }
-            }
+            for (int k = 0; k < U; ++k) acc += c[k] * dot(ri, x[k]);
         }
         pc += T(2) * acc;
     };
@@ -316,14 +309,14 @@ __global__ void __launch_bounds__(kBlock) k_eval(SparseView<T> v, const T *__res
     // every lane does one row's FP64 work.  An FP64 instruction holds a warp 64 cycles whatever
     // the number of active lanes, and a row takes about 16: one leader lane per row at a time
     // cost 206 us on 1e6 rows at r = 32, of which the memory traffic is 60.
-    constexpr int RW = 32 / GW;  // row groups of a warp
-    const int x = lane & (GW - 1);
+    constexpr int RW = 32 / LANES;  // row groups of a warp
+    const int x = gl;
     const int64_t tile = int64_t(RW) * nb;
     const int64_t nw = int64_t(gridDim.x) * (kBlock / 32);
     for (int64_t t0 = (int64_t(blockIdx.x) * (kBlock / 32) + (threadIdx.x >> 5)) * tile; t0 < v.n; t0 += nw * tile) {
         T kh = T(0), kl = T(0);
         for (int t = 0; t < nb; ++t) {
-            const int64_t i = t0 + int64_t(t) * RW + lane / GW;
+            const int64_t i = t0 + int64_t(t) * RW + lane / LANES;
             const bool in = i < v.n;  // group-uniform
             const V ri = mask_tail(load_row(R, in ? i : 0, ldr, gl, active && in), gl * W, r);
             T hi, lo;
@@ -332,13 +325,13 @@ __global__ void __launch_bounds__(kBlock) k_eval(SparseView<T> v, const T *__res
                 kh = hi;
                 kl = lo;
             }
-            if (in && !v.diag_only) {
+            if (BYROW && in && !v.diag_only) {
                 const int e0 = v.up_ptr[i];
                 upper(ri, i, e0, min(v.up_ptr[i + 1], e0 + kUpSeg));
             }
         }
         __syncwarp();
-        const int64_t i = t0 + int64_t(x) * RW + lane / GW;
+        const int64_t i = t0 + int64_t(x) * RW + lane / LANES;
         if (x < nb && i < v.n) {
             const double viid = double(kh) + double(kl);
             const T cii = v.d_c[i];
@@ -363,9 +356,48 @@ __global__ void __launch_bounds__(kBlock) k_eval(SparseView<T> v, const T *__res
         }
         __syncwarp();
     }
-    for (int64_t q = g0; q < v.n_useg && !v.diag_only; q += ng) {  // the rest of the long rows
-        const int i = v.us_row[q], e0 = v.us_e0[q], e1 = min(v.up_ptr[i + 1], e0 + kUpSeg);
-        upper(mask_tail(load_row(R, i, ldr, gl, active), gl * W, r), i, e0, e1);
+    if (BYROW) {
+        for (int64_t q = g0; q < v.n_useg && !v.diag_only; q += ng) {  // the rest of the long rows
+            const int i = v.us_row[q], e0 = v.us_e0[q], e1 = min(v.up_ptr[i + 1], e0 + kUpSeg);
+            upper(mask_tail(load_row(R, i, ldr, gl, active), gl * W, r), i, e0, e1);
+        }
+    } else if (!v.diag_only) {
+        for (int64_t e = g0; e < v.nnz_u; e += U * ng) {
+            V a[U], b[U];
+            T c[U];
+            bool has[U];
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+                has[k] = e + k * ng < v.nnz_u;  // group-uniform
+                const int64_t q = has[k] ? e + k * ng : e;
+                const int i = v.up_row[q], j = v.up_col[q];
+                c[k] = has[k] ? v.up_c[q] : T(0);
+                a[k] = load_row(R, i, ldr, gl, active);
+                b[k] = load_row(R, j, ldr, gl, active);
+            }
+#pragma unroll
+            for (int k = 0; k < U; ++k) {
+                a[k] = mask_tail(a[k], gl * W, r);
+                if (OFFSEL) {
+                    T hi, lo;
+                    dot_pair(a[k], b[k], hi, lo);
+                    if (sizeof(T) == 4) pc += T(2) * c[k] * hi;  // FP64: the leader's whole sum, one FMA
+                    pair_group_sum<LANES>(hi, lo, gmask);
+                    if (gl == 0 && has[k]) {
+                        const int64_t q = e + k * ng;
+                        const int s = v.up_sel_k[q];
+                        if (sizeof(T) == 8) {
+                            pc = fma(T(2) * c[k], hi, pc);
+                            if (s >= 0) AX[s] = double(v.up_sel_a2[q]) * double(hi);
+                        } else if (s >= 0) {
+                            AX[s] = 2.0 * v.up_sel_a[q] * (double(hi) + double(lo));
+                        }
+                    }
+                } else {
+                    pc += T(2) * c[k] * dot(a[k], b[k]);
+                }
+            }
+        }
     }
     double *part = partials + size_t(blockIdx.x) * kPartStride;
     if (FUSED) {
@@ -1233,18 +1265,33 @@ static inline bool wide_rows(const LaunchCtx &c, int64_t entries, int64_t n, int
     if (wide) { constexpr int SPW = 32 / LN; __VA_ARGS__; }                      \
     else { constexpr int SPW = 1; __VA_ARGS__; }
 
+// Whether k_eval walks the upper entries by rows: FP32, at most two upper entries a row and a factor
+// of 30 MB or more.  us a call, by rows / by entries: torus 449^2, r = 32 (26 MB) 65 / 64; 700^2,
+// r = 16 (31 MB) 69 / 72, r = 32 94 / 110; 1000^2, r = 32 150 / 183; random 3-regular 1e6, r = 32
+// 166 / 168; FP64, torus 700^2, r = 32 274 / 256.
+template <typename T>
+static inline bool eval_by_row(const SparseView<T> &v, int ldr) {
+    return sizeof(T) == 4 && v.nnz_u <= 2 * int64_t(v.n) && int64_t(v.n) * ldr * 4 >= 30000000;
+}
 template <typename T, int LN, bool OFF, bool LRB, bool FUS>
 static void eval_one(const LaunchCtx &c, const SparseView<T> &v, const T *R, int r, int ldr, double *AX,
                      const double *y, double *w, const int *done) {
-    ALM_ROW_SPLIT(wide_rows(c, v.nnz_u, v.n, LN), LN, {
-        auto *fn = k_eval<T, LN, SPW, OFF, LRB, FUS>;
-        // rows per row group and round: up to one per lane (for the FP64 work of the rows), as
-        // long as the rounds still give every multiprocessor 16 warps
-        const int64_t rw = 32 / (LN * SPW);
-        const int nb = int(std::max<int64_t>(1, std::min<int64_t>(LN * SPW, v.n / (rw * 16 * c.sms))));
-        const int grid = grid_for(c, fn, v.n + v.n_useg * nb, kBlock / (LN * SPW) * nb);
-        fn<<<grid, kBlock, 0, c.stream>>>(v, R, r, ldr, AX, y, w, nb, c.sigma, c.res, c.st, c.partials, done);
-    });
+    // rows per row group and round: up to one per lane (for the FP64 work of the rows), as
+    // long as the rounds still give every multiprocessor 16 warps
+    const int64_t rw = 32 / LN;
+    const int nb = int(std::max<int64_t>(1, std::min<int64_t>(LN, v.n / (rw * 16 * c.sms))));
+    if constexpr (sizeof(T) == 4 && !OFF) {
+        if (eval_by_row(v, ldr)) {
+            auto *fn = k_eval<T, LN, true, OFF, LRB, FUS>;
+            const int grid = grid_for(c, fn, v.n + v.n_useg * nb, kBlock / LN * nb);
+            fn<<<grid, kBlock, 0, c.stream>>>(v, R, r, ldr, AX, y, w, nb, c.sigma, c.res, c.st, c.partials, done);
+            return;
+        }
+    }
+    auto *fn = k_eval<T, LN, false, OFF, LRB, FUS>;
+    const int grid = std::max(grid_for(c, fn, v.n, kBlock / LN * nb),
+                              v.diag_only ? 1 : grid_for(c, fn, v.nnz_u, 2 * (kBlock / LN)));
+    fn<<<grid, kBlock, 0, c.stream>>>(v, R, r, ldr, AX, y, w, nb, c.sigma, c.res, c.st, c.partials, done);
 }
 
 template <typename T>

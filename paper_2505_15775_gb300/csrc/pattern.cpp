@@ -311,6 +311,10 @@ std::string build_pattern(const alm_problem *p, HostPattern *hp) {
             }
     }
 
+    hp->up_row.assign(size_t(nnz_u), 0);
+    for (int64_t i = 0; i < n; ++i)
+        for (int64_t e = hp->up_ptr[size_t(i)]; e < hp->up_ptr[size_t(i) + 1]; ++e) hp->up_row[size_t(e)] = int32_t(i);
+
     // ELL copies (fixed row width, padded with the row itself and value 0) when S's
     // off-diagonal values never change and every row is short: column indices then sit at
     // computable addresses, so the kernels can fetch them ahead of the row gathers
