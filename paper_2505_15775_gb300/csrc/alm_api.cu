@@ -91,6 +91,7 @@ struct alm_handle {
     bool off_fast = false;       // inner slack update without FP64 for off-diagonal selectors
     void *up_sel_a2 = nullptr, *up_sel_t = nullptr, *ob_hi = nullptr, *ob_lo = nullptr, *obb_hi = nullptr,
          *obb_lo = nullptr;
+    float f_len = 0.f, up_len = 0.f;  // SparseView
     int n_heavy = 0, n_hseg = 0; // rows above kHeavyRow entries, and segments of long upper rows
     int64_t n_useg = 0;
     int *hv_row = nullptr, *hv_ptr = nullptr, *hs_row = nullptr, *hs_e0 = nullptr, *us_row = nullptr, *us_e0 = nullptr;
@@ -302,6 +303,8 @@ static SparseView<T> view(const alm_handle *h) {
     v.obb_lo = static_cast<const T *>(h->obb_lo);
     v.up_sel_t = static_cast<const T *>(h->up_sel_t);
     v.off_fast = h->off_fast ? 1 : 0;
+    v.f_len = h->f_len;
+    v.up_len = h->up_len;
     v.n_heavy = h->n_heavy;
     v.hv_row = h->hv_row;
     v.hv_ptr = h->hv_ptr;
@@ -590,6 +593,19 @@ static alm_status create_impl(alm_handle *h, const alm_problem *p, const alm_opt
             TRY(dalloc(h, &h->base_hi, h->esz * nn));
             TRY(dalloc(h, &h->base_lo, h->esz * nn));
         }
+    }
+    {
+        auto entry_mean = [&](const std::vector<int32_t> &ptr, int64_t cap) {
+            double s1 = 0.0, s2 = 0.0;
+            for (size_t i = 0; i < size_t(h->n); ++i) {
+                const double len = double(std::min<int64_t>(int64_t(ptr[i + 1]) - ptr[i], cap));
+                s1 += len;
+                s2 += len * len;
+            }
+            return float(s1 > 0.0 ? s2 / s1 : 0.0);
+        };
+        h->f_len = entry_mean(hp.f_ptr, kHeavyRow);
+        h->up_len = entry_mean(hp.up_ptr, kUpSeg);
     }
     if (hp.ell_kf == 0) {  // the CSR kernels' long rows
         std::vector<int32_t> hv, first(1, 0), row, e0;

@@ -160,6 +160,8 @@ struct SparseView {
     const T *obb_hi, *obb_lo;        // b_k (both pairs; null unless off_fast)
     const T *up_sel_t;               // a in the working precision
     int off_fast;                    // the inner loop's slack update needs no FP64 (k_inner_off)
+    float f_len, up_len;             // mean length of an entry's row, in the full pattern (rows cut at
+                                     // kHeavyRow entries) and in the strict upper one (at kUpSeg)
     int n_heavy;                     // rows of more than kHeavyRow entries in the full pattern:
     const int *hv_row, *hv_ptr;      // ascending; their first segments (n_heavy + 1)
     int n_hseg;                      // segments of kHeavySeg entries: row, first entry and

@@ -19,12 +19,13 @@
 // [l W, l W + W), W = 4 floats or 2 doubles), so a gathered row is one coalesced
 // 16*LANES-byte read.  SP such subgroups share a row of the pattern (k_spmm, k_ls, k_inner_off):
 // subgroup s takes its entries s, s + SP, .., and a row group is LANES x SP lanes.  SP is
-// a whole warp's worth when the rows are long enough to give each subgroup two entries, else
-// one (wide_rows): with one subgroup a row of 80 entries is a serial walk and 10,000 rows at
+// a whole warp's worth when the rows are long, or too few to fill the chip, else one (wide_spmm,
+// wide_ls): with one subgroup a row of 80 entries is a serial walk and 10,000 rows at
 // rank 3 fill 40 of 152 multiprocessors.  Rows above kHeavyRow entries
 // (heavy-tailed graphs) would still be one warp's serial walk: the SpMM's are summed
-// beforehand, kHeavySeg entries by a CTA (k_spmm_heavy); the SDDMMs' sums are scalars, so their rows are
-// cut into segments of kUpSeg entries that any row group takes.
+// beforehand, kHeavySeg entries by a CTA (k_spmm_heavy); the SDDMMs' sums are scalars, so k_ls and
+// k_inner_off cut their rows into segments of kUpSeg entries that any row group takes, and k_eval
+// takes the entries one by one.
 // In FP32, against one subgroup a row and two rows a group: alm_grad on a Kronecker graph of
 // 2^16 rows at r = 32 1.62 -> 0.17 ms; 32 inner steps of matrix completion (n = 1e4, 829,000
 // entries, rank 3) 10.4 -> 4.5 ms.
@@ -1254,12 +1255,29 @@ static __global__ void __launch_bounds__(kBlock) k_sumsq(const double *__restric
 // host launchers
 // ---------------------------------------------------------------------------------------
 
-// Subgroups per row: a warp's worth when the pattern's rows give each of them two entries on
-// average, else one: with fewer, the split's reductions and idle lanes cost more than the
-// shorter walk saves -- unless one subgroup a row leaves most of the chip idle, where half
-// an entry each is enough.
-static inline bool wide_rows(const LaunchCtx &c, int64_t entries, int64_t n, int LN) {
-    return entries >= 2 * (32 / LN) * n || (n * LN < int64_t(c.sms) * 512 && entries >= (16 / LN) * n);
+// Subgroups per row, a warp's worth or one: splitting a row costs a merge of the subgroups' sums (in
+// FP64 up to ten additions), so it pays where the walk is long (the rows' mean length as an entry sees
+// it, f_len and up_len, so that the long rows of a heavy-tailed graph count for what they hold), or
+// where one subgroup a row leaves most of the chip idle.  The lines below give close to the smallest
+// loss against the better of the two over ER graphs of 400 to 60,000 rows and degree 4 to 320, Kronecker
+// graphs, theta and matrix completion problems, r = 1 to 32 (1,244 cells; at worst 1.25 of the better).
+// k_spmm: eight entries a subgroup, or half an entry below 152 x 128 lanes of rows.  us of alm_grad, one /
+// a warp's worth: ER(60,000) of degree 24, r = 1, FP64 61 / 147, r = 13, FP32 74 / 91; of degree 36,
+// r = 32, FP32 113 / 126; Kronecker of 2^16 rows, r = 8, FP32 139 / 110, FP64 215 / 178.
+template <typename T>
+static inline bool wide_spmm(const LaunchCtx &c, const SparseView<T> &v, int LN) {
+    return v.f_len >= 8 * (32 / LN) ||
+           (int64_t(v.n) * LN < int64_t(c.sms) * 128 && 4 * v.nnz_u >= (32 / LN) * int64_t(v.n));
+}
+// k_ls (two gathers an entry, a merge of scalars only) and k_inner_off: two entries, three where the rows
+// fill the chip several times over, or a quarter of an entry below 152 x 128 lanes.  us of
+// alm_linesearch: ER(60,000) of degree 36, r = 1, FP64 156 / 214, of degree 24, r = 8, FP64 206 / 249;
+// ER(2,000) of degree 48, r = 32, FP32 63 / 56; Kronecker of 2^16 rows, r = 1, FP64 384 / 248.
+template <typename T>
+static inline bool wide_ls(const LaunchCtx &c, const SparseView<T> &v, int LN) {
+    const int64_t lanes = int64_t(v.n) * LN;
+    return v.up_len >= (lanes < int64_t(c.sms) * 1024 ? 2 : 3) * (32 / LN) ||
+           (lanes < int64_t(c.sms) * 128 && 4 * v.nnz_u >= (32 / LN) * int64_t(v.n));
 }
 #define ALM_ROW_SPLIT(wide, LN, ...)                                             \
     if (wide) { constexpr int SPW = 32 / LN; __VA_ARGS__; }                      \
@@ -1344,7 +1362,7 @@ template <typename T>
 void launch_inner_off(const LaunchCtx &c, const SparseView<T> &v, const T *R, int r, int ldr, const int *done) {
     const int L = lanes_for(r, VecT<T>::W);
     ALM_DISPATCH_LANES(L, {
-        ALM_ROW_SPLIT(wide_rows(c, v.nnz_u, v.n, LN), LN, {
+        ALM_ROW_SPLIT(wide_ls(c, v, LN), LN, {
             auto *fn = k_inner_off<T, LN, SPW>;
             const int grid = grid_for(c, fn, v.n + v.n_useg, kBlock / (LN * SPW));
             fn<<<grid, kBlock, 0, c.stream>>>(v, R, r, ldr, c.st, done);
@@ -1386,7 +1404,7 @@ static void spmm_one(const LaunchCtx &c, const SparseView<T> &v, const T *R, int
         k_spmm_heavy<T, LN><<<std::min(v.n_hseg, c.grid), kBlock, 0, c.stream>>>(v, R, r, ldr, done);
         ++*c.launches;
     }
-    ALM_ROW_SPLIT(wide_rows(c, 2 * v.nnz_u, v.n, LN), LN, {
+    ALM_ROW_SPLIT(wide_spmm(c, v, LN), LN, {
         auto *fn = k_spmm<T, LN, SPW, LRB, MODE>;
         const int grid = grid_for(c, fn, v.n, kBlock / (LN * SPW));
         fn<<<grid, kBlock, 0, c.stream>>>(v, R, r, ldr, G, D, c.res, c.st, c.partials, done);
@@ -1447,7 +1465,7 @@ void launch_dir(const LaunchCtx &c, const T *G, T *D, int64_t count, const int *
 template <typename T, int LN, bool OFF, bool LRB, int MODE>
 static void ls_one(const LaunchCtx &c, const SparseView<T> &v, const T *R, const T *D, int r, int ldr,
                    const int *done) {
-    ALM_ROW_SPLIT(wide_rows(c, v.nnz_u, v.n, LN), LN, {
+    ALM_ROW_SPLIT(wide_ls(c, v, LN), LN, {
         auto *fn = k_ls<T, LN, SPW, OFF, LRB, MODE>;
         const int grid = grid_for(c, fn, v.n + v.n_useg, kBlock / (LN * SPW));
         fn<<<grid, kBlock, 0, c.stream>>>(v, R, D, r, ldr, c.res, c.st, c.partials, done);
