@@ -76,6 +76,12 @@ __device__ __forceinline__ float2 ld2(const float *p) { return *reinterpret_cast
 __device__ __forceinline__ float2 ld2(const __nv_bfloat16 *p) {
     return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p));
 }
+// ... as loaded, for loads that are to be in flight together: a conversion behind a condition makes the
+// compiler wait for each
+__device__ __forceinline__ float2 ld2_raw(const float *p) { return *reinterpret_cast<const float2 *>(p); }
+__device__ __forceinline__ unsigned ld2_raw(const __nv_bfloat16 *p) { return *reinterpret_cast<const unsigned *>(p); }
+__device__ __forceinline__ float2 to_f2(float2 x) { return x; }
+__device__ __forceinline__ float2 to_f2(unsigned x) { return __bfloat1622float2(*reinterpret_cast<__nv_bfloat162 *>(&x)); }
 __device__ __forceinline__ void st2(float *p, float x, float y) { *reinterpret_cast<float2 *>(p) = make_float2(x, y); }
 __device__ __forceinline__ void st2(__nv_bfloat16 *p, __nv_bfloat16 x, __nv_bfloat16 y) {
     *reinterpret_cast<__nv_bfloat162 *>(p) = __halves2bfloat162(x, y);
@@ -196,7 +202,7 @@ __global__ void __launch_bounds__(256, 2) k_gnn_layer(GnnGraph g, GnnLayerArgs<T
                     const int64_t r = r0 + lr + q;
                     own[q] = r < g.rows ? ld2(p.H + r * DIN + 2 * lane) : make_float2(0.f, 0.f);
                 }
-                for (int c0 = 0; c0 < most; c0 += 32) {  // 32 entries of each row at a time
+                for (int c0 = 0; c0 < min(most, 64); c0 += 32) {  // 32 entries of each row at a time
                     int jr[4];
                     float aw[4];
 #pragma unroll
@@ -234,6 +240,49 @@ __global__ void __launch_bounds__(256, 2) k_gnn_layer(GnnGraph g, GnnLayerArgs<T
                                 }
                     }
                 }
+                // the rest of longer rows, one row at a time with sixteen of its entries in flight and the
+                // next 32 places on their way (a hub among three short rows had four)
+                if (most > 64)
+#pragma unroll 1
+                    for (int q = 0; q < 4; ++q) {
+                        const int dq = __shfl_sync(0xffffffffu, dg, q4 + q);
+                        if (dq <= 64) continue;
+                        const int eq = __shfl_sync(0xffffffffu, e0, q4 + q);
+                        const float iq = __shfl_sync(0xffffffffu, icb, q4 + q);
+                        const T *hq = p.H + __shfl_sync(0xffffffffu, base, q4 + q) * DIN + 2 * lane;
+                        float s0 = q == 0 ? a0[0] : q == 1 ? a0[1] : q == 2 ? a0[2] : a0[3];
+                        float s1 = q == 0 ? a1[0] : q == 1 ? a1[1] : q == 2 ? a1[2] : a1[3];
+                        int jn = 64 + lane < dq ? g.col[eq + 64 + lane] : 0;
+                        float an = 64 + lane < dq ? g.val[eq + 64 + lane] * iq : 0.f;
+                        for (int c0 = 64; c0 < dq; c0 += 32) {
+                            const int jr = jn, left = min(32, dq - c0);
+                            const float aw = an;
+                            const bool more = c0 + 32 + lane < dq;
+                            jn = more ? g.col[eq + c0 + 32 + lane] : 0;
+                            an = more ? g.val[eq + c0 + 32 + lane] * iq : 0.f;
+                            for (int t = 0; t < left; t += 16) {
+                                decltype(ld2_raw(hq)) raw[16];
+#pragma unroll
+                                for (int u = 0; u < 16; ++u)  // past the row: column 0, not used
+                                    raw[u] = ld2_raw(hq + int64_t(__shfl_sync(0xffffffffu, jr, t + u)) * DIN);
+#pragma unroll
+                                for (int u = 0; u < 16; ++u) {
+                                    const float a = __shfl_sync(0xffffffffu, aw, t + u);
+                                    const float2 x = to_f2(raw[u]);
+                                    if (t + u < left) {
+                                        s0 = fmaf(a, x.x, s0);
+                                        s1 = fmaf(a, x.y, s1);
+                                    }
+                                }
+                            }
+                        }
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            if (k == q) {
+                                a0[k] = s0;
+                                a1[k] = s1;
+                            }
+                    }
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     const float inv = 1.f / float(max(deg[q], 1));
@@ -259,17 +308,18 @@ __global__ void __launch_bounds__(256, 2) k_gnn_layer(GnnGraph g, GnnLayerArgs<T
                     const int e0 = g.rowptr[r], e1 = g.rowptr[r + 1];
                     const float4 o = ld4(p.H + r * DIN + c);
                     h[0] = o.x, h[1] = o.y, h[2] = o.z, h[3] = o.w;
-                    for (int e = e0; e < e1; e += 4) {
-                        float4 x[4];
-                        float a[4];
+                    constexpr int U = TR == 32 ? 8 : 4;  // in flight; 64 threads gather for a tile of 32 rows
+                    for (int e = e0; e < e1; e += U) {
+                        float4 x[U];
+                        float a[U];
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) {
+                        for (int u = 0; u < U; ++u) {
                             const int ee = min(e + u, e1 - 1);
                             a[u] = g.val[ee] * icb;
                             x[u] = ld4(p.H + (base + g.col[ee]) * DIN + c);
                         }
 #pragma unroll
-                        for (int u = 0; u < 4; ++u)
+                        for (int u = 0; u < U; ++u)
                             if (e + u < e1) {
                                 q[0] = fmaf(a[u], x[u].x, q[0]);
                                 q[1] = fmaf(a[u], x[u].y, q[1]);
@@ -437,10 +487,13 @@ __global__ void __launch_bounds__(256) k_gnn_loss(GnnGraph g, const float *__res
         const float c0 = 4.f * inv_np * eii;
         float4 d = make_float4(c0 * ri.x, c0 * ri.y, c0 * ri.z, c0 * ri.w);
         float le = eii * eii;
-        const int e1 = g.rowptr[r + 1];
-        for (int e = g.rowptr[r]; e < e1; e += 2) {
+        const int e0 = g.rowptr[r], e1 = g.rowptr[r + 1];
+        int n0 = e0 < e1 ? g.col[e0] : 0, n1 = e0 + 1 < e1 ? g.col[e0 + 1] : n0;
+        for (int e = e0; e < e1; e += 2) {
             const bool two = e + 1 < e1;
-            const int j0 = g.col[e], j1 = two ? g.col[e + 1] : j0;
+            const int j0 = n0, j1 = two ? n1 : j0;
+            n0 = e + 2 < e1 ? g.col[e + 2] : 0;  // the next round's, ahead of this one's gathers
+            n1 = e + 3 < e1 ? g.col[e + 3] : n0;
             const float4 ra = ld4(rhat + (base + j0) * kGnnRank + 4 * gl), sa = ldrs(base + j0, 4 * gl);
             const float4 rb = ld4(rhat + (base + j1) * kGnnRank + 4 * gl), sb = ldrs(base + j1, 4 * gl);
             const float ea = oct_sum(dot4(ri, ra) - dot4(si, sa), gm);
@@ -706,9 +759,9 @@ __global__ void __launch_bounds__(256) k_gnn_first_bwd(int64_t rows, const T *__
 
 // The previous layer's dZ_i = (dHp_i + sum_{j in N(i)} a_ij U_j) (.) [H_i > 0] (the pattern is
 // symmetric), one warp per row, a lane two channels; the row's columns and weights are loaded
-// by the lanes beforehand, so that four 256-byte gathers are in flight
+// by the lanes beforehand, so that eight 256-byte gathers are in flight
 template <typename T>
-__global__ void __launch_bounds__(256) k_gnn_agg_t(GnnGraph g, const float *__restrict__ U,
+__global__ void __launch_bounds__(256, 5) k_gnn_agg_t(GnnGraph g, const float *__restrict__ U,
                                                    const float *__restrict__ dHp, const T *__restrict__ H,
                                                    float *__restrict__ dZ) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -720,24 +773,27 @@ __global__ void __launch_bounds__(256) k_gnn_agg_t(GnnGraph g, const float *__re
         const int e0 = g.rowptr[r], deg = g.rowptr[r + 1] - e0;
         const float2 d = ld2(dHp + r * kGnnHid + 2 * lane), h = ld2(H + r * kGnnHid + 2 * lane);
         float s0 = 0.f, s1 = 0.f;
+        const float *Ub = U + base * kGnnHid + 2 * lane;
+        int jn = lane < deg ? g.col[e0 + lane] : 0;
+        float an = lane < deg ? g.val[e0 + lane] * icb : 0.f;
         for (int c0 = 0; c0 < deg; c0 += 32) {
-            const bool in = c0 + lane < deg;
-            const int jl = in ? g.col[e0 + c0 + lane] : 0;
-            const float al = in ? g.val[e0 + c0 + lane] * icb : 0.f;
-            const int lim = min(32, deg - c0);
-            for (int t = 0; t < lim; t += 4) {
-                float2 x[4];
-                float a[4];
+            const int jl = jn, lim = min(32, deg - c0);
+            const float al = an;
+            const bool more = c0 + 32 + lane < deg;
+            jn = more ? g.col[e0 + c0 + 32 + lane] : 0;
+            an = more ? g.val[e0 + c0 + 32 + lane] * icb : 0.f;
+            for (int t = 0; t < lim; t += 8) {
+                float2 x[8];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {  // lanes past the row hold column 0 and weight 0
+                for (int u = 0; u < 8; ++u) {
                     const int j = __shfl_sync(0xffffffffu, jl, t + u);
-                    a[u] = __shfl_sync(0xffffffffu, al, t + u);
-                    x[u] = t + u < lim ? ld2(U + (base + j) * kGnnHid + 2 * lane) : make_float2(0.f, 0.f);
+                    x[u] = t + u < lim ? ld2(Ub + int64_t(j) * kGnnHid) : make_float2(0.f, 0.f);
                 }
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    s0 = fmaf(a[u], x[u].x, s0);
-                    s1 = fmaf(a[u], x[u].y, s1);
+                for (int u = 0; u < 8; ++u) {  // lanes past the row hold weight 0
+                    const float a = __shfl_sync(0xffffffffu, al, t + u);
+                    s0 = fmaf(a, x[u].x, s0);
+                    s1 = fmaf(a, x[u].y, s1);
                 }
             }
         }
