@@ -657,8 +657,8 @@ static alm_status create_impl(alm_handle *h, const alm_problem *p, const alm_opt
         TRY(dalloc(h, reinterpret_cast<void **>(&h->g_a2), sizeof(double) * size_t(hp.m_gen)));
         std::vector<int32_t> con, cptr(1, 0);
         for (int64_t g = 0; g < hp.m_gen; ++g) {
-            const int32_t cnt = hp.g_ptr[size_t(g) + 1] - hp.g_ptr[size_t(g)];
-            con.insert(con.end(), size_t(std::max(1, (cnt + kGenChunk - 1) / kGenChunk)), int32_t(g));
+            const int64_t cnt = int64_t(hp.g_ptr[size_t(g) + 1]) - hp.g_ptr[size_t(g)];
+            con.insert(con.end(), size_t(std::max<int64_t>(1, (cnt + kGenChunk - 1) / kGenChunk)), int32_t(g));
             cptr.push_back(int32_t(con.size()));
         }
         h->n_gchunk = int(con.size());

@@ -305,29 +305,29 @@ __global__ void __launch_bounds__(256, 2) k_gnn_layer(GnnGraph g, GnnLayerArgs<T
                     const int b = g.row_inst[r];
                     const int64_t base = g.row_off[b];
                     const float icb = g.scal[b].y;
-                    const int e0 = g.rowptr[r], e1 = g.rowptr[r + 1];
+                    const int e0 = g.rowptr[r], deg = g.rowptr[r + 1] - e0;
                     const float4 o = ld4(p.H + r * DIN + c);
                     h[0] = o.x, h[1] = o.y, h[2] = o.z, h[3] = o.w;
                     constexpr int U = TR == 32 ? 8 : 4;  // in flight; 64 threads gather for a tile of 32 rows
-                    for (int e = e0; e < e1; e += U) {
+                    for (int t = 0; t < deg; t += U) {  // by offset: e0 + t may be near 2^31
                         float4 x[U];
                         float a[U];
 #pragma unroll
                         for (int u = 0; u < U; ++u) {
-                            const int ee = min(e + u, e1 - 1);
+                            const int ee = e0 + min(t + u, deg - 1);
                             a[u] = g.val[ee] * icb;
                             x[u] = ld4(p.H + (base + g.col[ee]) * DIN + c);
                         }
 #pragma unroll
                         for (int u = 0; u < U; ++u)
-                            if (e + u < e1) {
+                            if (t + u < deg) {
                                 q[0] = fmaf(a[u], x[u].x, q[0]);
                                 q[1] = fmaf(a[u], x[u].y, q[1]);
                                 q[2] = fmaf(a[u], x[u].z, q[2]);
                                 q[3] = fmaf(a[u], x[u].w, q[3]);
                             }
                     }
-                    const float inv = 1.f / float(max(e1 - e0, 1));
+                    const float inv = 1.f / float(max(deg, 1));
 #pragma unroll
                     for (int k = 0; k < 4; ++k) q[k] = tof(fromf<T>(q[k] * inv));
                     if (STORE) st4(p.AGG + r * DIN + c, q);
@@ -487,13 +487,13 @@ __global__ void __launch_bounds__(256) k_gnn_loss(GnnGraph g, const float *__res
         const float c0 = 4.f * inv_np * eii;
         float4 d = make_float4(c0 * ri.x, c0 * ri.y, c0 * ri.z, c0 * ri.w);
         float le = eii * eii;
-        const int e0 = g.rowptr[r], e1 = g.rowptr[r + 1];
-        int n0 = e0 < e1 ? g.col[e0] : 0, n1 = e0 + 1 < e1 ? g.col[e0 + 1] : n0;
-        for (int e = e0; e < e1; e += 2) {
-            const bool two = e + 1 < e1;
+        const int e0 = g.rowptr[r], deg = g.rowptr[r + 1] - e0;
+        int n0 = 0 < deg ? g.col[e0] : 0, n1 = 1 < deg ? g.col[e0 + 1] : n0;
+        for (int t = 0; t < deg; t += 2) {  // by offset: e0 + t may be near 2^31
+            const bool two = t + 1 < deg;
             const int j0 = n0, j1 = two ? n1 : j0;
-            n0 = e + 2 < e1 ? g.col[e + 2] : 0;  // the next round's, ahead of this one's gathers
-            n1 = e + 3 < e1 ? g.col[e + 3] : n0;
+            n0 = t + 2 < deg ? g.col[e0 + t + 2] : 0;  // the next round's, ahead of this one's gathers
+            n1 = t + 3 < deg ? g.col[e0 + t + 3] : n0;
             const float4 ra = ld4(rhat + (base + j0) * kGnnRank + 4 * gl), sa = ldrs(base + j0, 4 * gl);
             const float4 rb = ld4(rhat + (base + j1) * kGnnRank + 4 * gl), sb = ldrs(base + j1, 4 * gl);
             const float ea = oct_sum(dot4(ri, ra) - dot4(si, sa), gm);

@@ -474,10 +474,10 @@ __global__ void __launch_bounds__(kBlock) k_gen(SparseView<T> v, const T *__rest
     for (int c = blockIdx.x; c < v.n_gchunk; c += gridDim.x) {
         const int g = v.gc_con[c], c0 = v.g_cptr[g], nc = v.g_cptr[g + 1] - c0;
         const int e0 = v.g_ptr[g] + (c - c0) * kGenChunk;
-        const int e1 = min(e0 + kGenChunk, v.g_ptr[g + 1]);
+        const int len = min(v.g_ptr[g + 1] - e0, kGenChunk);
         double a1 = 0.0, a2 = 0.0;
-        for (int t = e0 + threadIdx.x / LANES; t < e1; t += kBlock / LANES) {
-            const int i = v.g_i[t], j = v.g_j[t];
+        for (int q = threadIdx.x / LANES; q < len; q += kBlock / LANES) {  // by offset: e0 + q may be near 2^31
+            const int t = e0 + q, i = v.g_i[t], j = v.g_j[t];
             const double ka = (i == j ? 1.0 : 2.0) * v.g_a[t];
             const V ri = mask_tail(load_row(R, i, ldr, gl, active), gl * W, r);
             const V rj = load_row(R, j, ldr, gl, active);
@@ -728,18 +728,18 @@ __global__ void __launch_bounds__(kBlock) k_spmm_heavy(SparseView<T> v, const T 
     const bool active = gl * W < r;
     for (int q = blockIdx.x; q < v.n_hseg; q += gridDim.x) {
         const int i = v.hs_row[q], e0 = v.hs_e0[q];
-        const int e1 = min(v.f_ptr[i + 1], e0 + kHeavySeg);
+        const int len = min(v.f_ptr[i + 1] - e0, kHeavySeg);
         Acc acc;
         acc.init();
-        for (int e = e0 + threadIdx.x / LANES; e < e1; e += U * NSUB) {
+        for (int t = threadIdx.x / LANES; t < len; t += U * NSUB) {  // by offset: e0 + t may be near 2^31
             int j[U];
             T c[U];
             V x[U];
 #pragma unroll
             for (int k = 0; k < U; ++k) {
-                const bool in = e + k * NSUB < e1;
-                j[k] = in ? v.f_col[e + k * NSUB] : i;
-                c[k] = in ? v.f_val[e + k * NSUB] : T(0);
+                const bool in = t + k * NSUB < len;
+                j[k] = in ? v.f_col[e0 + t + k * NSUB] : i;
+                c[k] = in ? v.f_val[e0 + t + k * NSUB] : T(0);
             }
 #pragma unroll
             for (int k = 0; k < U; ++k) x[k] = load_row(R, j[k], ldr, gl, active);
@@ -793,7 +793,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 3 : 4) k_spmm(SparseV
     const T pc_floor = T(st->pc_floor);
     for (int64_t i = g0; i < v.n; i += ng) {
         const V ri = mask_tail(load_row(R, i, ldr, gl, active), gl * W, r);
-        const int e0 = v.f_ptr[i], e1 = v.f_ptr[i + 1];
+        const int e0 = v.f_ptr[i], len = v.f_ptr[i + 1] - e0;
         const T ds = v.d_s[i], dlo = v.d_s_lo ? v.d_s_lo[i] : T(0);
         V gold = vzero(T()), dold = vzero(T());
         if (MODE == 1 && active && sub == 0) {
@@ -808,7 +808,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 3 : 4) k_spmm(SparseV
             if (LR)
                 for (int l = 0; l < v.lr_k; ++l) acc.add(T(v.lr_u[int64_t(l) * v.n + i]), zl[l]);
         }
-        if (v.n_heavy > 0 && e1 - e0 > kHeavyRow) {  // its entries are summed already
+        if (v.n_heavy > 0 && len > kHeavyRow) {  // its entries are summed already
             int a = 0, b = v.n_heavy - 1;
             while (a < b) {
                 const int mid = (a + b) / 2;
@@ -820,15 +820,15 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 3 : 4) k_spmm(SparseV
             for (int q = v.hv_ptr[a] + sub; q < q1; q += SP)
                 acc.add_stored(v.hs_sum + (int64_t(q) * LANES + gl) * (Acc::kWords * W));
         } else {
-            for (int e = e0 + sub; e < e1; e += U * SP) {
+            for (int t = sub; t < len; t += U * SP) {  // by offset: e0 + t may be near 2^31
                 int j[U];
                 T c[U];
                 V x[U];
 #pragma unroll
                 for (int k = 0; k < U; ++k) {
-                    const bool in = e + k * SP < e1;
-                    j[k] = in ? v.f_col[e + k * SP] : int(i);
-                    c[k] = in ? v.f_val[e + k * SP] : T(0);
+                    const bool in = t + k * SP < len;
+                    j[k] = in ? v.f_col[e0 + t + k * SP] : int(i);
+                    c[k] = in ? v.f_val[e0 + t + k * SP] : T(0);
                 }
 #pragma unroll
                 for (int k = 0; k < U; ++k) x[k] = load_row(R, j[k], ldr, gl, active);
