@@ -554,7 +554,7 @@ static alm_status create_impl(alm_handle *h, const alm_problem *p, const alm_opt
         TRY(upload(h, &slot, hp.up_slot));
         h->up_slot = reinterpret_cast<int2 *>(slot);
     }
-    if (h->fused_dual && h->prec == ALM_FP64) {
+    if (h->fused_dual && h->prec == ALM_FP64 && hp.ell_kf > 0 && hp.lr_k == 0) {  // k_spmm_ell reads it
         void *p = nullptr;
         TRY(dalloc(h, &p, sizeof(double2) * size_t(h->n)));
         h->pc_rec = static_cast<double2 *>(p);

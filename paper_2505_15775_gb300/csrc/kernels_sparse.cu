@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(kBlock) k_inner_slack64(SparseView<double> v, 
         const int64_t i = t0 + gl * RW + lane / LANES;
         if (i < v.n) {
             slack_row<double, LANES>(v, i, p[0], 0.0, sigma);
-            if (v.pc_rec) {
+            if (v.pc_rec && st->precond) {
                 double sdi = v.d_s[i];
                 sdi = sdi > st->pc_floor ? sdi : st->pc_floor;
                 const double a = v.d_sel_k[i] >= 0 ? v.d_sel_a[i] : 0.0;
