@@ -16,7 +16,6 @@ constexpr int kMaxRank = 32;     // rank cap (r_max)
 constexpr int kLzMax = 64;       // Lanczos basis length per cycle
 constexpr int kBlock = 256;      // threads per block of the row kernels
 constexpr int kNumSMs = 152;     // GB300
-constexpr int kLzClusterRows = 8192;  // longest vectors of the one-launch eigensolve
 constexpr int kGenChunk = 256;   // entries of a general constraint per CTA
 constexpr int kHeavyRow = 256;   // longer rows of the full pattern are summed beforehand, by CTAs
 constexpr int kHeavySeg = 512;   // ... of this many entries each

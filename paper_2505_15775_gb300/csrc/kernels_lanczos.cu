@@ -14,10 +14,10 @@
 // (k_lz_spmv alone serves the residual check of the final Ritz pair)
 // and at the end of a cycle
 //   k_lz_tridiag    smallest eigenpair (theta, s) of the m x m tridiagonal T in FP64
-//                   (Sturm-sequence bisection, then inverse iteration with a pivoted
-//                   tridiagonal solve), residual estimate |beta_{m-1} s_{m-1}|
+//                   (tridiag.cuh), residual estimate |beta_{m-1} s_{m-1}|
 //   k_lz_ritz       v = Q s, the next start vector / the result.
-// Dot products accumulate in FP64; the vectors are stored in the working precision.
+// Vectors are stored in the working precision; dot products sum in it within a warp and in FP64
+// across warps, the start vector's norm in FP64 throughout.
 //
 // Short vectors (lz_cluster_rows) take k_lz_cluster instead: the whole eigensolve, start
 // vector to residual, in one launch of one thread-block cluster.
@@ -639,9 +639,17 @@ __global__ void __launch_bounds__(kLzcThreads, 1) k_lz_cluster(SparseView<T> v, 
 // ---------------------------------------------------------------------------------------
 // host launchers
 // ---------------------------------------------------------------------------------------
-// Whether the one-launch eigensolve takes vectors of n entries at basis length k: its FP64 work
-// runs on 16 of 152 multiprocessors, so that longer vectors are faster spread over all of them,
-// and the basis has to fit the cluster's shared memory.  LZ_LINE
+// Whether the one-launch eigensolve takes vectors of v.n entries: its work runs on 16 of 152
+// multiprocessors, so that long vectors are faster spread over all of them.  alm_lambda_min, ms,
+// by launches / in one, ER graphs of degree 24 (the share of the SpMV grows with the degree: 400):
+//   FP64   4000  2.61 / 2.00 (7.27 / 3.69)   6000  2.68 / 2.66 (7.37 / 5.17)   8192  6.52 / 8.18 (7.47 / 6.78)
+//   FP32   4000  0.99 / 0.55 (2.59 / 1.04)   8192  2.78 / 1.94 (2.67 / 1.72)  12000  1.09 / 0.92 (8.01 / 6.92)
+// At 8192 and degree 100 FP64 takes 5.62 / 6.45.  In FP32 one launch stays ahead up to where the basis
+// no longer fits the cluster's shared memory (lzc_smem); its line is below that.
+template <typename T>
+static bool lz_cluster_rows(const SparseView<T> &v) {
+    return v.n <= (sizeof(T) == 4 ? 8192 : 6000) || (v.n <= 8192 && v.nnz_u >= 125 * int64_t(v.n));
+}
 template <typename T>
 static size_t lzc_smem(int n, int k, int ctas) {
     const int nv = k + 1 + kMaxLR, nr = (n + ctas - 1) / ctas, P = k | 1;
@@ -697,7 +705,7 @@ static int lzc_ctas(const LaunchCtx &c, size_t *limit) {
 template <typename T>
 bool launch_lz_cluster(const LaunchCtx &c, const SparseView<T> &v, T *Q, int kk, int max_restarts, double tol_rel,
                        double tol_abs, uint64_t seed, bool warm) {
-    if (v.n > kLzClusterRows) return false;
+    if (!lz_cluster_rows(v)) return false;
     size_t limit = 0;
     const int ctas = lzc_ctas<T>(c, &limit);
     const size_t smem = ctas ? lzc_smem<T>(v.n, kk, ctas) : 0;
