@@ -1270,13 +1270,16 @@ static inline bool wide_spmm(const LaunchCtx &c, const SparseView<T> &v, int LN)
            (int64_t(v.n) * LN < int64_t(c.sms) * 128 && 4 * v.nnz_u >= (32 / LN) * int64_t(v.n));
 }
 // k_ls (two gathers an entry, a merge of scalars only) and k_inner_off: two entries, three where the rows
-// fill the chip several times over, or a quarter of an entry below 152 x 128 lanes.  us of
+// fill the chip several times over, one with off-diagonal selectors (whose dot products are summed over
+// the row group entry by entry), or a quarter of an entry below 152 x 128 lanes.  us of
 // alm_linesearch: ER(60,000) of degree 36, r = 1, FP64 156 / 214, of degree 24, r = 8, FP64 206 / 249;
-// ER(2,000) of degree 48, r = 32, FP32 63 / 56; Kronecker of 2^16 rows, r = 1, FP64 384 / 248.
+// ER(2,000) of degree 48, r = 32, FP32 63 / 56; Kronecker of 2^16 rows, r = 1, FP64 384 / 248; theta SDP
+// n = 5000, r = 8, FP64 141 / 126, n = 20,000, r = 1, FP64 140 / 158.
 template <typename T>
 static inline bool wide_ls(const LaunchCtx &c, const SparseView<T> &v, int LN) {
     const int64_t lanes = int64_t(v.n) * LN;
-    return v.up_len >= (lanes < int64_t(c.sms) * 1024 ? 2 : 3) * (32 / LN) ||
+    const int need = v.has_off_sel ? 1 : lanes < int64_t(c.sms) * 1024 ? 2 : 3;
+    return v.up_len >= need * (32 / LN) ||
            (lanes < int64_t(c.sms) * 128 && 4 * v.nnz_u >= (32 / LN) * int64_t(v.n));
 }
 #define ALM_ROW_SPLIT(wide, LN, ...)                                             \
