@@ -16,6 +16,12 @@ constexpr int kMaxRank = 32;     // rank cap (r_max)
 constexpr int kLzMax = 64;       // Lanczos basis length per cycle
 constexpr int kBlock = 256;      // threads per block of the row kernels
 constexpr int kNumSMs = 152;     // GB300
+// Lengths at which work is cut, us a call with half of it / it / twice it (the others as they are):
+// kGenChunk: alm_eval on theta SDPs, r = 32, FP64, n = 2000 99 / 101 / 111, n = 20,000 156 / 156 / 174.
+// kHeavyRow: alm_grad, r = 32, Kronecker of 2^11 rows FP64 74 / 83 / 106, ER(4000) of degree 300 FP32
+//   100 / 97 / 82 (uniform rows of just above the line are better walked).
+// kHeavySeg: alm_grad, ER(4000) of degree 1200, r = 1 FP32 138 / 105 / 95, r = 32 FP64 377 / 358 / 433.
+// kUpSeg: alm_linesearch, Kronecker of 2^16 rows, r = 1 FP32 103 / 81 / 83, r = 32 FP64 606 / 675 / 709.
 constexpr int kGenChunk = 256;   // entries of a general constraint per CTA
 constexpr int kHeavyRow = 256;   // longer rows of the full pattern are summed beforehand, by CTAs
 constexpr int kHeavySeg = 512;   // ... of this many entries each

@@ -6,9 +6,10 @@
 //     agg_i = (sum_j a_ij h_j) / max(deg_i, 1),   h'_i = relu(Ws h_i + Wn agg_i + b),
 // a_ij = C_ij / mean|C_ij|, then the heads rhat_i = W_R h_i (32 columns) and
 // yhat_i = w_y . h_i + b_y.  Activations are stored in BF16 (or FP32) and every product
-// accumulates in FP32; gradients are FP32.  The products stay FP32 FMAs in a fixed order per
-// output: a BF16 activation is rounded from the FP32 sum, and a sum in another order (or from
-// split operands on the tensor cores) rounds some of them the other way, 2^-8 off.  A 64-wide
+// accumulates in FP32; gradients are FP32.  The products are FP32 FMAs in a fixed order per
+// output, so that a row's activations have the same bits in every tile size and batch (accuracy
+// does not ask for it: the error against 64 bits is BF16 storage's, 2.5e-3 on the warm start of
+// the torus; FP32 weights in BF16 parts on the tensor cores have not been tried).  A 64-wide
 // layer is then 8192 FMAs a row, bound by the FP32 pipe, provided that its operands come from
 // registers: tiles of rows (k_gnn_layer), each thread 8 rows x 4 outputs.
 //
@@ -126,12 +127,16 @@ __device__ __forceinline__ void lds_vec(const float *p, float (&x)[N]) {
 //   gather   64 channels: a warp loads the places of all its rows and their first 32 entries at
 //            once (a lane per row, then a lane per entry: the dependent loads are paid once a
 //            tile), then takes four rows at a time, a lane two channels of each, with the gathers
-//            of sixteen neighbour rows in flight.  8 channels: two threads a row.
+//            of sixteen neighbour rows in flight; what a row has beyond 64 entries is gathered by
+//            itself, sixteen at a time (warm start on a graph with hubs of 30,000 entries, BF16:
+//            15.0 -> 8.5 ms; Kronecker of 2^14 rows 1.54 -> 0.54 ms).  8 channels: two threads a row.
 //   product  thread (rg, og) holds TR / 16 rows x 4 outputs; inputs lie transposed in shared
 //            memory ([channel][row]), so an input costs TR / 16 x 4 FMAs per 16-byte load.
 //            Per output the FMAs run over k in order, Wn's before Ws's, from the bias on.
 // 128 rows a tile hold the FP32 pipe busy (6 shared loads per 64 FMAs); fewer rows than one
-// such tile per multiprocessor take tiles of 32, to use more of them.
+// such tile per multiprocessor take tiles of 32, to use more of them.  us of alm_gnn_warm_start,
+// tiles of 32 / 128, ER graphs of degree 10, BF16 (FP32): 8,000 rows 90 / 113 (90 / 106), 16,000
+// 119 / 118 (120 / 110), 19,456 (the line) 119 / 117 (120 / 108), 32,000 158 / 131 (153 / 129).
 // Bound: the FP32 pipe (8192 FMAs a row: 0.21 ms per million rows) and the gathers.  One warp
 // per row with both operands of every FMA from shared memory took 1.25 ms a layer on 1e6 torus
 // rows and 0.37 ms for the heads: alm_gnn_warm_start 3.60 -> 1.50 ms.

@@ -27,8 +27,7 @@
 // k_inner_off cut their rows into segments of kUpSeg entries that any row group takes, and k_eval
 // takes the entries one by one.
 // In FP32, against one subgroup a row and two rows a group: alm_grad on a Kronecker graph of
-// 2^16 rows at r = 32 1.62 -> 0.17 ms; 32 inner steps of matrix completion (n = 1e4, 829,000
-// entries, rank 3) 10.4 -> 4.5 ms.
+// 2^16 rows at r = 32 1.62 -> 0.14 ms.
 //
 // Precision.  FP64 arithmetic is scarce on GB300, so in the FP32 form every per-entry
 // product and every per-thread partial sum is FP32; partials are promoted to FP64 once
