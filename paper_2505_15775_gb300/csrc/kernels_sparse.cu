@@ -637,7 +637,8 @@ __device__ __forceinline__ void selector_slack(double h, double, double m, doubl
 // pairs (selector_slack), in one pass over the upper pattern.  k_eval and
 // k_dual_slack (still what ends an inner solve) put the values through FP64 A(X) and w, some 15
 // FP64 instructions an entry at 64 cycles a warp: together 85 us on 829,000 entries
-// at rank 3 (cold caches), this 18 us; 32 inner steps there 4.49 -> 3.00 ms with it.
+// at rank 3 (cold caches), this 21 us (18 with sigma and the products rounded to floats, which loses S
+// where its terms cancel); 32 inner steps there 4.49 -> 3.00 ms with it.
 template <typename T, int LANES, int SP>
 __global__ void __launch_bounds__(kBlock) k_inner_off(SparseView<T> v, const T *__restrict__ R, int r, int ldr,
                                                       const DevState *st, const int *done) {
